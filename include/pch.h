@@ -26,7 +26,7 @@
  *    least (a short selected list is spread over every resident warp above this floor).
  *  - PCH_TAIL_CUT [0]: once the selected list is exhausted, a warp keeps chaining only
  *    while it holds at least this many queued windows.
- *  - PCH_PROP_BLOCKS_PER_SM [384 / block threads, range 1..32]: resident propagation
+ *  - PCH_PROP_BLOCKS_PER_SM [512 / block threads, range 1..32]: resident propagation
  *    blocks per SM (the grid is this times the SM count).
  */
 #ifndef PCH_H_

@@ -69,7 +69,7 @@ int default_tail_cut() {
     return 0;
 }
 
-// Resident propagation blocks per SM: 384 threads per SM (12 warps of up to 168
+// Resident propagation blocks per SM: 512 threads per SM (16 warps of up to 128
 // registers a thread fill the register file), unless PCH_PROP_BLOCKS_PER_SM says otherwise.
 int default_prop_blocks_per_sm(int block) {
     const char* e = std::getenv("PCH_PROP_BLOCKS_PER_SM");
@@ -77,7 +77,7 @@ int default_prop_blocks_per_sm(int block) {
         int v = std::atoi(e);
         if (v > 0 && v <= 32) return v;
     }
-    return block >= 384 ? 1 : 384 / block;
+    return block >= 512 ? 1 : 512 / block;
 }
 
 // ---------------------------------------------------------------- training kernels

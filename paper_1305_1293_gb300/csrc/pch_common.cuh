@@ -69,17 +69,22 @@ struct DevMesh {
 // as coordinates (px, py) in the edge frame instead of (d0, d1)) ------------------------
 struct WinSoA {
     int* he;        // half-edge (local to the instance's mesh); -1 = empty slot
-    int* inst;      // instance
+    int* inst;      // instance | kPendA | kPendB
     double* d;      // pseudo-source distance to the source
     double* A;      // interval [A, B] along the edge from its start vertex
     double* B;
     double* px;     // pseudo-source position in the edge frame (py < 0)
     double* py;
-    double* key;    // d + dist(I, [A, B]): the window's distance back to the source
+    double* key;    // d + dist(I, [A, B]): the window's distance back to the source (pools; the
+                    // append computes it, so that propagation does not)
     int* src;       // mesh vertex at the pseudo-source (-1 for a point inside a face)
-    double* IA;     // |I A|, |I B| (kept so that propagation never recomputes them)
-    double* IB;
 };
+// Endpoint events still to be made: the window's end A (or B) may lie at the edge's start
+// (end) vertex, and no event has been made there for this pseudo-source yet.  A child whose
+// end comes from the vertex its parent was split at, or stays at a vertex its parent ended
+// at, repeats that event and is not flagged.
+constexpr unsigned kPendA = 0x80000000u, kPendB = 0x40000000u;
+constexpr int kInstMask = 0x3fffffff;
 
 // ---- instances -------------------------------------------------------------------
 struct Inst {
@@ -101,6 +106,8 @@ struct Inst {
     long long keybase;          // sort key = keybase + half-edge
     double lbar;
     double ilbar;
+    unsigned fbias;             // exponent offset of FP32 images: lbar's binade becomes [1, 2)
+    unsigned pad;
 };
 
 struct InstCtl {
@@ -115,7 +122,7 @@ struct InstCtl {
     float last_ratio;           // children / selected of the previous iteration
     float ctl_out;              // last controller output
     int active;
-    int pad;
+    float tauf;                 // tau as an FP32 image (scaled by the instance's power of two)
 };
 
 // ---- global counters of one solve -------------------------------------------------

@@ -44,7 +44,8 @@ __device__ __forceinline__ unsigned rs_key(const RsIn& in, int i) {
     if (in.keys) return in.keys[i];
     int h = in.he[i];
     if (h < 0) return ~0u;
-    return in.by_edge ? (unsigned)(in.insts[in.inst[i]].keybase + h) : (unsigned)in.inst[i];
+    const int inst = in.inst[i] & kInstMask;
+    return in.by_edge ? (unsigned)(in.insts[inst].keybase + h) : (unsigned)inst;
 }
 
 __global__ void __launch_bounds__(kRsThreads) k_rs_hist(RsIn in, const int* n_ptr, int cap, int shift, int* hist) {

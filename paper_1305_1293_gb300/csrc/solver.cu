@@ -26,6 +26,7 @@
 #include "pch_host.h"
 #include "radix.cuh"
 #include "solver.cuh"
+#include "twofloat.cuh"
 
 namespace pch {
 
@@ -68,14 +69,12 @@ __device__ __forceinline__ WarpScan warp_scan(int x) {
 }
 
 // Warp-aggregated reservation of `x` slots per lane on counter `c`; returns the lane's
-// base.  With `fill`, a warp that reserved anything gets the counter's value after its
-// reservation there (unchanged otherwise).
-__device__ __forceinline__ int warp_reserve(int* c, int x, int* fill = nullptr) {
+// base.
+__device__ __forceinline__ int warp_reserve(int* c, int x) {
     WarpScan s = warp_scan(x);
     int base = 0;
     if ((threadIdx.x & 31) == 31 && s.total) base = atomicAdd(c, s.total);
     base = __shfl_sync(0xffffffffu, base, 31);
-    if (fill && s.total) *fill = base + s.total;
     return base + s.excl;
 }
 
@@ -224,15 +223,20 @@ __device__ __forceinline__ void pool_stat(const Work& w, const PoolStats& ps, in
     }
 }
 
-__device__ __forceinline__ void load_win(const WinSoA& s, int i, int& he, int& inst, double& d, double& A, double& B,
-                                         double& px, double& py, double& key, int& src, double& IA, double& IB) {
-    he = s.he[i]; inst = s.inst[i]; d = s.d[i]; A = s.A[i]; B = s.B[i]; px = s.px[i]; py = s.py[i]; key = s.key[i];
-    src = s.src[i]; IA = s.IA[i]; IB = s.IB[i];
+// A pool window.  `inst` is the instance without the pending-event bits, `pend` those bits.
+struct Win {
+    int he, inst, src;
+    unsigned pend;
+    double d, A, B, px, py, key;
+};
+__device__ __forceinline__ Win load_win(const WinSoA& s, int i) {
+    const int fi = s.inst[i];
+    return {s.he[i], fi & kInstMask, s.src[i], (unsigned)fi & ~(unsigned)kInstMask, s.d[i], s.A[i], s.B[i], s.px[i],
+            s.py[i], 0.0};
 }
-__device__ __forceinline__ void store_win(const WinSoA& s, int i, int he, int inst, double d, double A, double B,
-                                          double px, double py, double key, int src, double IA, double IB) {
-    s.he[i] = he; s.inst[i] = inst; s.d[i] = d; s.A[i] = A; s.B[i] = B; s.px[i] = px; s.py[i] = py; s.key[i] = key;
-    s.src[i] = src; s.IA[i] = IA; s.IB[i] = IB;
+__device__ __forceinline__ void store_win(const WinSoA& s, int i, const Win& W) {
+    s.he[i] = W.he; s.inst[i] = W.inst | (int)W.pend; s.src[i] = W.src;
+    s.d[i] = W.d; s.A[i] = W.A; s.B[i] = W.B; s.px[i] = W.px; s.py[i] = W.py;
 }
 
 // A window whose pseudo-source vertex has since been reached by a shorter path is
@@ -290,10 +294,9 @@ __global__ void k_init_face_sources(Work w, const SrcDev* __restrict__ srcs, int
             if (R.twin < 0) continue;
             // window on twin(h) = (v1 -> v0): point at (L - x, -y), interval [0, L]
             double px = R.L - x, py = -y;
-            const double IA = sqrt(px * px + py * py), IB = sqrt((px - R.L) * (px - R.L) + py * py);
-            double key = px < 0 ? IA : (px > R.L ? IB : -py);
             int slot = atomicAdd(&cnt->n_child, 1);
-            if (slot < w.arena_cap) store_win(w.arena, slot, R.twin, s.inst, 0.0, 0.0, R.L, px, py, key, -1 - s.label, IA, IB);
+            if (slot < w.arena_cap)
+                store_win(w.arena, slot, {R.twin, s.inst, -1 - s.label, kPendA | kPendB, 0.0, 0.0, R.L, px, py, 0.0});
         }
     }
 }
@@ -359,6 +362,7 @@ __global__ void k_tau(Work w, int control, const float* __restrict__ mlp) {
             // the strided selection decides by per-thread thresholds instead; tau = -inf
             // also turns chaining off (the paper propagates each selected window one hop)
             c.tau = control == PCH_CONTROL_STRIDED ? -INFINITY : tau;
+            c.tauf = f_of(c.tau, w.inst[inst].fbias);
             c.n_pending = np;
             c.n_next = 0;
             if (c.kmin != ~0ull) c.ref = bitsd(c.kmin);   // min key of the current pool
@@ -423,27 +427,30 @@ __global__ void __launch_bounds__(256) k_compact(Work w) {
     for (int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
         int i = base + threadIdx.x;
         bool valid = i < n;
-        int he = 0, inst = 0, src = -1;
-        double d = 0, A = 0, B = 0, px = 0, py = 0, key = 0, IA = 0, IB = 0;
+        Win W{0, 0, -1, 0u, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         if (valid) {
-            load_win(cur, i, he, inst, d, A, B, px, py, key, src, IA, IB);
-            if (stale_source(w.inst[inst], src, d)) valid = false;   // dropped from the pool
+            W = load_win(cur, i);
+            W.key = cur.key[i];
+            if (stale_source(w.inst[W.inst], W.src, W.d)) valid = false;   // dropped from the pool
         }
         bool sel;
         if (w.stride_T > 0) {           // strided selection: the owning thread's threshold
             const int t = i % w.stride_T;
-            const unsigned long long kb = dbits(key), tk = w.sthr_key[t];
+            const unsigned long long kb = dbits(W.key), tk = w.sthr_key[t];
             sel = valid && (kb < tk || (kb == tk && i <= w.sthr_idx[t]));
         } else {
-            sel = valid && key <= w.ctl[inst].tau;
+            sel = valid && W.key <= w.ctl[W.inst].tau;
         }
         int slot = warp_reserve(&cnt->n_sel, sel ? 1 : 0);
         if (sel && slot >= w.sel_cap) sel = false;   // work list full: stays pending
-        if (sel) store_win(w.sel, slot, he, inst, d, A, B, px, py, key, src, IA, IB);
+        if (sel) store_win(w.sel, slot, W);
         bool rest = valid && !sel;
         int rslot = warp_reserve(&cnt->n_rest, rest ? 1 : 0);
-        if (rest) store_win(nxt, rslot, he, inst, d, A, B, px, py, key, src, IA, IB);
-        pool_stat(w, ps, inst, key, rest);
+        if (rest) {
+            store_win(nxt, rslot, W);
+            nxt.key[rslot] = W.key;
+        }
+        pool_stat(w, ps, W.inst, W.key, rest);
     }
     if (ps.sh_hist) {
         __syncthreads();
@@ -453,253 +460,248 @@ __global__ void __launch_bounds__(256) k_compact(Work w) {
 }
 
 // ====================================================================== Step 2: propagation
+// A window on its way through the propagation kernel: the pool's fields and the offsets
+// of its ends from the pseudo-source's foot, ax = A - px and bx = B - px, which the
+// child's filter needs before they are needed again here.
+struct LaneWin {
+    int h, inst, src, hop;
+    bool task;              // a deferred left child: the window's own part is done
+    unsigned pend;          // kPendA | kPendB
+    double d, A, B, px, py, ax, bx;
+};
+constexpr int kHopTask = 1 << 30;     // hop-field flags of a queue entry: a deferred left child,
+constexpr int kHopPend = 28;          // bits 28, 29: kPendB, kPendA
+constexpr int kHopMask = (1 << kHopPend) - 1;
+
 struct ChildOut {
     int he;
-    double A, B, px, py, key;
-    double IA, IB;          // |I A|, |I B| (reused when the child is propagated at once)
+    unsigned pend;
+    float key;              // FP32 image of the window's key (decides only whether it is chained)
+    double A, B, px, py, ax, bx;
 };
 
-// The ray from I along D = P - I (P a window endpoint on the parent edge, D = (dx, -py)
-// in the parent frame) meets the child's line O + s u where
-//   s = cross(I - O, D) / cross(u, D),   I + t D with t = cross(I - O, u) / cross(u, D),
-// and cross(I - O, u) = -Ipy.  Inputs: upy = ux py, rpy = rx py, (rx, ry) = I - O.
-// Returns s and |I X| = t |D|.  A hit within 2^-40 Lc beyond an end (rounding, for a
-// parent window that ends on a vertex) is clamped to that end with |I X| kept; a hit
-// further outside [0, Lc] (or a ray that does not cross) is clamped to the nearer end
-// with |I X| recomputed there.
-__device__ __forceinline__ void ray_hit(double dx, double ID, double ux, double uy, double ry, double upy, double rpy,
-                                        double py, double Ipx, double Ipy, double Lc, double& xh, double& IX) {
-    const double den = -fma(uy, dx, upy);   // cross(u, D)
-    const double r = rcp_nr(den);           // full precision: |I X| compounds along a lineage
-    xh = -fma(ry, dx, rpy) * r;             // cross(I - O, D) / cross(u, D)
-    IX = (-Ipy * r) * ID;
-    if (!gt0_s(den) || !(ge0_s(xh) && le_s(xh, Lc))) {
-        const long long xb = sbits(xh);
-        if (gt0_s(den) && xb < 0 && (xb & 0x7fffffffffffffffll) <= sbits(times_eps(Lc))) {
-            xh = 0.0;
-            return;
-        }
-        if (gt0_s(den) && xb > sbits(Lc) && xb - sbits(Lc) <= kSnapUlps) {
-            xh = Lc;
-            return;
-        }
-        xh = gt0_s(den) ? (lt_s(xh, 0.0) ? 0.0 : (lt_s(Lc, xh) ? Lc : xh))
-                        : (gt0_s(fma(ux, dx, -uy * py)) ? Lc : 0.0);   // dot(u, D) > 0: towards Lc
+// Where the ray from I through a parent end P = (x, 0) meets the child's edge, measured
+// from its start.  With D = P - I = (dx, -py), u the child edge's axis and V the vertex it
+// shares with the parent edge (at `base` along the child's edge, at x - m along the
+// parent's): base + cross(P - V, D) / cross(u, D) = base + m py / (ux py + uy dx).
+// A hit outside [0, Lc], or a ray that does not cross, is clamped to the nearer end.
+__device__ __forceinline__ double ray_hit(double m, double dx, double ux, double uy, double upy, double py, double base,
+                                          double Lc) {
+    const double dn = fma(uy, dx, upy);     // -cross(u, D): negative when the ray crosses
+    double xh = fma(m * py, rcp_nr(dn), base);
+    if (!(sbits(dn) < 0 && ge0_s(xh) && le_s(xh, Lc))) {
+        xh = sbits(dn) < 0 ? (lt_s(xh, 0.0) ? 0.0 : (lt_s(Lc, xh) ? Lc : xh))
+                           : (gt0_s(fma(ux, dx, -uy * py)) ? Lc : 0.0);   // dot(u, D) > 0: towards Lc
         if (!(xh == xh)) xh = 0.0;
-        const double ex = xh - Ipx;
-        IX = sqrt_nr(fma(ex, ex, Ipy * Ipy));
     }
+    return xh;
 }
 
-__device__ __forceinline__ double child_key(double d, double a, double b, double Ipx, double Ipy, double IA,
-                                            double IB) {
-    return d + (lt_s(Ipx, a) ? IA : (lt_s(b, Ipx) ? IB : -Ipy));
-}
+// FP32 margins of the filters below.  A window is dropped only when it is longer by more
+// than the relative margin 1e-12 (kDomRel) after the two-float rounding (below 2^-43 of
+// the sum) is taken off, and by more than 2^-20 of the lengths around the edge, which
+// enter the tests as plain floats (their rounding is below 2^-22).
+constexpr float kDomF = 1.3e-12f;
+constexpr float kLocalF = 0x1p-20f;
 
-// dominated(lhs, rhs) with rhs = g + sqrt(q): compares squares, no square root.
-constexpr double kInvDom = 1.0 / (1.0 + kDomRel);
-__device__ __forceinline__ bool dominated_sq(double lhs, double g, double q) {
-    const double t = lhs * kInvDom - g;
-    return gt0_s(t) && gt0_s(fma(t, t, -q));
-}
-
-// The round's write side of the propagation kernel's shared-memory queue: the second
-// child of a window whose rays reach v2 is deferred there as a task, so that each lane
-// computes one child per round.
-struct TaskQueue {
-    double *d, *A, *B, *px, *py, *IA, *IB;
-    int *he, *inst, *src, *hop;
-    int* count;   // entries reserved this round
-    int cap;      // entries the next round can take
-};
-constexpr int kHopTask = 1 << 30;   // hop-field flag of a queue entry: a deferred left child
-
-// Algorithm 2 for one window: events, one angle one split, children with the Xin-Wang
-// filter.  Returns whether the window passed the filter; children in c0, c1 (nch).  When
-// both children exist the left one is deferred to q as a task (if q has room).  A task
-// (task = true) skips the window's own part, done in an earlier round, and computes the
-// left child only; IB_in then holds |I v2|.
+// Algorithm 2 for one window: events, one angle one split, the child with the Xin-Wang
+// filter.  A window with two children computes the right one and asks for the left one
+// to be deferred (`defer`): each lane computes one child a round.  Returns whether the
+// window passed the filter; has_child says whether `c` holds a child.
+//
+// What bounds this kernel is the FP64 unit (16 SM cycles a warp instruction).  The
+// positions (pseudo-source and interval in the child's frame) are FP64, 21 instructions
+// for a window that does not reach v2: ray_hit measures from the vertex that the two edges
+// share, which needs no cross product of far points.  What is only decided (occupancy,
+// the filters, the chaining) runs in FP32 with error bounds (twofloat.cuh); the lengths
+// |I A|, |I B| that the filters compare are two-float values made from the coordinates
+// when they are needed, so no rounding of theirs accumulates along a lineage.  Before,
+// all of it was FP64, 62 instructions a window: eight fields on the 327,680-face sphere
+// took 86.1 ms and take 40.6, the 1M-face torus 49.3 and 23.5.
 template <bool PROV>
-__device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, FanReq* req, int inst,
-                                                 int src, double d, int h, double A, double B, double px, double py,
-                                                 bool task, int hop, const TaskQueue& q, ChildOut& c0, ChildOut& c1,
-                                                 int& nch, int& occ_out, int& ncomp, int& nray, double IA_in,
-                                                 double IB_in) {
-    bool prop = false;
-    nch = 0;
-    occ_out = 0;
-    ncomp = 0;
-    nray = 0;
-    {
-        const Inst& I = w.inst[inst];
-        const HERec R = I.rec[h];
-        const double L = R.L;
-        double g0 = ldg_dist(I.g, R.v0 & ~kPseudoBit);
-        double g1 = ldg_dist(I.g, R.v1 & ~kPseudoBit);
-        double g2 = ldg_dist(I.g, R.v2 & ~kPseudoBit);
-        const double ax = A - px, bx = B - px;
-        // |IA|, |IB|: carried over from the parent when the window was chained
-        const double IA = ge0_s(IA_in) ? IA_in : sqrt_nr(fma(ax, ax, py * py));
-        const double IB = ge0_s(IB_in) ? IB_in : sqrt_nr(fma(bx, bx, py * py));
-        const double xc = R.xc, yc = R.yc;
-        bool left = false, right = false, occ = false;
-        double Iv2 = IB;
-        if (task) {
-            occ = true;
-            left = R.tw2 >= 0;
-        } else if ((hop > 0 || !(dominated(d + IB, g0 + B) || dominated(d + IA, g1 + (L - A)))) &&
-                   !stale_source(I, src, d)) {
-            // Xin-Wang endpoint tests against the current distances passed: the window is
-            // useless if the path via v0 beats it at B, or the path via v1 at A.  A chained
-            // window (hop > 0) passed the same two tests when its parent created it a round
-            // ago; distances only fall, so repeating them could only prune more, never keep
-            // a window that must go, and they are skipped.
-            prop = true;
-            const EvSrc es{inst, h, src, 0, px, py};   // event origin, recorded with PROV only
-            const double py2 = py * py;
-            const double tol = times_eps(L);
-            const double tiny = tol;
-            // Algorithm 2: endpoint events at v0 (A = v0) and v1 (B = v1)
-            if (le_s(A, tol)) {
-                double D0 = d + (sbits(A) == 0 ? IA : sqrt_nr(fma(px, px, py2)));
-                if (const int ev = vertex_event<PROV>(I, R.v0, D0, g0, &w, &es))   // the ray arrives at v0 from I (h's frame)
-                    push_fan(req, &cnt->n_req, w.req_cap, &cnt->error, inst, R.v0 & ~kPseudoBit, D0, h, px, py, ev);
-            }
-            if (sbits(L) - sbits(B) <= kSnapUlps) {
-                double q = L - px;
-                double D1 = d + (sbits(B) == sbits(L) ? IB : sqrt_nr(fma(q, q, py2)));
-                if (const int ev = vertex_event<PROV>(I, R.v1, D1, g1, &w, &es))   // at v1, in the frame of twin(h) = (v1 -> v0)
-                    push_fan(req, &cnt->n_req, w.req_cap, &cnt->error, inst, R.v1 & ~kPseudoBit, D1, R.twin, q, -py, ev);
-            }
-            // occupancy of v2: the ray I -> v2 crosses e at xs = px + num / den;
-            // decided without the division (den > 0), by the signs of fused residuals
-            const double den = yc - py, num = (xc - px) * (-py);
-            const bool before_A = gt0_s(fma(ax - tol, den, -num));
-            occ = !before_A && ge0_s(fma(bx + tol, den, -num));
-            occ_out = occ;
-            if (occ) {
-                const double xs = px + num * rcp_nr(den);
-                const double xcl = lt_s(xs, A) ? A : (lt_s(B, xs) ? B : xs);
-                // angle_split position: xs in units of 2^-24 |e| (only the order of positions
-                // on one edge matters, so any fixed scale per edge will do)
-                const double xq = xs * (rcp_nr(L) * (double)(1 << kAngleXBits));
-                const double dx = xc - px, dy = yc - py;
-                Iv2 = sqrt_nr(dx * dx + dy * dy);
-                const double D2 = d + Iv2;
-                // one angle one split (Fig. `fig:filter`(a)) against angle_split[h]
-                unsigned long long* ap = I.ang + h;
-                const unsigned long long aw = __ldcg(ap);
-                bool win = aw == kEmptyAngle || dbits(D2) < (aw & ~kAngleXMask);
-                if (win) {
-                    left = right = true;
-                    atomicMin(ap, pack_angle(D2, xq));
-                } else {
-                    // loser: keep the child on its own side of the winner's ray, which
-                    // crosses e in [q, q + 1] (angle_split units), widened by the snap
-                    // tolerance
-                    // (positions compared after the same clamping the stored one had)
-                    const long long q = (long long)(aw & kAngleXMask);
-                    left = angle_pos(xq + kSplitTol) < q;
-                    right = angle_pos(xq - kSplitTol) > q;
-                    if (!left && !right) left = right = true;
-                }
-                if (const int ev = vertex_event<PROV>(I, R.v2, D2, g2, &w, &es)) {
-                    // the ray arrives at v2 inside face(h); direction to I in the frame of
-                    // prev(h) = (v2 -> v0), whose axis is (-xc, -yc) / L2
-                    const int hp = 3 * (h / 3) + (h % 3 + 2) % 3;
-                    const double ux = -R.u2x, uy = -R.u2y, ex = px - xc, ey = py - yc;
-                    push_fan(req, &cnt->n_req, w.req_cap, &cnt->error, inst, R.v2 & ~kPseudoBit, D2, hp,
-                             ex * ux + ey * uy, ux * ey - uy * ex, ev);
-                }
-                if (le_s(B - xcl, tiny)) right = false;
-                if (le_s(xcl - A, tiny)) left = false;
-            } else {
-                right = before_A;
-                left = !right;
-            }
-            right = right && R.tw1 >= 0;
-            left = left && R.tw2 >= 0;
-        }
-        {
-            // Children, one code path in child order (right first): the right child
-            // lies on edge v2 -> v1 (frame origin v2), the left on v0 -> v2 (origin v0).
-            // When v2 is occupied the child's endpoint at v2 is exact.
-#pragma unroll 1
-            for (int j = 0; j < 2; ++j) {
-                if (!(j == 0 ? (right || left) : (right && left))) break;
-                if (j == 1) {   // defer the left child: one child per lane and round
-                    const int ts = atomicAdd(q.count, 1);
-                    if (ts < q.cap) {
-                        q.he[ts] = h; q.inst[ts] = inst; q.src[ts] = src; q.hop[ts] = hop | kHopTask;
-                        q.d[ts] = d; q.A[ts] = A; q.B[ts] = B; q.px[ts] = px; q.py[ts] = py;
-                        q.IA[ts] = IA; q.IB[ts] = Iv2;
-                        break;
-                    }
-                }
-                const bool rt = j == 0 && right;
-                ++ncomp;
-                nray += occ ? 1 : 2;
-                {   // the child's record, needed when it is propagated (next round when chained)
-                    const char* cr = reinterpret_cast<const char*>(I.rec + (rt ? R.tw1 : R.tw2));
-                    asm volatile("prefetch.global.L1 [%0];" ::"l"(cr));
-                    asm volatile("prefetch.global.L1 [%0];" ::"l"(cr + sizeof(HERec) - 8));
-                }
-                // both sides as one select-driven path (a warp holds left and right children)
-                const double Lc = rt ? R.L1 : R.L2;
-                const double ox = rt ? xc : 0.0, oy = rt ? yc : 0.0;
-                const double ux = rt ? R.u1x : R.u2x;
-                const double uy = rt ? R.u1y : R.u2y;
-                const double rx = px - ox, ry = py - oy;
-                const double Ipx = fma(rx, ux, ry * uy), Ipy = fma(ux, ry, -(uy * rx));
-                const double upy = ux * py, rpy = rx * py;
-                // rays through A and B; at v2 (occupied) the right child starts at 0,
-                // the left child ends at Lc
-                double a, IAc, b, IBc;
-                if (occ && rt) {
-                    a = 0.0;
-                    IAc = Iv2;
-                } else {
-                    ray_hit(ax, IA, ux, uy, ry, upy, rpy, py, Ipx, Ipy, Lc, a, IAc);
-                }
-                if (occ && !rt) {
-                    b = Lc;
-                    IBc = Iv2;
-                } else {
-                    ray_hit(bx, IB, ux, uy, ry, upy, rpy, py, Ipx, Ipy, Lc, b, IBc);
-                }
-                if (!lt_s(times_eps(Lc), b - a)) continue;
-                // Xin-Wang filter (Fig. `fig:filter`(b)) on the new window: against its
-                // start and end vertices (right child: v2, v1; left child: v0, v2), and
-                // against the vertex T of the parent edge off the child's edge (right: v0;
-                // left: v1), at both ends of the child.  d + |I x| - |T x| is smallest at
-                // the end nearer the vertex shared with the parent edge (the end the paper
-                // tests); requiring both ends is the same decision in exact arithmetic and
-                // keeps the child when rounding puts one end's test on the wrong side of
-                // the margin.
-                const double gS = rt ? g2 : g0, gE = rt ? g1 : g2, gT = rt ? g0 : g1;
-                const double dA = d + IAc, dB = d + IBc;
-                const double Tx = rt ? xc : -L;           // the child's origin relative to T
-                const double Xax = fma(a, ux, Tx), Xay = fma(a, uy, oy);
-                const double Xbx = fma(b, ux, Tx), Xby = fma(b, uy, oy);
-                const bool useless = dominated(dB, gS + b) || dominated(dA, gE + (Lc - a)) ||
-                                     (dominated_sq(dA, gT, fma(Xax, Xax, Xay * Xay)) &&
-                                      dominated_sq(dB, gT, fma(Xbx, Xbx, Xby * Xby)));
-                if (useless) continue;
-                const ChildOut co{rt ? R.tw1 : R.tw2, a, b, Ipx, Ipy, child_key(d, a, b, Ipx, Ipy, IAc, IBc), IAc, IBc};
-                if (nch == 0) c0 = co;
-                else c1 = co;
-                ++nch;
-            }
+__device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, FanReq* req, const LaneWin& W,
+                                                 ChildOut& c, bool& has_child, bool& defer, bool& occ, bool& comp) {
+    has_child = defer = occ = comp = false;
+    const Inst& I = w.inst[W.inst];
+    const HERec R = I.rec[W.h];
+    const unsigned fb = I.fbias;
+    const double px = W.px, py = W.py, A = W.A, B = W.B, ax = W.ax, bx = W.bx, d = W.d, L = R.L;
+    double g0 = ldg_dist(I.g, R.v0 & ~kPseudoBit);
+    double g1 = ldg_dist(I.g, R.v1 & ~kPseudoBit);
+    double g2 = ldg_dist(I.g, R.v2 & ~kPseudoBit);
+    const F2 df = f2_mag(d, fb);
+    const float Lf = f_of(L, fb), xcf = f_of(R.xc, fb), ycf = f_of(R.yc, fb);
+    bool left = false, right = false, prop = false;
+    const double tol = times_eps(L);
+    if (W.task) {
+        occ = true;
+        left = R.tw2 >= 0;
+    } else if (!stale_source(I, W.src, d)) {
+        prop = true;
+        if (W.hop == 0) {
+            // Xin-Wang endpoint tests of a window from the pool against the current
+            // distances: useless if the path via v0 beats it at B, or the path via v1 at A.
+            // A chained window passed them a round ago, when its parent created it.
+            const F2 yy = f2_sq(f2_mag(py, fb));
+            const F2 lenA = f2_hyp(f2_mag(ax, fb), yy), lenB = f2_hyp(f2_mag(bx, fb), yy);
+            const float mrg = fmaf(df.h + fmaxf(lenA.h, lenB.h), kDomF, Lf * kLocalF);
+            const float t0 = f2_add_f(f2_sub(df, f2_mag(g0, fb)), lenB);
+            const float t1 = f2_add_f(f2_sub(df, f2_mag(g1, fb)), lenA);
+            prop = !(t0 > f_of(B, fb) + mrg || t1 > (Lf - f_of(A, fb)) + mrg);
         }
     }
+    if (prop) {
+        const EvSrc es{W.inst, W.h, W.src, 0, px, py};   // event origin, recorded with PROV only
+        // Algorithm 2: endpoint events at v0 (A = v0) and v1 (B = v1)
+        if (W.pend) {
+            const double py2 = py * py;
+            if ((W.pend & kPendA) && le_s(A, tol)) {
+                const double D0 = d + sqrt_nr(fma(px, px, py2));
+                if (const int ev = vertex_event<PROV>(I, R.v0, D0, g0, &w, &es))   // the ray arrives at v0 from I (h's frame)
+                    push_fan(req, &cnt->n_req, w.req_cap, &cnt->error, W.inst, R.v0 & ~kPseudoBit, D0, W.h, px, py, ev);
+            }
+            if ((W.pend & kPendB) && sbits(L) - sbits(B) <= kSnapUlps) {
+                const double q = L - px;
+                const double D1 = d + sqrt_nr(fma(q, q, py2));
+                if (const int ev = vertex_event<PROV>(I, R.v1, D1, g1, &w, &es))   // at v1, in the frame of twin(h) = (v1 -> v0)
+                    push_fan(req, &cnt->n_req, w.req_cap, &cnt->error, W.inst, R.v1 & ~kPseudoBit, D1, R.twin, q, -py, ev);
+            }
+        }
+        // occupancy of v2: the ray I -> v2 crosses e at xs; xs < A exactly when
+        // cross(A - I, v2 - A) = ax yc + py (xc - A) > 0, and the same at B.  FP32 decides
+        // unless a value is within its rounding of 0; then FP64, with the tolerance 2^-40 L.
+        const float axf = f_of(ax, fb), bxf = f_of(bx, fb), pyf = f_of(py, fb);
+        const float vA = fmaf(axf, ycf, pyf * (xcf - f_of(A, fb)));
+        const float vB = fmaf(bxf, ycf, pyf * (xcf - f_of(B, fb)));
+        const float ext = fmaf(fabsf(pyf), fabsf(xcf) + Lf, Lf * ycf * 0x1p-10f);
+        const float eA = fmaf(fabsf(axf), ycf, ext) * 0x1p-20f, eB = fmaf(fabsf(bxf), ycf, ext) * 0x1p-20f;
+        bool before_A;
+        if (vA > eA) {
+            before_A = true;
+        } else if (vB < -eB) {
+            before_A = false;
+        } else if (vA < -eA && vB > eB) {
+            before_A = false;
+            occ = true;
+        } else {
+            const double den = R.yc - py, num = (R.xc - px) * (-py);
+            before_A = gt0_s(fma(ax - tol, den, -num));
+            occ = !before_A && ge0_s(fma(bx + tol, den, -num));
+        }
+        if (occ) {
+            const double dx = R.xc - px, dy = R.yc - py;
+            const double xs = fma(dx * (-py), rcp_nr(dy), px);
+            const double xcl = lt_s(xs, A) ? A : (lt_s(B, xs) ? B : xs);
+            // angle_split position: xs in units of 2^-24 |e| (only the order of positions
+            // on one edge matters, so any fixed scale per edge will do)
+            const double xq = xs * (rcp_nr(L) * (double)(1 << kAngleXBits));
+            const double D2 = d + sqrt_nr(dx * dx + dy * dy);
+            // one angle one split (Fig. `fig:filter`(a)) against angle_split[h]
+            unsigned long long* ap = I.ang + W.h;
+            const unsigned long long aw = __ldcg(ap);
+            const bool win = aw == kEmptyAngle || dbits(D2) < (aw & ~kAngleXMask);
+            if (win) {
+                left = right = true;
+                atomicMin(ap, pack_angle(D2, xq));
+            } else {
+                // loser: keep the child on its own side of the winner's ray, which
+                // crosses e in [q, q + 1] (angle_split units), widened by the snap
+                // tolerance
+                // (positions compared after the same clamping the stored one had)
+                const long long q = (long long)(aw & kAngleXMask);
+                left = angle_pos(xq + kSplitTol) < q;
+                right = angle_pos(xq - kSplitTol) > q;
+                if (!left && !right) left = right = true;
+            }
+            if (const int ev = vertex_event<PROV>(I, R.v2, D2, g2, &w, &es)) {
+                // the ray arrives at v2 inside face(h); direction to I in the frame of
+                // prev(h) = (v2 -> v0), whose axis is (-xc, -yc) / L2
+                const int hp = 3 * (W.h / 3) + (W.h % 3 + 2) % 3;
+                const double ux = -R.u2x, uy = -R.u2y, ex = px - R.xc, ey = py - R.yc;
+                push_fan(req, &cnt->n_req, w.req_cap, &cnt->error, W.inst, R.v2 & ~kPseudoBit, D2, hp,
+                         ex * ux + ey * uy, ux * ey - uy * ex, ev);
+            }
+            if (le_s(B - xcl, tol)) right = false;
+            if (le_s(xcl - A, tol)) left = false;
+        } else {
+            right = before_A;
+            left = !right;
+        }
+        right = right && R.tw1 >= 0;
+        left = left && R.tw2 >= 0;
+    }
+    if (!(right || left)) return prop;
+    // The child, one select-driven path for both sides (a warp holds left and right
+    // children): the right child lies on edge v2 -> v1 (frame origin v2), the left one on
+    // v0 -> v2 (origin v0).  When v2 is occupied the child's end at v2 is exact.
+    const bool rt = right;
+    defer = right && left;
+    comp = true;
+    const int che = rt ? R.tw1 : R.tw2;
+    {   // the child's record, needed when it is propagated (next round when chained)
+        const char* cr = reinterpret_cast<const char*>(I.rec + che);
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(cr));
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(cr + sizeof(HERec) - 8));
+    }
+    const double Lc = rt ? R.L1 : R.L2;
+    const double ux = rt ? R.u1x : R.u2x, uy = rt ? R.u1y : R.u2y;
+    const double shared = rt ? L : 0.0;       // the vertex of both edges, on the parent's
+    const double base = rt ? Lc : 0.0;        // and on the child's
+    const double rx = px - shared, upy = ux * py;
+    const double Ipx = fma(rx, ux, fma(py, uy, base)), Ipy = fma(-uy, rx, upy);
+    double a, b;
+    if (occ && rt) a = 0.0;
+    else a = ray_hit(A - shared, ax, ux, uy, upy, py, base, Lc);
+    if (occ && !rt) b = Lc;
+    else b = ray_hit(B - shared, bx, ux, uy, upy, py, base, Lc);
+    const float Lcf = f_of(Lc, fb), af = f_of(a, fb), bf = f_of(b, fb);
+    // narrower than 2^-40 of the edge: dropped
+    if (!(bf - af > Lcf * kLocalF) && !lt_s(times_eps(Lc), b - a)) return prop;
+    const double axc = a - Ipx, bxc = b - Ipx;
+    // Xin-Wang filter (Fig. `fig:filter`(b)) on the new window: against its start and end
+    // vertices (right child: v2, v1; left child: v0, v2), and against the vertex T of the
+    // parent edge off the child's edge (right: v0; left: v1), at both ends of the child.
+    // d + |I x| - |T x| is smallest at the end nearer the vertex shared with the parent
+    // edge (the end the paper tests); requiring both ends is the same decision in exact
+    // arithmetic and keeps the child when rounding puts one end's test on the wrong side
+    // of the margin.
+    {
+        const F2 yy = f2_sq(f2_mag(Ipy, fb));
+        const F2 lenA = f2_hyp(f2_mag(axc, fb), yy), lenB = f2_hyp(f2_mag(bxc, fb), yy);
+        const float loc = (Lf + Lcf + fabsf(xcf) + ycf) * kLocalF;
+        const float mrg = fmaf(df.h + fmaxf(lenA.h, lenB.h), kDomF, loc);
+        const F2 eS = f2_sub(df, f2_mag(rt ? g2 : g0, fb)), eE = f2_sub(df, f2_mag(rt ? g1 : g2, fb));
+        const F2 eT = f2_sub(df, f2_mag(rt ? g0 : g1, fb));
+        const float uxf = (float)f_of(ux, 896u << 20), uyf = f_of(uy, 896u << 20);
+        const float Tx = rt ? xcf : -Lf, Ty = rt ? ycf : 0.f;     // the child's origin relative to T
+        const float Xax = fmaf(af, uxf, Tx), Xay = fmaf(af, uyf, Ty);
+        const float Xbx = fmaf(bf, uxf, Tx), Xby = fmaf(bf, uyf, Ty);
+        const float tA = f2_add_f(eT, lenA) - mrg, tB = f2_add_f(eT, lenB) - mrg;
+        const bool useless = f2_add_f(eS, lenB) > bf + mrg || f2_add_f(eE, lenA) > (Lcf - af) + mrg ||
+                             (tA > 0.f && tB > 0.f && tA * tA > fmaf(Xax, Xax, Xay * Xay) * (1.f + 0x1p-18f) &&
+                              tB * tB > fmaf(Xbx, Xbx, Xby * Xby) * (1.f + 0x1p-18f));
+        if (useless) return prop;
+        c.key = df.h + (gt0_s(axc) ? lenA.h : (sbits(bxc) < 0 ? lenB.h : -f_of(Ipy, fb)));
+    }
+    // ends at a vertex whose event is still to be made: not v2 of an occupied window, nor
+    // the shared vertex when the parent's end is at it
+    c.pend = (le_s(a, times_eps(Lc)) && !(occ && rt) && (rt || !le_s(A, tol)) ? kPendA : 0u) |
+             (sbits(Lc) - sbits(b) <= kSnapUlps && !(occ && !rt) && (!rt || sbits(L) - sbits(B) > kSnapUlps) ? kPendB : 0u);
+    c.he = che;
+    c.A = a;
+    c.B = b;
+    c.px = Ipx;
+    c.py = Ipy;
+    c.ax = axc;
+    c.bx = bxc;
+    has_child = true;
     return prop;
 }
 
 // Windows in flight per warp: the shared-memory queue of chained children holds at most
-// one window per lane, in two buffers (read / written by alternate rounds) of 7 doubles
-// and 4 ints per entry (blocks of at most 256 threads: 36 KB).
-constexpr int kPropQueueBytesPerThread = 2 * (7 * 8 + 4 * 4);
-constexpr int kPropMaxWarps = 8;      // warps per block at most (256 threads)
+// one window per lane, 7 doubles and 4 ints an entry.  A round reads its entries before
+// it writes the next round's, so one buffer serves both.
+constexpr int kPropQueueBytesPerThread = 7 * 8 + 4 * 4;
 
 // Step 3 of the iteration (Algorithm 2 over the selected windows), persistent.  Every
 // warp advances on its own in rounds: in each round lane t takes entry t of the warp's
@@ -712,66 +714,65 @@ constexpr int kPropMaxWarps = 8;      // warps per block at most (256 threads)
 // A warp takes at most ceil(selected / resident warps) fresh windows at once (take_min
 // at least), so that a short list (the first iterations, a ring-shaped frontier) keeps
 // every resident warp busy and the chains' deferred children fill the free lanes.
-// 168 registers a thread at most (164 used, no spills): 6 blocks of 64 threads per SM.
 // PROV: also record the distance events (geodesic paths).
 template <bool PROV>
-__global__ void __maxnreg__(168) k_propagate(Work w, int hops, int tail_cut, int take_min) {
+__global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int take_min) {
     extern __shared__ double q_mem[];   // blockDim.x * kPropQueueBytesPerThread bytes
-    const int QB = 2 * blockDim.x;
+    const int QB = blockDim.x;
     double* q_d = q_mem;
     double* q_A = q_d + QB;
     double* q_B = q_A + QB;
     double* q_px = q_B + QB;
     double* q_py = q_px + QB;
-    double* q_IA = q_py + QB;
-    double* q_IB = q_IA + QB;
-    int* q_he = reinterpret_cast<int*>(q_IB + QB);
+    double* q_ax = q_py + QB;
+    double* q_bx = q_ax + QB;
+    int* q_he = reinterpret_cast<int*>(q_bx + QB);
     int* q_inst = q_he + QB;
     int* q_src = q_inst + QB;
     int* q_hop = q_src + QB;
-    // per warp and buffer: entries written (by the round that writes that buffer)
-    __shared__ int s_cnt[kPropMaxWarps][2];
     Counters* cnt = w.cnt;
     if (cnt->halt) return;
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const int wid = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const int it = cnt->iter;
     const int n = min(cnt->n_sel, w.sel_cap);
     FanReq* req = w.req[it & 1];
-    const int room = w.arena_cap / 2 - 2 * (int)(gridDim.x * blockDim.x);
+    // The arena cannot overflow: past `room` a warp stops chaining once it has seen the fill
+    // (at its next write, of 32 children at most), and after that its 32 queued windows
+    // and each fresh one make two children at most.
+    const int threads = (int)(gridDim.x * blockDim.x);
+    const int room = min(w.arena_cap / 2, w.arena_cap - 2 * n - 3 * threads);
     // Fresh windows a warp holds at once: a short selected list is spread over all
     // resident warps (take_min a warp at least), so that the lanes left free take the
     // deferred children of the chains instead of the arena; a list of a warp's width per
     // resident warp or more fills whole warps.
-    const int nwarps = (int)(gridDim.x * (blockDim.x >> 5));
+    const int nwarps = threads >> 5;
     const int quota = max(take_min, min(32, (n + nwarps - 1) / max(nwarps, 1)));
     const unsigned take_mask = quota >= 32 ? 0xffffffffu : (1u << quota) - 1u;
-    // the arena fill this warp last saw (updated whenever it reserves arena slots): a
-    // warp overshoots the room by at most one round of its own writes
+    // the arena fill this warp last saw (updated whenever it reserves arena slots)
     int seen_child = *(volatile int*)&cnt->n_child;
-    // statistics, kept per thread and added to the counters once when the warp ends
+    // statistics, kept per warp and added to the counters once when the warp ends
     unsigned n_prop = 0, n_chain = 0, n_exam = 0, n_occ = 0, n_comp = 0, n_ray = 0;
-    if (lane == 0) s_cnt[wid][0] = s_cnt[wid][1] = 0;
-    bool dry = false;          // uniform over the warp: the selected list is exhausted
-    for (int r = 0;; ++r) {
-        const int rb = r & 1, wb = rb ^ 1;
-        __syncwarp();          // last round's queue writes are visible, its reads are done
-        const int nq = min(s_cnt[wid][rb], 32);
-        __syncwarp();          // every lane has read the count before it is reused
-        if (lane == 0) s_cnt[wid][wb] = 0;
-        __syncwarp();
-        const int qr = rb * blockDim.x + wid * 32 + lane;   // this lane's entry in the read buffer
-        bool have = lane < nq, task = false;
-        int h = 0, inst = 0, src = -1, hop = 0;
-        double d = 0.0, A = 0.0, B = 0.0, px = 0.0, py = 0.0, cIA = -1.0, cIB = -1.0;
+    bool dry = false;          // the selected list is exhausted
+    int nq = 0;                // queue entries
+    for (;;) {
+        LaneWin W;
+        bool have = lane < nq;
+        W.task = false;
+        W.h = W.inst = W.hop = 0;
+        W.src = -1;
+        W.pend = 0u;
+        W.d = W.A = W.B = W.px = W.py = W.ax = W.bx = 0.0;
+        const int q0 = threadIdx.x & ~31;                   // the warp's region of the queue
         if (have) {
-            h = q_he[qr]; inst = q_inst[qr]; src = q_src[qr]; hop = q_hop[qr];
-            task = (hop & kHopTask) != 0;
-            hop &= ~kHopTask;
-            d = q_d[qr]; A = q_A[qr]; B = q_B[qr]; px = q_px[qr]; py = q_py[qr];
-            cIA = q_IA[qr]; cIB = q_IB[qr];
+            const int q = q0 + lane;
+            W.h = q_he[q]; W.inst = q_inst[q]; W.src = q_src[q];
+            const int hop = q_hop[q];
+            W.task = (hop & kHopTask) != 0;
+            W.pend = (unsigned)hop << (30 - kHopPend) & (kPendA | kPendB);
+            W.hop = hop & kHopMask;
+            W.d = q_d[q]; W.A = q_A[q]; W.B = q_B[q]; W.px = q_px[q]; W.py = q_py[q]; W.ax = q_ax[q]; W.bx = q_bx[q];
         }
         const unsigned need = __ballot_sync(full, !have) & take_mask;   // lanes nq.. below the quota
         if (need && !dry) {
@@ -782,64 +783,85 @@ __global__ void __maxnreg__(168) k_propagate(Work w, int hops, int tail_cut, int
             if ((need >> lane) & 1u) {
                 const int idx = base + __popc(need & lt);
                 if (idx < n) {
-                    h = w.sel.he[idx]; inst = w.sel.inst[idx]; d = w.sel.d[idx]; src = w.sel.src[idx];
-                    A = w.sel.A[idx]; B = w.sel.B[idx]; px = w.sel.px[idx]; py = w.sel.py[idx];
-                    cIA = w.sel.IA[idx]; cIB = w.sel.IB[idx];
+                    const int fi = w.sel.inst[idx];
+                    W.h = w.sel.he[idx]; W.src = w.sel.src[idx]; W.d = w.sel.d[idx];
+                    W.A = w.sel.A[idx]; W.B = w.sel.B[idx]; W.px = w.sel.px[idx]; W.py = w.sel.py[idx];
+                    W.inst = fi & kInstMask;
+                    W.pend = (unsigned)fi & ~(unsigned)kInstMask;
+                    W.ax = W.A - W.px;
+                    W.bx = W.B - W.px;
                     have = true;
                 }
             }
         }
-        if (!__any_sync(full, have)) {             // nothing queued and nothing left to take
-            const unsigned sums[6] = {__reduce_add_sync(full, n_prop), __reduce_add_sync(full, n_chain),
-                                      __reduce_add_sync(full, n_exam), __reduce_add_sync(full, n_occ),
-                                      __reduce_add_sync(full, n_comp), __reduce_add_sync(full, n_ray)};
+        const unsigned live = __ballot_sync(full, have);    // (also: every lane has read its entry)
+        if (!live) {                                        // nothing queued and nothing left to take
+            const unsigned long long sums[6] = {n_prop, n_chain, n_exam, n_occ, n_comp, n_ray};
             unsigned long long* dst[6] = {&cnt->propagated, &cnt->chained, &cnt->examined, &cnt->occupied,
                                           &cnt->children, &cnt->rays};
-            if (lane < 6 && sums[lane]) atomicAdd(dst[lane], (unsigned long long)sums[lane]);
+            if (lane == 0)
+                for (int j = 0; j < 6; ++j)
+                    if (sums[j]) atomicAdd(dst[j], sums[j]);
             break;
         }
-        ChildOut c0, c1;
-        int nch = 0, occ = 0, ncomp = 0, nray = 0;
-        bool prop = false;
-        const int wo = wb * blockDim.x + wid * 32;  // the warp's region of the write buffer
-        const TaskQueue tq{q_d + wo, q_A + wo, q_B + wo, q_px + wo, q_py + wo, q_IA + wo, q_IB + wo,
-                           q_he + wo, q_inst + wo, q_src + wo, q_hop + wo, &s_cnt[wid][wb], 32};
-        if (have)
-            prop = propagate_window<PROV>(w, cnt, req, inst, src, d, h, A, B, px, py, task, hop, tq, c0, c1, nch,
-                                          occ, ncomp, nray, cIA, cIB);
-        bool cont = have && nch > 0 && hop + 1 < hops && le_s(c0.key, w.ctl[inst].tau) &&
+        ChildOut c;
+        bool child = false, defer = false, occ = false, comp = false, prop = false;
+        if (have) prop = propagate_window<PROV>(w, cnt, req, W, c, child, defer, occ, comp);
+        __syncwarp();
+        bool cont = child && W.hop + 1 < hops && c.key <= w.ctl[W.inst].tauf &&
                     (!dry || nq >= tail_cut) && seen_child < room;
-        // the continuing child goes to the queue while it has room, every other child to
-        // the arena
-        const int qs = warp_reserve(&s_cnt[wid][wb], cont ? 1 : 0);
-        if (cont && qs >= 32) cont = false;
+        // the deferred left children first, then the continuing children while the queue
+        // has room; every other child goes to the arena
+        const unsigned tm = __ballot_sync(full, defer), cm = __ballot_sync(full, cont);
+        const int ntask = __popc(tm);
+        if (defer) {
+            const int q = q0 + __popc(tm & lt);
+            q_he[q] = W.h; q_inst[q] = W.inst; q_src[q] = W.src; q_hop[q] = W.hop | kHopTask;
+            q_d[q] = W.d; q_A[q] = W.A; q_B[q] = W.B; q_px[q] = W.px; q_py[q] = W.py; q_ax[q] = W.ax; q_bx[q] = W.bx;
+        }
         if (cont) {
-            const int q = wo + qs;
-            q_he[q] = c0.he; q_inst[q] = inst; q_src[q] = src; q_hop[q] = hop + 1;
-            q_d[q] = d; q_A[q] = c0.A; q_B[q] = c0.B; q_px[q] = c0.px; q_py[q] = c0.py;
-            q_IA[q] = c0.IA; q_IB[q] = c0.IB;
+            const int slot = ntask + __popc(cm & lt);
+            if (slot < 32) {
+                const int q = q0 + slot;
+                q_he[q] = c.he; q_inst[q] = W.inst; q_src[q] = W.src;
+                q_hop[q] = (W.hop + 1) | (int)(c.pend >> (30 - kHopPend));
+                q_d[q] = W.d; q_A[q] = c.A; q_B[q] = c.B; q_px[q] = c.px; q_py[q] = c.py; q_ax[q] = c.ax; q_bx[q] = c.bx;
+            } else {
+                cont = false;
+            }
         }
-        const int nwrite = have ? (cont ? nch - 1 : nch) : 0;
-        int fill = -1;
-        const int slot = warp_reserve(&cnt->n_child, nwrite, &fill);
-        if (fill >= 0) seen_child = fill;
-        if (nwrite > 0) {
-            const ChildOut& cf = cont ? c1 : c0;
-            if (slot < w.arena_cap)
-                store_win(w.arena, slot, cf.he, inst, d, cf.A, cf.B, cf.px, cf.py, cf.key, src, cf.IA, cf.IB);
-            else atomicOr(&cnt->error, kErrPoolFull);
+        const unsigned wm = __ballot_sync(full, child && !cont);
+        if (wm) {
+            int base = 0;
+            if (lane == 0) base = atomicAdd(&cnt->n_child, __popc(wm));
+            base = __shfl_sync(full, base, 0);
+            seen_child = base + __popc(wm);
+            if (child && !cont) {
+                const int slot = base + __popc(wm & lt);
+                if (slot < w.arena_cap) {
+                    w.arena.he[slot] = c.he;
+                    w.arena.inst[slot] = W.inst | (int)c.pend;
+                    w.arena.src[slot] = W.src;
+                    w.arena.d[slot] = W.d;
+                    w.arena.A[slot] = c.A;
+                    w.arena.B[slot] = c.B;
+                    w.arena.px[slot] = c.px;
+                    w.arena.py[slot] = c.py;
+                } else {
+                    atomicOr(&cnt->error, kErrPoolFull);
+                }
+            }
         }
-        if (nwrite > 1) {
-            if (slot + 1 < w.arena_cap)
-                store_win(w.arena, slot + 1, c1.he, inst, d, c1.A, c1.B, c1.px, c1.py, c1.key, src, c1.IA, c1.IB);
-            else atomicOr(&cnt->error, kErrPoolFull);
-        }
-        n_prop += prop ? 1u : 0u;
-        n_chain += cont ? 1u : 0u;
-        n_exam += have && !task ? 1u : 0u;
-        n_occ += (unsigned)occ;
-        n_comp += (unsigned)ncomp;
-        n_ray += (unsigned)nray;
+        const unsigned om = __ballot_sync(full, occ), pm = __ballot_sync(full, comp);
+        const unsigned km = __ballot_sync(full, W.task);
+        n_prop += __popc(__ballot_sync(full, prop));
+        n_exam += __popc(live & ~km);
+        n_occ += __popc(om & ~km);
+        n_comp += __popc(pm);
+        n_ray += 2 * __popc(pm) - __popc(pm & om);
+        nq = min(32, ntask + __popc(cm));
+        n_chain += nq - ntask;
+        __syncwarp();          // the queue is written
     }
 }
 
@@ -1125,8 +1147,7 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
                 w.arena.he[slot] = -1;
                 continue;
             }
-            const double key = D + (px < A ? IA : (px > B ? IB : -py));
-            store_win(w.arena, slot, Ro.twin, rq.inst, D, A, B, px, py, key, (int)v, IA, IB);
+            store_win(w.arena, slot, {Ro.twin, rq.inst, (int)v, kPendA | kPendB, D, A, B, px, py, 0.0});
             ++n_fwin;
         }
     }
@@ -1156,17 +1177,21 @@ __global__ void __launch_bounds__(256) k_append(Work w, const unsigned* __restri
         // without a sort (keys == nullptr) the arena is appended in its own order
         unsigned k = i < n ? (keys ? keys[i] : (w.arena.he[i] < 0 ? ~0u : 0u)) : ~0u;
         bool keep = k != ~0u;
-        int he = 0, inst = 0, src = -1;
-        double d = 0, A = 0, B = 0, px = 0, py = 0, key = 0, IA = 0, IB = 0;
+        Win W{0, 0, -1, 0u, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         int trimmed = 0;
         if (keep) {
-            load_win(w.arena, keys ? vals[i] : i, he, inst, d, A, B, px, py, key, src, IA, IB);
-            const Inst& I = w.inst[inst];
-            const HERec R = I.rec[he];
+            W = load_win(w.arena, keys ? vals[i] : i);
+            const double d = W.d, A = W.A, B = W.B;
+            const Inst& I = w.inst[W.inst];
+            const HERec R = I.rec[W.he];
+            // the window's distance back to the source: from the point of [A, B] nearest I
+            const double foot = W.px < A ? A - W.px : (W.px > B ? B - W.px : 0.0);
+            const double key = d + (foot == 0.0 ? -W.py : sqrt_nr(fma(foot, foot, W.py * W.py)));
+            W.key = key;
             // re-filter against the distances after this iteration's events (the window
             // is nowhere closer than `key`)
             double g0 = ldg_dist(I.g, R.v0 & ~kPseudoBit), g1 = ldg_dist(I.g, R.v1 & ~kPseudoBit);
-            if (dominated(key, g0 + B) || dominated(key, g1 + (R.L - A)) || stale_source(I, src, d)) keep = false;
+            if (dominated(key, g0 + B) || dominated(key, g1 + (R.L - A)) || stale_source(I, W.src, d)) keep = false;
             // per-edge trimming: a window on the same edge that covers [A, B] and is
             // everywhere shorter than this window's nearest point makes it useless
             if (keep && trim) {
@@ -1188,10 +1213,14 @@ __global__ void __launch_bounds__(256) k_append(Work w, const unsigned* __restri
         int slot = warp_reserve(&cnt->n_app, keep ? 1 : 0);
         if (keep) {
             int pos = n_rest + slot;
-            if (pos < w.pool_cap) store_win(nxt, pos, he, inst, d, A, B, px, py, key, src, IA, IB);
-            else atomicOr(&cnt->error, kErrPoolFull);
+            if (pos < w.pool_cap) {
+                store_win(nxt, pos, W);
+                nxt.key[pos] = W.key;
+            } else {
+                atomicOr(&cnt->error, kErrPoolFull);
+            }
         }
-        pool_stat(w, ps, inst, key, keep);
+        pool_stat(w, ps, W.inst, W.key, keep);
         warp_add_ull(&cnt->trimmed, trimmed);
         warp_add_ull(&cnt->created, keep ? 1 : 0);
     }
@@ -1313,7 +1342,8 @@ static void drop_graph(Workspace* ws) {
     ws->graph = nullptr;
 }
 
-static cudaError_t alloc_soa(Alloc& a, WinSoA& s, int cap) {
+// `keyed`: the pending pools; the work list and the arena hold no keys.
+static cudaError_t alloc_soa(Alloc& a, WinSoA& s, int cap, bool keyed) {
     cudaError_t e;
     if ((e = a.get(&s.he, cap))) return e;
     if ((e = a.get(&s.inst, cap))) return e;
@@ -1322,25 +1352,26 @@ static cudaError_t alloc_soa(Alloc& a, WinSoA& s, int cap) {
     if ((e = a.get(&s.B, cap))) return e;
     if ((e = a.get(&s.px, cap))) return e;
     if ((e = a.get(&s.py, cap))) return e;
-    if ((e = a.get(&s.key, cap))) return e;
-    if ((e = a.get(&s.IA, cap))) return e;
-    if ((e = a.get(&s.IB, cap))) return e;
+    if (keyed && (e = a.get(&s.key, cap))) return e;
     return a.get(&s.src, cap);
 }
 
 // Capacities: the work list holds sel_cap windows (more selected windows simply stay
 // pending), the child arena 6 * sel_cap (two children per selected window plus the half
-// that chaining may fill, so it cannot overflow), the pending pools at least twice the
+// that chaining may fill) and what the resident propagation warps may hold when it is
+// full (3 a thread: k_propagate's `room`), so it cannot overflow, the pending pools at least twice the
 // arena (the loop halts for the host to grow them before they could overflow), and the
 // fan requests req_cap (an overflow fails the attempt; the solve is then re-run with
 // twice the room).
+static int arena_for(int sel_cap) { return 6 * sel_cap + 4 * 512 * sm_count(); }
+
 static pch_status ensure_pools(Workspace* ws, int sel_cap, int pool_cap, int req_min = 0) {
-    int arena_cap = 6 * sel_cap;
+    int arena_cap = arena_for(sel_cap);
     if (pool_cap < 2 * arena_cap) pool_cap = 2 * arena_cap;
     if (sel_cap <= ws->sel_cap && pool_cap <= ws->pool_cap && req_min <= ws->req_cap) return PCH_OK;
     sel_cap = std::max(sel_cap, ws->sel_cap);
     pool_cap = std::max(pool_cap, ws->pool_cap);
-    arena_cap = 6 * sel_cap;
+    arena_cap = arena_for(sel_cap);
     const int req_cap = std::max({4 * sel_cap + (1 << 20), req_min, ws->req_cap});
     const int sort_blocks = 2 * sm_count();
     drop_graph(ws);
@@ -1348,10 +1379,10 @@ static pch_status ensure_pools(Workspace* ws, int sel_cap, int pool_cap, int req
     Work nw = w;
     Alloc fresh;
     cudaError_t e = cudaSuccess;
-    if (!e) e = alloc_soa(fresh, nw.pool[0], pool_cap);
-    if (!e) e = alloc_soa(fresh, nw.pool[1], pool_cap);
-    if (!e) e = alloc_soa(fresh, nw.sel, sel_cap);
-    if (!e) e = alloc_soa(fresh, nw.arena, arena_cap);
+    if (!e) e = alloc_soa(fresh, nw.pool[0], pool_cap, true);
+    if (!e) e = alloc_soa(fresh, nw.pool[1], pool_cap, true);
+    if (!e) e = alloc_soa(fresh, nw.sel, sel_cap, false);
+    if (!e) e = alloc_soa(fresh, nw.arena, arena_cap, false);
     if (!e) e = fresh.get(&nw.req[0], req_cap);
     if (!e) e = fresh.get(&nw.req[1], req_cap);
     if (!e) e = fresh.get(&nw.sort_key[0], arena_cap);
@@ -1377,8 +1408,6 @@ static pch_status ensure_pools(Workspace* ws, int sel_cap, int pool_cap, int req
             cudaMemcpy(nw.pool[p].py, w.pool[p].py, n * 8, cudaMemcpyDeviceToDevice);
             cudaMemcpy(nw.pool[p].key, w.pool[p].key, n * 8, cudaMemcpyDeviceToDevice);
             cudaMemcpy(nw.pool[p].src, w.pool[p].src, n * 4, cudaMemcpyDeviceToDevice);
-            cudaMemcpy(nw.pool[p].IA, w.pool[p].IA, n * 8, cudaMemcpyDeviceToDevice);
-            cudaMemcpy(nw.pool[p].IB, w.pool[p].IB, n * 8, cudaMemcpyDeviceToDevice);
             cudaMemcpy(nw.req[p], w.req[p], sizeof(FanReq) * (size_t)ws->req_cap, cudaMemcpyDeviceToDevice);
         }
         e = cudaDeviceSynchronize();
@@ -1631,18 +1660,13 @@ static pch_status run_solve(Workspace* ws, cudaStream_t s, const SolveCfg& cfg_i
         stats->children_computed = (int64_t)c.children;
         stats->fan_ties = (int64_t)c.fan_ties;
         // algorithmic FP64 operations of k_propagate (add, sub, mul, div, sqrt = 1; fma = 2),
-        // counted per code path of propagate_window: a window taken from the work list 7
-        // (2 offsets, 5 for the endpoint filter), a chained window 2 (its filter was its
-        // parent's child filter), a window that passed +9 (occupancy test), an occupied
-        // one +17 (crossing point and its angle_split position, |I v2|, event distance),
-        // a child +25 (frame change 7: the child edge's unit axis comes with the half-edge
-        // record; width 1, child filter 16, key 1) plus 8 per ray intersected (two per
-        // child, one when the window occupies v2); the filter's test against the parent
-        // edge's far vertex at the second end (+11) is not counted: it is evaluated only
-        // where the first end's test holds (the warp runs it when any lane needs it)
+        // counted per code path of propagate_window: a window taken from the work list 2
+        // (its ends' offsets), an occupied one 14 (crossing point, its angle_split position,
+        // |I v2|, event distance), a child 10 (frame change 8, its ends' offsets 2) plus 7
+        // per ray intersected (two per child, one when the window occupies v2); the tests
+        // run in FP32 and are not counted
         const unsigned long long fresh = c.examined > c.chained ? c.examined - c.chained : 0ull;
-        stats->prop_fp64_ops = (int64_t)(7ull * fresh + 2ull * c.chained + 9ull * c.propagated +
-                                         17ull * c.occupied + 25ull * c.children + 8ull * c.rays);
+        stats->prop_fp64_ops = (int64_t)(2ull * fresh + 14ull * c.occupied + 10ull * c.children + 7ull * c.rays);
         for (int p = 0; p < 6; ++p) stats->ms_phase[p] = phase_ms[p];
     }
     return PCH_OK;
@@ -1659,7 +1683,7 @@ static SolveCfg make_cfg(const pch_options* opt, int n_inst, long long total_key
     cfg.trim = !(opt && (opt->flags & PCH_FLAG_NO_TRIM));
     cfg.full_fan = (opt && (opt->flags & PCH_FLAG_FULL_FAN)) ? 1 : 0;
     cfg.profile = (opt && (opt->flags & PCH_FLAG_PROFILE)) ? 1 : 0;
-    cfg.hops = (opt && opt->hops > 0) ? opt->hops : default_hops();
+    cfg.hops = std::min((opt && opt->hops > 0) ? opt->hops : default_hops(), kHopMask);
     cfg.tail_cut = default_tail_cut();
     cfg.take_min = default_take_min();
     cfg.unroll = 2;
@@ -1772,6 +1796,7 @@ pch_status solve_instances(pch_mesh* const* meshes, int n_inst, const SrcDev* sr
         I.keybase = kbase;
         kbase += dm.nh;
         I.lbar = dm.lbar; I.ilbar = 1.0 / dm.lbar;
+        I.fbias = (unsigned)(1023 - 127 + std::ilogb(dm.lbar)) << 20;
         InstCtl& c = hctl[i];
         std::memset(&c, 0, sizeof c);
         c.kmin = ~0ull;

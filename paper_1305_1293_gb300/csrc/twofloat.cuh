@@ -1,0 +1,74 @@
+// Two-float images of doubles for the propagation kernel's order tests.
+//
+// GB300's FP64 unit is 64 times slower than its FP32 units, and most of a window's
+// arithmetic only decides something (does a ray pass a vertex, is a window dominated).
+// Such a test is evaluated in FP32, on images of the doubles scaled by a power of two
+// (the mesh's mean edge length lands in [1, 2)), with a bound of its error: it acts only
+// where the sign is certain.  A value becomes the unevaluated sum h + l of two floats by
+// integer operations (h its leading 24 bits, l the next 23: truncation below 2^-46
+// relative); F2F conversions would run on the FP64 unit.  Sums use the exact two-sum of
+// D. Knuth (The Art of Computer Programming, vol. 2, section 4.2.2, theorem B), products the exact
+// FMA residual.  Zero and magnitudes below the float range become 0, magnitudes above it
+// (and infinities) infinity or NaN; every test is written so that a NaN decides nothing.
+#pragma once
+#include <cuda_runtime.h>
+
+#include "fastmath.cuh"
+
+namespace pch {
+
+struct F2 {
+    float h, l;
+};
+
+// |x| as a float bit pattern, truncated; `bias` = (1023 - 127 + E) << 20 for a scale 2^-E.
+__device__ __forceinline__ unsigned f_mag_bits(double x, unsigned bias) {
+    const unsigned m = (unsigned)__double2hiint(x) & 0x7fffffffu;
+    const unsigned f = __funnelshift_l((unsigned)__double2loint(x), min(m - bias, 0x0ff00000u), 3);
+    return m < bias + 0x00100000u ? 0u : f;
+}
+// x scaled, rounded towards zero.
+__device__ __forceinline__ float f_of(double x, unsigned bias) {
+    return __uint_as_float(f_mag_bits(x, bias) | ((unsigned)__double2hiint(x) & 0x80000000u));
+}
+// |x| scaled, as a two-float.
+__device__ __forceinline__ F2 f2_mag(double x, unsigned bias) {
+    const unsigned f = f_mag_bits(x, bias);
+    // bits 28..6 of the low word follow the leading 24 bits of the mantissa
+    const float m = __uint_as_float((((unsigned)__double2loint(x) >> 6) & 0x7fffffu) | 0x4b000000u) - 8388608.f;
+    const float ulp = __uint_as_float(max(f & 0x7f800000u, 46u << 23) - (46u << 23));
+    return {__uint_as_float(f), m * ulp};
+}
+
+__device__ __forceinline__ F2 two_sum(float a, float b) {
+    const float s = a + b, bb = s - a;
+    return {s, (a - (s - bb)) + (b - bb)};
+}
+
+// d - g for nonnegative two-floats (an exact leading sum, the rest rounded).
+__device__ __forceinline__ F2 f2_sub(F2 d, F2 g) {
+    F2 r = two_sum(d.h, -g.h);
+    r.l += d.l - g.l;
+    return r;
+}
+// x + y rounded to one float.
+__device__ __forceinline__ float f2_add_f(F2 x, F2 y) {
+    const F2 s = two_sum(x.h, y.h);
+    return s.h + (s.l + (x.l + y.l));
+}
+// x^2 as a two-float (the square of the low part, below 2^-46, is dropped).
+__device__ __forceinline__ F2 f2_sq(F2 x) {
+    const float p = x.h * x.h;
+    return {p, fmaf(x.h + x.h, x.l, fmaf(x.h, x.h, -p))};
+}
+// sqrt(x^2 + yy) as a two-float, relative error below 2^-44.
+__device__ __forceinline__ F2 f2_hyp(F2 x, F2 yy) {
+    const F2 xx = f2_sq(x);
+    const F2 s = two_sum(xx.h, yy.h);
+    const float e = s.l + (xx.l + yy.l);
+    const float r = rsqrt_approx_f32(s.h);
+    const float q = s.h * r;
+    return {q, 0.5f * r * (fmaf(-q, q, s.h) + e)};
+}
+
+}  // namespace pch
