@@ -27,19 +27,19 @@ __device__ __forceinline__ int face_mask(const double d[3], double L) {
     return m;
 }
 
-__device__ __forceinline__ void face_dist(const HERec* __restrict__ rec, const double* __restrict__ dist, int f,
+__device__ __forceinline__ void face_dist(const int* __restrict__ tri, const double* __restrict__ dist, int f,
                                           double d[3]) {
 #pragma unroll
-    for (int i = 0; i < 3; ++i) d[i] = dist[rec[3 * f + i].v0 & ~kPseudoBit];
+    for (int i = 0; i < 3; ++i) d[i] = dist[tri[3 * f + i]];
 }
 
-__global__ void k_contour_count(const HERec* __restrict__ rec, int nf, const double* __restrict__ dist,
+__global__ void k_contour_count(const int* __restrict__ tri, int nf, const double* __restrict__ dist,
                                 const double* __restrict__ levels, int n_levels, int* count,
                                 unsigned long long* total) {
     unsigned long long t = 0;
     for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += gridDim.x * blockDim.x) {
         double d[3];
-        face_dist(rec, dist, f, d);
+        face_dist(tri, dist, f, d);
         int c = 0;
         for (int l = 0; l < n_levels; ++l) c += face_mask(d, levels[l]) != 0;
         count[f] = c;
@@ -52,12 +52,12 @@ __global__ void k_contour_count(const HERec* __restrict__ rec, int nf, const dou
 // crossing on the edge whose start corner is outside, so that the inside (distance
 // below L) lies to the left of the segment seen from the face's front side (corners
 // counter-clockwise).
-__global__ void k_contour_write(const HERec* __restrict__ rec, int nf, const double* __restrict__ dist,
+__global__ void k_contour_write(const int* __restrict__ tri, int nf, const double* __restrict__ dist,
                                 const double* __restrict__ levels, int n_levels, const int* __restrict__ offset,
                                 long long capacity, pch_contour_segment* __restrict__ out) {
     for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += gridDim.x * blockDim.x) {
         double d[3];
-        face_dist(rec, dist, f, d);
+        face_dist(tri, dist, f, d);
         long long o = offset[f];
         for (int l = 0; l < n_levels; ++l) {
             const double L = levels[l];
@@ -122,7 +122,7 @@ extern "C" pch_status pch_iso_contours(const pch_mesh* m, const double* dist, in
     const double* dd = dist_on_device ? dist : ddist;
     const int grid = sm_count() * 4;
     if (!e) {
-        k_contour_count<<<grid, 256, 0, s>>>(m->dm.rec, nf, dd, dlev, n_levels, cnt, dtotal);
+        k_contour_count<<<grid, 256, 0, s>>>(m->dm.tri, nf, dd, dlev, n_levels, cnt, dtotal);
         e = cudaGetLastError();
     }
     if (!e) e = cudaMemcpy(&total, dtotal, sizeof(unsigned long long), cudaMemcpyDeviceToHost);
@@ -133,7 +133,7 @@ extern "C" pch_status pch_iso_contours(const pch_mesh* m, const double* dist, in
         e = exclusive_scan(cnt, off, nf, tmp, s);
         if (!e && keep > 0) e = cudaMalloc(&dseg, sizeof(pch_contour_segment) * (size_t)keep);
         if (!e && keep > 0) {
-            k_contour_write<<<grid, 256, 0, s>>>(m->dm.rec, nf, dd, dlev, n_levels, off, keep, dseg);
+            k_contour_write<<<grid, 256, 0, s>>>(m->dm.tri, nf, dd, dlev, n_levels, off, keep, dseg);
             e = cudaGetLastError();
         }
         if (!e && keep > 0) e = cudaMemcpy(segments, dseg, sizeof(pch_contour_segment) * (size_t)keep, cudaMemcpyDeviceToHost);

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "pch_host.h"
+#include "radix.cuh"
 
 namespace pch {
 
@@ -259,6 +260,83 @@ __global__ void k_rec_ids(int nh, const int* __restrict__ twin, const unsigned c
     }
 }
 
+// ---------------------------------------------------------------- face order
+// Faces are kept in the order of the Morton codes of their centroids (the Z-order curve
+// of G. M. Morton, 1966): neighbours on the surface are then neighbours in memory, whatever
+// order the caller's list has.  A window reads the 96-byte records of a band of the
+// surface; scattered over the 1.5 GB of a 5.2M-face sphere (whose subdivision puts the four
+// children of a face a quarter of the list apart) those reads were bound by address
+// translation and L2 misses: a field took 647 ms, and takes 335 in this order.  A mesh of
+// fewer than kReorderFaces faces (its records fit L2 and the TLBs) gains nothing and
+// keeps its order: 8.4 ms either way at 327,680 faces, 46 against 39 at 1,310,720.
+constexpr int kReorderFaces = 1 << 19;
+constexpr int kMortonBits = 24;
+
+// Signed 64-bit image of a double whose integer order is the doubles' order.
+__device__ __forceinline__ long long ordered(double x) {
+    const long long b = __double_as_longlong(x);
+    return b < 0 ? b ^ 0x7fffffffffffffffll : b;
+}
+__device__ __forceinline__ double unordered(long long b) {
+    return __longlong_as_double(b < 0 ? b ^ 0x7fffffffffffffffll : b);
+}
+
+// box[0..2]: minimum, box[3..5]: minimum of the negated coordinates.
+__global__ void __launch_bounds__(256) k_bounds(int nv, const double* __restrict__ xyz, long long* box) {
+    long long m[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) m[j] = 0x7fffffffffffffffll;
+    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += gridDim.x * blockDim.x) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const double x = xyz[3 * (size_t)v + j];
+            m[j] = min(m[j], ordered(x));
+            m[j + 3] = min(m[j + 3], ordered(-x));
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m[j] = min(m[j], __shfl_xor_sync(0xffffffffu, m[j], o));
+        if ((threadIdx.x & 31) == 0) atomicMin(box + j, m[j]);
+    }
+}
+
+__device__ __forceinline__ unsigned spread3(unsigned x) {   // 8 bits, two zeros between
+    x = (x | x << 8) & 0x00f00fu;
+    x = (x | x << 4) & 0x0c30c3u;
+    return (x | x << 2) & 0x249249u;
+}
+
+__global__ void k_morton(int nf, const double* __restrict__ xyz, const int* __restrict__ tri, const long long* box,
+                         unsigned* key) {
+    double lo[3], ext = 0.0;
+    for (int j = 0; j < 3; ++j) {
+        lo[j] = unordered(box[j]);
+        ext = fmax(ext, -unordered(box[j + 3]) - lo[j]);
+    }
+    const double scale = 256.0 / (3.0 * ext);
+    for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += gridDim.x * blockDim.x) {
+        unsigned code = 0;
+        for (int j = 0; j < 3; ++j) {
+            double s = 0.0;
+            for (int c = 0; c < 3; ++c) s += xyz[3 * (size_t)tri[3 * f + c] + j] - lo[j];
+            const double q = s * scale;
+            code |= spread3(q > 0.0 ? (unsigned)fmin(q, 255.0) : 0u) << j;   // (a NaN: 0)
+        }
+        key[f] = code;
+    }
+}
+
+__global__ void k_permute_faces(int nf, const int* __restrict__ tri, const int* __restrict__ perm, int* tri_out,
+                                int* finv) {
+    for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += gridDim.x * blockDim.x) {
+        const int o = perm[f];
+        finv[o] = f;
+        for (int c = 0; c < 3; ++c) tri_out[3 * f + c] = tri[3 * o + c];
+    }
+}
+
 // Deterministic mean edge length and counts: block b reduces a fixed contiguous range of
 // half-edges and vertices in a fixed order, then k_stats_final adds the kStatBlocks
 // partial results in a fixed tree, so the sum does not depend on scheduling.
@@ -305,6 +383,7 @@ __global__ void __launch_bounds__(256) k_stats_final(const double* part_l, const
 
 static void free_mesh(DevMesh& d) {
     cudaFree(d.rec); cudaFree(d.vstart); cudaFree(d.vlist); cudaFree(d.hang);
+    cudaFree(d.tri); cudaFree(d.fperm); cudaFree(d.finv);
     cudaFree(d.vtheta); cudaFree(d.vphi); cudaFree(d.vflag); cudaFree(d.vrot); cudaFree(d.vtrot);
     d = DevMesh{};
 }
@@ -333,11 +412,14 @@ extern "C" pch_status pch_create_mesh(const double* vertices, int32_t n_vertices
     DevMesh d{};
     d.nv = nv; d.nf = nf; d.nh = nh;
     double* xyz = nullptr;
-    int *tri = nullptr, *twin = nullptr, *vcount = nullptr, *vout = nullptr, *err = nullptr, *scan_tmp = nullptr,
+    int *tri = nullptr, *tri_sorted = nullptr, *fval[2] = {nullptr, nullptr}, *fhist = nullptr, *twin = nullptr, *vcount = nullptr, *vout = nullptr, *err = nullptr, *scan_tmp = nullptr,
         *hvals = nullptr, *counts = nullptr;
     unsigned long long* hkeys = nullptr;
     double* lsum = nullptr;
     double* hang64 = nullptr;
+    unsigned* fkey[2] = {nullptr, nullptr};
+    long long* box = nullptr;
+    const int sort_blocks = 2 * sm_count();
     unsigned long long cap = 1;
     while (cap < 2ull * (unsigned long long)nh) cap <<= 1;
     pch_status st = PCH_OK;
@@ -356,7 +438,7 @@ extern "C" pch_status pch_create_mesh(const double* vertices, int32_t n_vertices
     } while (0)
     {
         MCHK(cudaMalloc(&xyz, sizeof(double) * 3 * nv));
-        MCHK(cudaMalloc(&tri, sizeof(int) * nh));
+        MCHK(cudaMalloc(&d.tri, sizeof(int) * nh));
         MCHK(cudaMalloc(&d.rec, sizeof(HERec) * nh));
         MCHK(cudaMalloc(&hang64, sizeof(double) * nh));
         MCHK(cudaMalloc(&d.hang, sizeof(float) * nh));
@@ -377,7 +459,8 @@ extern "C" pch_status pch_create_mesh(const double* vertices, int32_t n_vertices
         MCHK(cudaMalloc(&hkeys, sizeof(unsigned long long) * cap));
         MCHK(cudaMalloc(&hvals, sizeof(int) * cap));
         MCHK(cudaMemcpy(xyz, vertices, sizeof(double) * 3 * nv, cudaMemcpyHostToDevice));
-        MCHK(cudaMemcpy(tri, faces, sizeof(int) * nh, cudaMemcpyHostToDevice));
+        MCHK(cudaMemcpy(d.tri, faces, sizeof(int) * nh, cudaMemcpyHostToDevice));
+        tri = d.tri;
         MCHK(cudaMemset(err, 0, sizeof(int)));
         MCHK(cudaMemset(vcount, 0, sizeof(int) * (nv + 1)));
         MCHK(cudaMemset(vout, 0x7f, sizeof(int) * nv));
@@ -385,6 +468,26 @@ extern "C" pch_status pch_create_mesh(const double* vertices, int32_t n_vertices
         const int tb = 256;
         const int gb = std::max(1, std::min((nh + tb - 1) / tb, sm_count() * 8));
         const int gv = std::max(1, std::min((nv + tb - 1) / tb, sm_count() * 8));
+        if (nf >= kReorderFaces) {
+            MCHK(cudaMalloc(&tri_sorted, sizeof(int) * nh));
+            MCHK(cudaMalloc(&d.finv, sizeof(int) * nf));
+            for (int j = 0; j < 2; ++j) {
+                MCHK(cudaMalloc(&fkey[j], sizeof(unsigned) * nf));
+                MCHK(cudaMalloc(&fval[j], sizeof(int) * nf));
+            }
+            MCHK(cudaMalloc(&fhist, sizeof(int) * (kRsDigits * sort_blocks + 1)));
+            MCHK(cudaMalloc(&box, sizeof(long long) * 6));
+            MCHK(cudaMemset(box, 0x7f, sizeof(long long) * 6));
+            MCHK(cudaMemcpy(fhist + kRsDigits * sort_blocks, &nf, sizeof(int), cudaMemcpyHostToDevice));
+            k_bounds<<<gv, tb>>>(nv, xyz, box);
+            k_morton<<<gb, tb>>>(nf, xyz, tri, box, fkey[0]);
+            const int r = launch_sort_keys(fhist + kRsDigits * sort_blocks, nf, kMortonBits, fkey, fval, fhist, sort_blocks, 0);
+            d.fperm = fval[r];
+            fval[r] = nullptr;
+            k_permute_faces<<<gb, tb>>>(nf, tri, d.fperm, tri_sorted, d.finv);
+            MCHK(cudaGetLastError());
+            tri = tri_sorted;
+        }
         k_frames<<<gb, tb>>>(nh, xyz, tri, d.rec, hang64, err);
         k_hash_insert<<<gb, tb>>>(nh, tri, hkeys, hvals, cap - 1, err);
         k_twins<<<gb, tb>>>(nh, tri, hkeys, hvals, cap - 1, twin, vcount, vout);
@@ -414,7 +517,9 @@ extern "C" pch_status pch_create_mesh(const double* vertices, int32_t n_vertices
     }
 cleanup:
 #undef MCHK
-    cudaFree(xyz); cudaFree(tri); cudaFree(twin); cudaFree(vcount); cudaFree(vout); cudaFree(err);
+    cudaFree(xyz); cudaFree(tri_sorted); cudaFree(twin); cudaFree(box); cudaFree(fhist);
+    for (int j = 0; j < 2; ++j) { cudaFree(fkey[j]); cudaFree(fval[j]); }
+    cudaFree(vcount); cudaFree(vout); cudaFree(err);
     cudaFree(scan_tmp); cudaFree(hkeys); cudaFree(hvals); cudaFree(counts); cudaFree(lsum); cudaFree(hang64);
     if (st != PCH_OK) free_mesh(d);
     return st;

@@ -53,6 +53,11 @@ struct DevMesh {
     int nv, nf, nh;
     double lbar;           // mean edge length
     HERec* rec;            // [nh]
+    int* tri;              // [nh] vertex ids of the faces, in the caller's order
+    // the caller's face of every internal face and the reverse (nullptr: the same order);
+    // half-edges are internal everywhere but in results
+    int* fperm;            // [nf]
+    int* finv;             // [nf]
     int* vstart;           // [nv + 1] CSR of outgoing half-edges, one-ring order
     int* vlist;            // [nh]
     // angles, kept in FP32: they only steer the pseudo-source fans, whose wedges are
@@ -97,6 +102,8 @@ struct Inst {
     const double2* vrot;        // (cos, sin) of the angular position of every half-edge
     const double2* vtrot;       // (cos, sin) of the total angle of every vertex
     const unsigned char* vflag; // bit0: boundary vertex
+    const int* fperm;           // the caller's face of every internal face (nullptr: the same)
+    const int* finv;            // and the reverse
     unsigned long long* g;      // geod_dist[] as ordered u64 images of nonnegative doubles
     unsigned long long* ang;    // angle_split[]: packed (rounded-up distance, crossing position)
     unsigned* stamp;            // per-vertex iteration stamp (one fan request per iteration)

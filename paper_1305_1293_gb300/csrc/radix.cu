@@ -160,6 +160,20 @@ int launch_sort_children(const WinSoA& arena, const Inst* insts, const int* n_pt
     return src;
 }
 
+int launch_sort_keys(const int* n_ptr, int n_max, int key_bits, unsigned* key_buf[2], int* val_buf[2], int* hist,
+                     int blocks, cudaStream_t s) {
+    int src = 0;
+    for (int shift = 0; shift < key_bits; shift += kRsDigitBits) {
+        RsIn in{};
+        in.keys = key_buf[src];
+        in.vals = shift ? val_buf[src] : nullptr;   // the first pass numbers the elements
+        k_rs_hist<<<blocks, kRsThreads, 0, s>>>(in, n_ptr, n_max, shift, hist);
+        k_rs_scatter<<<blocks, kRsThreads, 0, s>>>(in, key_buf[src ^ 1], val_buf[src ^ 1], n_ptr, n_max, shift, hist);
+        src ^= 1;
+    }
+    return src;
+}
+
 int sort_kernels_per_pass() { return 2; }
 
 }  // namespace pch

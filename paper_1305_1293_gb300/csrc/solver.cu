@@ -278,8 +278,9 @@ __global__ void k_init_face_sources(Work w, const SrcDev* __restrict__ srcs, int
         SrcDev s = srcs[i];
         if (s.kind != 1) continue;
         const Inst& I = w.inst[s.inst];
+        const int face = I.finv ? I.finv[s.face] : s.face;
         for (int k = 0; k < 3; ++k) {
-            int h = 3 * s.face + k;
+            int h = 3 * face + k;
             HERec R = I.rec[h];
             // barycentric weights of h's end vertex and apex (its start vertex sits at 0)
             double b1 = s.bary[(k + 1) % 3], b2 = s.bary[(k + 2) % 3];
@@ -1786,7 +1787,7 @@ pch_status solve_instances(pch_mesh* const* meshes, int n_inst, const SrcDev* sr
         const DevMesh& dm = meshes[i]->dm;
         Inst& I = hinst[i];
         I.rec = dm.rec; I.vstart = dm.vstart; I.vlist = dm.vlist; I.vphi = dm.vphi; I.vtheta = dm.vtheta;
-        I.hang = dm.hang; I.vflag = dm.vflag; I.vrot = dm.vrot; I.vtrot = dm.vtrot;
+        I.hang = dm.hang; I.vflag = dm.vflag; I.fperm = dm.fperm; I.finv = dm.finv; I.vrot = dm.vrot; I.vtrot = dm.vtrot;
         I.g = ws->g_all + gofs[i];
         I.ang = ws->ang_all + aofs[i];
         I.stamp = ws->stamp_all + gofs[i];
@@ -1928,7 +1929,7 @@ __global__ void k_prov_pick(const ProvRec* __restrict__ log, int per, const Coun
 }
 
 // Barycentric weights over the stored corners of face(e) of the point (x, y) in e's frame.
-__device__ __forceinline__ pch_path_point face_point(const HERec& E, int e, double x, double y) {
+__device__ __forceinline__ pch_path_point face_point(const Inst& In, const HERec& E, int e, double x, double y) {
     const double b2 = y / E.yc, b1 = (x - b2 * E.xc) / E.L, b0 = 1.0 - b1 - b2;
     double b[3];
     const int i = e % 3;
@@ -1936,7 +1937,7 @@ __device__ __forceinline__ pch_path_point face_point(const HERec& E, int e, doub
     b[(i + 1) % 3] = b1;
     b[(i + 2) % 3] = b2;
     pch_path_point p;
-    p.kind = PCH_POINT_FACE; p.id = e / 3; p.t0 = b[1]; p.t1 = b[2];
+    p.kind = PCH_POINT_FACE; p.id = In.fperm ? In.fperm[e / 3] : e / 3; p.t0 = b[1]; p.t1 = b[2];
     return p;
 }
 
@@ -1963,9 +1964,9 @@ __global__ void k_trace(Inst In, const ProvRec* __restrict__ log, const int* __r
             p.kind = PCH_POINT_VERTEX; p.id = v; p.t0 = 0.0; p.t1 = 0.0;
             return p;
         };
-        auto edge_pt = [](int h, double t) {
+        auto edge_pt = [&](int h, double t) {
             pch_path_point p;
-            p.kind = PCH_POINT_EDGE; p.id = h; p.t0 = t; p.t1 = 0.0;
+            p.kind = PCH_POINT_EDGE; p.id = In.fperm ? 3 * In.fperm[h / 3] + h % 3 : h; p.t0 = t; p.t1 = 0.0;
             return p;
         };
         int v = targets[i];
@@ -1993,7 +1994,7 @@ __global__ void k_trace(Inst In, const ProvRec* __restrict__ log, const int* __r
             if (r.h < 0 || r.h >= In.nh) break;
             const HERec R = In.rec[r.h];
             if (r.kind == 2) {                   // straight to the face-point source
-                emit(face_point(R, r.h, r.px, r.py));
+                emit(face_point(In, R, r.h, r.px, r.py));
                 ok = true;
                 break;
             }
@@ -2028,7 +2029,7 @@ __global__ void k_trace(Inst In, const ProvRec* __restrict__ log, const int* __r
                 if (r.src < 0) {                 // the face-point source inside this face?
                     const double b2 = Iy / E.yc, b1 = (Ix - b2 * E.xc) / E.L;
                     if (b2 >= -1e-9 && b1 >= -1e-9 && 1.0 - b1 - b2 >= -1e-9) {
-                        emit(face_point(E, e, Ix, Iy));
+                        emit(face_point(In, E, e, Ix, Iy));
                         path_done = true;
                         break;
                     }
