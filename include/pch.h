@@ -291,7 +291,7 @@ pch_status pch_mlp_backward(const float* params_dev, const float* x_dev, const f
  * cudaMalloc, such as a host application whose own memory manager owns all device
  * memory, or a training loop that must not stall on or fail an allocation mid-run.
  * There is no counterpart in the paper.  Its scratch is one fixed device array of the
- * library (6.3 MB, held on every GPU that loads the library until exit), so n is
+ * library (2.6 MB, held on every GPU that loads the library until exit), so n is
  * limited to 4096 samples; a larger n returns PCH_ERR_CAPACITY and computes nothing.
  * The first call on a device (and the first after its CUDA context was replaced, e.g. by
  * cudaDeviceReset) looks the array up for that device; make that first call before any

@@ -2,7 +2,9 @@
 // and the FP64 peak microbenchmark.  The network and its role are described in
 // controller.cuh; none of this has a counterpart in the paper, which fixes k by hand
 // (Section 5.2).
+#include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdlib>
 #include <mutex>
 #include <vector>
@@ -81,118 +83,260 @@ int default_prop_blocks_per_sm(int block) {
 }
 
 // ---------------------------------------------------------------- training kernels
-// One block of kHidden threads per sample.  act: [n][3][kHidden] post-ReLU activations.
-__global__ void __launch_bounds__(kHidden) k_mlp_fwd(const float* __restrict__ p, const float* __restrict__ x, int n,
-                                                     float* __restrict__ y, float* __restrict__ act) {
-    __shared__ float xs[kFeatures], h0[kHidden], h1[kHidden], h2[kHidden];
-    const int t = threadIdx.x;
-    for (int b = blockIdx.x; b < n; b += gridDim.x) {
-        if (t < kFeatures) xs[t] = x[(size_t)b * kFeatures + t];
-        __syncthreads();
-        float s = p[kMlpB1 + t];
-        for (int i = 0; i < kFeatures; ++i) s = fmaf(p[kMlpW1 + t * kFeatures + i], xs[i], s);
-        h0[t] = fmaxf(s, 0.f);
-        __syncthreads();
-        s = p[kMlpB2 + t];
-        for (int i = 0; i < kHidden; ++i) s = fmaf(p[kMlpW2 + t * kHidden + i], h0[i], s);
-        h1[t] = fmaxf(s, 0.f);
-        __syncthreads();
-        s = p[kMlpB3 + t];
-        for (int i = 0; i < kHidden; ++i) s = fmaf(p[kMlpW3 + t * kHidden + i], h1[i], s);
-        h2[t] = fmaxf(s, 0.f);
-        __syncthreads();
-        if (act) {
-            act[((size_t)b * 3 + 0) * kHidden + t] = h0[t];
-            act[((size_t)b * 3 + 1) * kHidden + t] = h1[t];
-            act[((size_t)b * 3 + 2) * kHidden + t] = h2[t];
-        }
-        if (t == 0) {
-            float o = p[kMlpB4];
-            for (int i = 0; i < kHidden; ++i) o = fmaf(p[kMlpW4 + i], h2[i], o);
-            y[b] = o;
-        }
-        __syncthreads();
+// Forward, backward and weight gradients of a batch in one pass over it.
+//
+// A block takes tiles of kTile samples: the three hidden layers are 64 x 64 x 64 products
+// (FP32 FMA: the controller's arithmetic is FP32 throughout) of the weights, resident in shared
+// memory, with activations that never leave it, 4 x 4 outputs a thread; the deltas replace
+// the activations they belong to once these are used up, and each thread keeps the same
+// 41 of the 9,985 weight gradients in registers over all tiles of its block.  Every sum
+// over a layer's inputs keeps the order bias, input 0, 1, ...; the sums over samples are
+// per block, and k_mlp_reduce adds the blocks in a fixed order (deterministic).
+// What bounds it: FMA issue and the last, partly filled round of tiles (31,722 samples =
+// 3.3 tiles an SM).  Before, one 64-thread block a sample re-read all weights from L2, and
+// one thread a weight summed over all samples in turn: 31,722 samples took 2.41 ms and
+// take 97 us (with the Adam step).
+constexpr int kTile = 64;                // samples per tile
+constexpr int kTilePad = kTile + 4;      // row stride of activations [neuron][sample]
+constexpr int kMlpThreads = 256;         // 16 x 16 threads, 4 x 4 outputs each
+constexpr int kGrid = 16;
+static_assert(kHidden == 4 * kGrid && kTile == 4 * kGrid && kFeatures <= 2 * kGrid, "tile layout");
+
+struct MlpShared {
+    float x[kFeatures][kTilePad];
+    float h0[kHidden][kTilePad], h1[kHidden][kTilePad], h2[kHidden][kTilePad];
+    // [input][4 (o mod 16) + o / 16]: the four outputs of a thread (o = tx + 16 q) are adjacent
+    float w1[kFeatures][kHidden], w2[kHidden][kHidden], w3[kHidden][kHidden];
+    float b1[kHidden], b2[kHidden], b3[kHidden], w4[kHidden], dy[kTile];
+    // TRAIN only: [output][4 (i mod 16) + i / 16]
+    float t2[kHidden][kHidden], t3[kHidden][kHidden];
+};
+constexpr size_t kMlpForwardBytes = offsetof(MlpShared, t2);
+
+__device__ __forceinline__ int mlp_perm(int o) { return 4 * (o & (kGrid - 1)) + o / kGrid; }
+
+// acc[q][r] += sum over rows i in order of w[i][tx + 16 q] * in[i][4 ty + r]
+template <int K>
+__device__ __forceinline__ void mlp_product(const float (*w)[kHidden], const float (*in)[kTilePad], float acc[4][4], int tx,
+                                            int ty) {
+#pragma unroll 4
+    for (int i = 0; i < K; ++i) {
+        const float4 a = *reinterpret_cast<const float4*>(&in[i][4 * ty]);
+        const float4 v = *reinterpret_cast<const float4*>(&w[i][4 * tx]);
+        const float av[4] = {a.x, a.y, a.z, a.w}, wv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) acc[q][r] = fmaf(wv[q], av[r], acc[q][r]);
     }
 }
 
-// Per-sample back-propagation of L = 0.5 mean((y - target)^2): dlt [n][3][kHidden]
-// holds dL/dz for each hidden layer's pre-activation; dy[n] = (y - t) / n.
-__global__ void __launch_bounds__(kHidden) k_mlp_bwd(const float* __restrict__ p, const float* __restrict__ act,
-                                                     const float* __restrict__ y, const float* __restrict__ target,
-                                                     int n, float* __restrict__ dlt, float* __restrict__ dy) {
-    __shared__ float d2[kHidden], d1[kHidden];
-    const int t = threadIdx.x;
-    for (int b = blockIdx.x; b < n; b += gridDim.x) {
-        const float* a = act + (size_t)b * 3 * kHidden;
-        const float e = (y[b] - target[b]) / (float)n;
-        if (t == 0) dy[b] = e;
-        float v = a[2 * kHidden + t] > 0.f ? e * p[kMlpW4 + t] : 0.f;
-        d2[t] = v;
-        dlt[((size_t)b * 3 + 2) * kHidden + t] = v;
-        __syncthreads();
-        float s = 0.f;
-        for (int j = 0; j < kHidden; ++j) s = fmaf(p[kMlpW3 + j * kHidden + t], d2[j], s);
-        v = a[kHidden + t] > 0.f ? s : 0.f;
-        d1[t] = v;
-        dlt[((size_t)b * 3 + 1) * kHidden + t] = v;
-        __syncthreads();
-        s = 0.f;
-        for (int j = 0; j < kHidden; ++j) s = fmaf(p[kMlpW2 + j * kHidden + t], d1[j], s);
-        dlt[((size_t)b * 3 + 0) * kHidden + t] = a[t] > 0.f ? s : 0.f;
-        __syncthreads();
+// out = relu(w in + b); samples past `valid` get 0
+template <int K>
+__device__ __forceinline__ void mlp_layer(const float (*w)[kHidden], const float* b, const float (*in)[kTilePad],
+                                          float (*out)[kTilePad], int valid, int tx, int ty) {
+    float acc[4][4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[q][r] = b[tx + kGrid * q];
+    mlp_product<K>(w, in, acc, tx, ty);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        float v[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] = 4 * ty + r < valid ? fmaxf(acc[q][r], 0.f) : 0.f;
+        *reinterpret_cast<float4*>(&out[tx + kGrid * q][4 * ty]) = make_float4(v[0], v[1], v[2], v[3]);
     }
 }
 
-// One thread per parameter, sums over the samples in order: deterministic.
-__global__ void k_mlp_grad(const float* __restrict__ x, const float* __restrict__ act, const float* __restrict__ dlt,
-                           const float* __restrict__ dy, int n, float* __restrict__ grad) {
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < kMlpParams; q += gridDim.x * blockDim.x) {
-        float s = 0.f;
-        if (q < kMlpB1) {
-            int o = (q - kMlpW1) / kFeatures, i = (q - kMlpW1) % kFeatures;
-            for (int b = 0; b < n; ++b) s = fmaf(dlt[((size_t)b * 3 + 0) * kHidden + o], x[(size_t)b * kFeatures + i], s);
-        } else if (q < kMlpW2) {
-            int o = q - kMlpB1;
-            for (int b = 0; b < n; ++b) s += dlt[((size_t)b * 3 + 0) * kHidden + o];
-        } else if (q < kMlpB2) {
-            int o = (q - kMlpW2) / kHidden, i = (q - kMlpW2) % kHidden;
-            for (int b = 0; b < n; ++b)
-                s = fmaf(dlt[((size_t)b * 3 + 1) * kHidden + o], act[((size_t)b * 3 + 0) * kHidden + i], s);
-        } else if (q < kMlpW3) {
-            int o = q - kMlpB2;
-            for (int b = 0; b < n; ++b) s += dlt[((size_t)b * 3 + 1) * kHidden + o];
-        } else if (q < kMlpB3) {
-            int o = (q - kMlpW3) / kHidden, i = (q - kMlpW3) % kHidden;
-            for (int b = 0; b < n; ++b)
-                s = fmaf(dlt[((size_t)b * 3 + 2) * kHidden + o], act[((size_t)b * 3 + 1) * kHidden + i], s);
-        } else if (q < kMlpW4) {
-            int o = q - kMlpB3;
-            for (int b = 0; b < n; ++b) s += dlt[((size_t)b * 3 + 2) * kHidden + o];
-        } else if (q < kMlpB4) {
-            int i = q - kMlpW4;
-            for (int b = 0; b < n; ++b) s = fmaf(dy[b], act[((size_t)b * 3 + 2) * kHidden + i], s);
-        } else {
-            for (int b = 0; b < n; ++b) s += dy[b];
+// grad[q][p] += sum over the tile's samples of d[tx + 16 q] * in[ty + 16 p]
+template <int P>
+__device__ __forceinline__ void mlp_outer(const float (*d)[kTilePad], const float (*in)[kTilePad], float grad[4][P], int rows,
+                                          int tx, int ty) {
+#pragma unroll 2
+    for (int s = 0; s < kTile; s += 4) {
+        float4 dv[4], iv[P];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) dv[q] = *reinterpret_cast<const float4*>(&d[tx + kGrid * q][s]);
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+            iv[p] = *reinterpret_cast<const float4*>(&in[min(ty + kGrid * p, rows - 1)][s]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                float g = grad[q][p];
+                g = fmaf(dv[q].x, iv[p].x, g);
+                g = fmaf(dv[q].y, iv[p].y, g);
+                g = fmaf(dv[q].z, iv[p].z, g);
+                grad[q][p] = fmaf(dv[q].w, iv[p].w, g);
+            }
+    }
+}
+
+// TRAIN: loss L = 0.5 mean((y - target)^2); part [gridDim.x][kMlpParams] gets the blocks'
+// gradient sums, part_loss their sums of (y - target)^2.  Else y [n] gets the outputs.
+template <bool TRAIN>
+__global__ void __launch_bounds__(kMlpThreads) k_mlp_tiles(const float* __restrict__ p, const float* __restrict__ x,
+                                                           const float* __restrict__ target, int n, float* __restrict__ y,
+                                                           float* __restrict__ part, double* __restrict__ part_loss) {
+    extern __shared__ __align__(16) unsigned char mlp_smem[];
+    MlpShared& S = *reinterpret_cast<MlpShared*>(mlp_smem);
+    const int t = threadIdx.x, tx = t & (kGrid - 1), ty = t / kGrid;
+    for (int j = t; j < kHidden * kFeatures; j += kMlpThreads)
+        S.w1[j % kFeatures][mlp_perm(j / kFeatures)] = p[kMlpW1 + j];
+    for (int j = t; j < kHidden * kHidden; j += kMlpThreads) {
+        const int o = j / kHidden, i = j % kHidden;
+        const float w2 = p[kMlpW2 + j], w3 = p[kMlpW3 + j];
+        S.w2[i][mlp_perm(o)] = w2;
+        S.w3[i][mlp_perm(o)] = w3;
+        if (TRAIN) {
+            S.t2[o][mlp_perm(i)] = w2;
+            S.t3[o][mlp_perm(i)] = w3;
         }
-        grad[q] = s;
     }
-}
-
-__global__ void k_mlp_loss(const float* __restrict__ y, const float* __restrict__ target, int n, float* loss) {
-    __shared__ double sh[256];
-    double s = 0.0;
-    for (int b = threadIdx.x; b < n; b += blockDim.x) {
-        double e = (double)y[b] - (double)target[b];
-        s += e * e;
+    if (t < kHidden) {
+        S.b1[t] = p[kMlpB1 + t];
+        S.b2[t] = p[kMlpB2 + t];
+        S.b3[t] = p[kMlpB3 + t];
+        S.w4[t] = p[kMlpW4 + t];
     }
-    sh[threadIdx.x] = s;
+    const float b4 = p[kMlpB4];
+    float g3[4][4] = {}, g2[4][4] = {}, g1[4][2] = {};
+    float gv = 0.f, gb4 = 0.f;      // one of W4, b3, b2, b1 (by thread / 64); b4
+    double loss = 0.0;
+    const int tiles = (n + kTile - 1) / kTile;
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int s0 = tile * kTile, valid = min(kTile, n - s0);
+        __syncthreads();             // weights are loaded / the last tile is done
+        for (int j = t; j < kTile * kFeatures; j += kMlpThreads)
+            S.x[j % kFeatures][j / kFeatures] = j / kFeatures < valid ? x[(size_t)s0 * kFeatures + j] : 0.f;
+        __syncthreads();
+        mlp_layer<kFeatures>(S.w1, S.b1, S.x, S.h0, valid, tx, ty);
+        __syncthreads();
+        mlp_layer<kHidden>(S.w2, S.b2, S.h0, S.h1, valid, tx, ty);
+        __syncthreads();
+        mlp_layer<kHidden>(S.w3, S.b3, S.h1, S.h2, valid, tx, ty);
+        __syncthreads();
+        if (t < kTile) {
+            float o = b4;
+#pragma unroll 8
+            for (int i = 0; i < kHidden; ++i) o = fmaf(S.w4[i], S.h2[i][t], o);
+            if (TRAIN) {
+                const float want = t < valid ? target[s0 + t] : 0.f;
+                const double e = t < valid ? (double)o - (double)want : 0.0;
+                loss += e * e;
+                S.dy[t] = t < valid ? (o - want) / (float)n : 0.f;
+            } else if (t < valid) {
+                y[s0 + t] = o;
+            }
+        }
+        if (!TRAIN) continue;
+        __syncthreads();
+        const int row = t & (kHidden - 1), role = t / kHidden;
+        if (role == 0) {
+            for (int s = 0; s < kTile; ++s) gv = fmaf(S.dy[s], S.h2[row][s], gv);
+        } else if (t == kHidden) {
+            for (int s = 0; s < kTile; ++s) gb4 += S.dy[s];
+        }
+        __syncthreads();
+        // d2 = dL/dz of the last hidden layer, in place of its activations
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                float& a = S.h2[tx + kGrid * q][4 * ty + r];
+                a = a > 0.f ? S.dy[4 * ty + r] * S.w4[tx + kGrid * q] : 0.f;
+            }
+        __syncthreads();
+        auto back = [&](const float (*w)[kHidden], const float (*d)[kTilePad], float (*h)[kTilePad], float grad[4][4],
+                        int bias_role) {
+            mlp_outer<4>(d, h, grad, kHidden, tx, ty);
+            if (role == bias_role)
+                for (int s = 0; s < kTile; ++s) gv += d[row][s];
+            float acc[4][4] = {};
+            mlp_product<kHidden>(w, d, acc, tx, ty);
+            __syncthreads();         // every thread has read h
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    float& a = h[tx + kGrid * q][4 * ty + r];
+                    a = a > 0.f ? acc[q][r] : 0.f;
+                }
+            __syncthreads();
+        };
+        back(S.t3, S.h2, S.h1, g3, 1);
+        back(S.t2, S.h1, S.h0, g2, 2);
+        mlp_outer<2>(S.h0, S.x, g1, kFeatures, tx, ty);
+        if (role == 3)
+            for (int s = 0; s < kTile; ++s) gv += S.h0[row][s];
+    }
+    if (!TRAIN) return;
+    float* out = part + (size_t)blockIdx.x * kMlpParams;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int o = tx + kGrid * q;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            out[kMlpW3 + o * kHidden + ty + kGrid * r] = g3[q][r];
+            out[kMlpW2 + o * kHidden + ty + kGrid * r] = g2[q][r];
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+            if (ty + kGrid * r < kFeatures) out[kMlpW1 + o * kFeatures + ty + kGrid * r] = g1[q][r];
+    }
+    const int at[4] = {kMlpW4, kMlpB3, kMlpB2, kMlpB1};
+    out[at[t / kHidden] + (t & (kHidden - 1))] = gv;
+    if (t == kHidden) out[kMlpB4] = gb4;
+    // the block's loss: the first two warps hold it
+    __shared__ double sl[2];
+    for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+    if (t < kTile && (t & 31) == 0) sl[t / 32] = loss;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *loss = (float)(0.5 * sh[0] / n);
+    if (t == 0) part_loss[blockIdx.x] = sl[0] + sl[1];
 }
+
+// Adds the blocks' partial gradients (and losses) in a fixed order: four threads a weight,
+// each every fourth block.
+__global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ part, const double* __restrict__ part_loss,
+                                                    int blocks, int n, float* __restrict__ grad, float* __restrict__ loss) {
+    __shared__ float sh[4][64];
+    const int c = threadIdx.x & 63, seg = threadIdx.x / 64, q = blockIdx.x * 64 + c;
+    float s = 0.f;
+    if (q < kMlpParams) {
+#pragma unroll 8
+        for (int b = seg; b < blocks; b += 4) s += part[(size_t)b * kMlpParams + q];
+    }
+    sh[seg][c] = s;
+    __syncthreads();
+    if (seg == 0 && q < kMlpParams) grad[q] = (sh[0][c] + sh[1][c]) + (sh[2][c] + sh[3][c]);
+    if (blockIdx.x == 0 && threadIdx.x >= 64 && threadIdx.x < 96) {
+        double l = 0.0;
+        for (int b = threadIdx.x - 64; b < blocks; b += 32) l += part_loss[b];
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (threadIdx.x == 64) *loss = (float)(0.5 * l / n);
+    }
+}
+
+// Blocks of a training pass over n samples: one an SM at most.
+static int mlp_blocks(int n) { return std::max(1, std::min((n + kTile - 1) / kTile, sm_count())); }
+
+// Launches the pass with `scratch` for mlp_blocks(n) partial results of kMlpParams floats, the
+// losses (doubles) first.
+static cudaError_t launch_backward(const float* params, const float* x, const float* target, int n, float* grad, float* loss,
+                                   void* scratch, cudaStream_t s) {
+    const int blocks = mlp_blocks(n);
+    double* part_loss = static_cast<double*>(scratch);
+    float* part = reinterpret_cast<float*>(part_loss + blocks);
+    cudaError_t e = cudaFuncSetAttribute(k_mlp_tiles<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MlpShared));
+    if (e) return e;
+    k_mlp_tiles<true><<<blocks, kMlpThreads, sizeof(MlpShared), s>>>(params, x, target, n, nullptr, part, part_loss);
+    k_mlp_reduce<<<(kMlpParams + 63) / 64, 256, 0, s>>>(part, part_loss, blocks, n, grad, loss);
+    return cudaGetLastError();
+}
+static size_t backward_bytes(int blocks) { return (size_t)blocks * (sizeof(double) + sizeof(float) * kMlpParams); }
 
 __global__ void k_mlp_adam(float* p, const float* __restrict__ g, float* m, float* v, int t, float lr) {
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
@@ -255,7 +399,9 @@ extern "C" pch_status pch_mlp_forward(const float* params_dev, const float* x_de
     clear_error();
     if (!params_dev || !x_dev || !y_dev || n <= 0) return set_error(PCH_ERR_INVALID_ARG, "bad arguments");
     cudaStream_t s = (cudaStream_t)stream;
-    k_mlp_fwd<<<std::min(n, 65535), kHidden, 0, s>>>(params_dev, x_dev, n, y_dev, nullptr);
+    PCH_CUDA(cudaFuncSetAttribute(k_mlp_tiles<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMlpForwardBytes));
+    const int blocks = std::min((n + kTile - 1) / kTile, 2 * sm_count());
+    k_mlp_tiles<false><<<blocks, kMlpThreads, kMlpForwardBytes, s>>>(params_dev, x_dev, nullptr, n, y_dev, nullptr, nullptr);
     PCH_CUDA(cudaGetLastError());
     return PCH_OK;
 }
@@ -266,20 +412,9 @@ extern "C" pch_status pch_mlp_backward(const float* params_dev, const float* x_d
     if (!params_dev || !x_dev || !target_dev || !grad_dev || !loss_dev || n <= 0)
         return set_error(PCH_ERR_INVALID_ARG, "bad arguments");
     cudaStream_t s = (cudaStream_t)stream;
-    // scratch: activations, deltas, outputs
-    float* scratch = nullptr;
-    size_t nact = (size_t)n * 3 * kHidden;
-    PCH_CUDA(cudaMallocAsync(&scratch, sizeof(float) * (2 * nact + 2 * (size_t)n), s));
-    float* act = scratch;
-    float* dlt = act + nact;
-    float* y = dlt + nact;
-    float* dy = y + n;
-    int g = std::min(n, 65535);
-    k_mlp_fwd<<<g, kHidden, 0, s>>>(params_dev, x_dev, n, y, act);
-    k_mlp_bwd<<<g, kHidden, 0, s>>>(params_dev, act, y, target_dev, n, dlt, dy);
-    k_mlp_grad<<<(kMlpParams + 255) / 256, 256, 0, s>>>(x_dev, act, dlt, dy, n, grad_dev);
-    k_mlp_loss<<<1, 256, 0, s>>>(y, target_dev, n, loss_dev);
-    cudaError_t e = cudaGetLastError();
+    void* scratch = nullptr;
+    PCH_CUDA(cudaMallocAsync(&scratch, backward_bytes(mlp_blocks(n)), s));
+    cudaError_t e = launch_backward(params_dev, x_dev, target_dev, n, grad_dev, loss_dev, scratch, s);
     cudaFreeAsync(scratch, s);
     PCH_CUDA(e);
     return PCH_OK;
@@ -321,14 +456,13 @@ extern "C" pch_status pch_measure_fp64_peak(double* tflops) {
 
 // ---------------------------------------------------------------- allocation-free backward
 // Scratch of pch_mlp_backward_noalloc, in a file-scope device array instead of a
-// cudaMallocAsync buffer: per-sample activations and deltas (3 x 64 floats each), the
-// outputs and their errors, for at most kNoAllocMaxSamples samples (6.3 MB).  Every
-// GPU that loads the library holds this array until the process exits.
+// stream-ordered allocation: the partial results of the blocks of at most
+// kNoAllocMaxSamples samples (2.6 MB).  Every GPU that loads the library holds this array
+// until the process exits.
 namespace pch {
 constexpr int kNoAllocMaxSamples = 4096;
-constexpr size_t kNoAllocActFloats = (size_t)kNoAllocMaxSamples * 3 * kHidden;
-constexpr size_t kNoAllocFloats = 2 * kNoAllocActFloats + 2 * (size_t)kNoAllocMaxSamples;
-static __device__ __align__(256) float g_noalloc_scratch[kNoAllocFloats];
+constexpr size_t kNoAllocBlocks = (kNoAllocMaxSamples + kTile - 1) / kTile;
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBlocks * (sizeof(double) + sizeof(float) * kMlpParams)];
 // Host side: the array's device address, resolved once per device and context (a reset
 // device gets a new context, and the array a new address).  The symbol itself is only a
 // host-side stand-in and must never be handed to a kernel.
@@ -347,7 +481,7 @@ extern "C" pch_status pch_mlp_backward_noalloc(const float* params_dev, const fl
     int dev = 0;
     PCH_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kMaxDevices) return set_error(PCH_ERR_INVALID_ARG, "device id %d out of range", dev);
-    float* scratch = nullptr;
+    void* scratch = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_noalloc_mu);
         DevPtrSlot& sl = g_noalloc_slot[dev];
@@ -362,22 +496,13 @@ extern "C" pch_status pch_mlp_backward_noalloc(const float* params_dev, const fl
             if (e != cudaSuccess || p == nullptr)
                 return set_error(PCH_ERR_CUDA, "cudaGetSymbolAddress of the scratch array failed: %s",
                                  cudaGetErrorString(e));
-            scratch = static_cast<float*>(p);
-            sl.ptr = scratch;
+            scratch = p;
+            sl.ptr = static_cast<float*>(p);
             sl.ctx = current_context_id();
         }
     }
     cudaStream_t s = (cudaStream_t)stream;
-    float* act = scratch;
-    float* dlt = act + kNoAllocActFloats;
-    float* y = dlt + kNoAllocActFloats;
-    float* dy = y + kNoAllocMaxSamples;
-    // every scratch element read below is written first by the same call: nothing to clear
-    int g = std::min(n, 65535);
-    k_mlp_fwd<<<g, kHidden, 0, s>>>(params_dev, x_dev, n, y, act);
-    k_mlp_bwd<<<g, kHidden, 0, s>>>(params_dev, act, y, target_dev, n, dlt, dy);
-    k_mlp_grad<<<(kMlpParams + 255) / 256, 256, 0, s>>>(x_dev, act, dlt, dy, n, grad_dev);
-    k_mlp_loss<<<1, 256, 0, s>>>(y, target_dev, n, loss_dev);
-    PCH_CUDA(cudaGetLastError());
+    // every scratch element read is written first by the same call: nothing to clear
+    PCH_CUDA(launch_backward(params_dev, x_dev, target_dev, n, grad_dev, loss_dev, scratch, s));
     return PCH_OK;
 }
