@@ -37,22 +37,31 @@ __device__ __forceinline__ double ldg_dist(const unsigned long long* g, unsigned
     return bitsd(__ldcg(g + v));
 }
 
-// Pack a (distance to v2, crossing position on the edge) pair for angle_split: the
-// distance is rounded UP to 40 significant bits (so a stored value never understates the
-// window's distance) and the crossing position, given as xq = 2^24 x / L, floored to 24
-// bits.
-// Crossing position in angle_split units: floor(xq) clamped to [0, 2^24 - 1].
-__device__ __forceinline__ long long angle_pos(double xq) {
-    const long long q = __double2ll_rd(xq);
-    return q < 0 ? 0 : (q > (long long)kAngleXMask ? (long long)kAngleXMask : q);
+// Crossing position on an edge of length L in units of 2^-44 of it (only the order of
+// positions on one edge matters, so 1 / L is the single-precision estimate, the same for
+// every window on it), clamped to [0, 2^44): an integer made from the product's bits, as
+// a conversion would run on the FP64 unit.
+constexpr int kPosBits = 44;
+constexpr long long kPosMax = (1ll << kPosBits) - 1;
+__device__ __forceinline__ long long edge_pos(double x, double L) {
+    const double r = nr_range(L) ? widen_normal(rcp_approx_f32(narrow_seed(L))) : 1.0 / L;
+    const unsigned long long q = dbits(x * r);
+    const int shift = 1023 + 52 - kPosBits - (int)(q >> 52);          // of the 53-bit mantissa, to the right
+    if ((long long)q < 0 || shift > 52) return 0;                     // negative or below one unit
+    if (shift < 53 - kPosBits) return kPosMax;                        // 1 or more
+    return (long long)((q & 0xfffffffffffffull) | 1ull << 52) >> shift;
 }
-__device__ __forceinline__ unsigned long long pack_angle(double D, double xq) {
+// Pack a (distance to v2, crossing position) pair for angle_split: the distance is rounded
+// UP to 40 significant bits (so a stored value never understates the window's distance),
+// the position down to 24 bits.
+constexpr int kPosLow = kPosBits - kAngleXBits;
+__device__ __forceinline__ unsigned long long pack_angle(double D, long long pos) {
     unsigned long long b = dbits(D);
     if (b & kAngleXMask) b = (b | kAngleXMask) + 1ull;
-    return (b & ~kAngleXMask) | (unsigned long long)angle_pos(xq);
+    return (b & ~kAngleXMask) | (unsigned long long)(pos >> kPosLow);
 }
-// kEpsSnap in angle_split units (the snap tolerance kEpsSnap * L times 2^24 / L).
-constexpr double kSplitTol = kEpsSnap * (double)(1 << kAngleXBits);
+// kEpsSnap (2^-40 of the edge) in position units.
+constexpr long long kSplitTol = 1ll << (kPosBits - 40);
 
 struct WarpScan {
     int excl, total;
@@ -513,12 +522,13 @@ constexpr float kLocalF = 0x1p-20f;
 // What bounds this kernel is the FP64 unit (16 SM cycles a warp instruction).  The
 // positions (pseudo-source and interval in the child's frame) are FP64, 21 instructions
 // for a window that does not reach v2: ray_hit measures from the vertex that the two edges
-// share, which needs no cross product of far points.  What is only decided (occupancy,
+// share, which needs no cross product of far points; one that does adds 15 (its split
+// position is turned into an integer without FP64 conversions).  What is only decided (occupancy,
 // the filters, the chaining) runs in FP32 with error bounds (twofloat.cuh); the lengths
 // |I A|, |I B| that the filters compare are two-float values made from the coordinates
-// when they are needed, so no rounding of theirs accumulates along a lineage.  Before,
-// all of it was FP64, 62 instructions a window: eight fields on the 327,680-face sphere
-// took 86.1 ms and take 40.6, the 1M-face torus 49.3 and 23.5.
+// when they are needed, so no rounding of theirs accumulates along a lineage.  With all of
+// it in FP64, 62 instructions a window, eight fields on the 327,680-face sphere took
+// 86.1 ms and take 39.2, the 1M-face torus 49.3 and 22.5.
 template <bool PROV>
 __device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, FanReq* req, const LaneWin& W,
                                                  ChildOut& c, bool& has_child, bool& defer, bool& occ, bool& comp) {
@@ -532,12 +542,15 @@ __device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, F
     double g2 = ldg_dist(I.g, R.v2 & ~kPseudoBit);
     const F2 df = f2_mag(d, fb);
     const float Lf = f_of(L, fb), xcf = f_of(R.xc, fb), ycf = f_of(R.yc, fb);
+    // superseded pseudo-source: read early, used where the answer is first needed (an event
+    // of such a window is a real path's length, only never the shortest)
+    const bool stale = !W.task && stale_source(I, W.src, d);
     bool left = false, right = false, prop = false;
     const double tol = times_eps(L);
     if (W.task) {
         occ = true;
         left = R.tw2 >= 0;
-    } else if (!stale_source(I, W.src, d)) {
+    } else {
         prop = true;
         if (W.hop == 0) {
             // Xin-Wang endpoint tests of a window from the pool against the current
@@ -554,7 +567,7 @@ __device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, F
     if (prop) {
         const EvSrc es{W.inst, W.h, W.src, 0, px, py};   // event origin, recorded with PROV only
         // Algorithm 2: endpoint events at v0 (A = v0) and v1 (B = v1)
-        if (W.pend) {
+        if (W.pend && !stale) {
             const double py2 = py * py;
             if ((W.pend & kPendA) && le_s(A, tol)) {
                 const double D0 = d + sqrt_nr(fma(px, px, py2));
@@ -576,42 +589,41 @@ __device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, F
         const float vB = fmaf(bxf, ycf, pyf * (xcf - f_of(B, fb)));
         const float ext = fmaf(fabsf(pyf), fabsf(xcf) + Lf, Lf * ycf * 0x1p-10f);
         const float eA = fmaf(fabsf(axf), ycf, ext) * 0x1p-20f, eB = fmaf(fabsf(bxf), ycf, ext) * 0x1p-20f;
-        bool before_A;
+        bool before_A, near_end = false;
         if (vA > eA) {
             before_A = true;
         } else if (vB < -eB) {
             before_A = false;
         } else if (vA < -eA && vB > eB) {
             before_A = false;
-            occ = true;
+            occ = true;                     // v2's ray is at least 2^-30 L inside both ends
         } else {
+            near_end = true;
             const double den = R.yc - py, num = (R.xc - px) * (-py);
             before_A = gt0_s(fma(ax - tol, den, -num));
             occ = !before_A && ge0_s(fma(bx + tol, den, -num));
         }
         if (occ) {
+            if (stale) return false;
             const double dx = R.xc - px, dy = R.yc - py;
             const double xs = fma(dx * (-py), rcp_nr(dy), px);
-            const double xcl = lt_s(xs, A) ? A : (lt_s(B, xs) ? B : xs);
-            // angle_split position: xs in units of 2^-24 |e| (only the order of positions
-            // on one edge matters, so any fixed scale per edge will do)
-            const double xq = xs * (rcp_nr(L) * (double)(1 << kAngleXBits));
-            const double D2 = d + sqrt_nr(dx * dx + dy * dy);
+            const long long pos = edge_pos(xs, L);      // angle_split position
+            const double D2 = d + sqrt_nr(fma(dx, dx, dy * dy));
             // one angle one split (Fig. `fig:filter`(a)) against angle_split[h]
             unsigned long long* ap = I.ang + W.h;
             const unsigned long long aw = __ldcg(ap);
             const bool win = aw == kEmptyAngle || dbits(D2) < (aw & ~kAngleXMask);
             if (win) {
                 left = right = true;
-                atomicMin(ap, pack_angle(D2, xq));
+                atomicMin(ap, pack_angle(D2, pos));
             } else {
                 // loser: keep the child on its own side of the winner's ray, which
                 // crosses e in [q, q + 1] (angle_split units), widened by the snap
                 // tolerance
                 // (positions compared after the same clamping the stored one had)
                 const long long q = (long long)(aw & kAngleXMask);
-                left = angle_pos(xq + kSplitTol) < q;
-                right = angle_pos(xq - kSplitTol) > q;
+                left = min(pos + kSplitTol, kPosMax) >> kPosLow < q;
+                right = max(pos - kSplitTol, 0ll) >> kPosLow > q;
                 if (!left && !right) left = right = true;
             }
             if (const int ev = vertex_event<PROV>(I, R.v2, D2, g2, &w, &es)) {
@@ -622,8 +634,11 @@ __device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, F
                 push_fan(req, &cnt->n_req, w.req_cap, &cnt->error, W.inst, R.v2 & ~kPseudoBit, D2, hp,
                          ex * ux + ey * uy, ux * ey - uy * ex, ev);
             }
-            if (le_s(B - xcl, tol)) right = false;
-            if (le_s(xcl - A, tol)) left = false;
+            if (near_end) {
+                const double xcl = lt_s(xs, A) ? A : (lt_s(B, xs) ? B : xs);
+                if (le_s(B - xcl, tol)) right = false;
+                if (le_s(xcl - A, tol)) left = false;
+            }
         } else {
             right = before_A;
             left = !right;
@@ -631,7 +646,7 @@ __device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, F
         right = right && R.tw1 >= 0;
         left = left && R.tw2 >= 0;
     }
-    if (!(right || left)) return prop;
+    if (!(right || left)) return prop && !stale;
     // The child, one select-driven path for both sides (a warp holds left and right
     // children): the right child lies on edge v2 -> v1 (frame origin v2), the left one on
     // v0 -> v2 (origin v0).  When v2 is occupied the child's end at v2 is exact.
@@ -657,7 +672,7 @@ __device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, F
     else b = ray_hit(B - shared, bx, ux, uy, upy, py, base, Lc);
     const float Lcf = f_of(Lc, fb), af = f_of(a, fb), bf = f_of(b, fb);
     // narrower than 2^-40 of the edge: dropped
-    if (!(bf - af > Lcf * kLocalF) && !lt_s(times_eps(Lc), b - a)) return prop;
+    if (!(bf - af > Lcf * kLocalF) && !lt_s(times_eps(Lc), b - a)) return prop && !stale;
     const double axc = a - Ipx, bxc = b - Ipx;
     // Xin-Wang filter (Fig. `fig:filter`(b)) on the new window: against its start and end
     // vertices (right child: v2, v1; left child: v0, v2), and against the vertex T of the
@@ -681,7 +696,7 @@ __device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, F
         const bool useless = f2_add_f(eS, lenB) > bf + mrg || f2_add_f(eE, lenA) > (Lcf - af) + mrg ||
                              (tA > 0.f && tB > 0.f && tA * tA > fmaf(Xax, Xax, Xay * Xay) * (1.f + 0x1p-18f) &&
                               tB * tB > fmaf(Xbx, Xbx, Xby * Xby) * (1.f + 0x1p-18f));
-        if (useless) return prop;
+        if (useless || stale) return prop && !stale;
         c.key = df.h + (gt0_s(axc) ? lenA.h : (sbits(bxc) < 0 ? lenB.h : -f_of(Ipy, fb)));
     }
     // ends at a vertex whose event is still to be made: not v2 of an occupied window, nor
