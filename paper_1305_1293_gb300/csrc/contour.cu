@@ -33,32 +33,84 @@ __device__ __forceinline__ void face_dist(const int* __restrict__ tri, const dou
     for (int i = 0; i < 3; ++i) d[i] = dist[tri[3 * f + i]];
 }
 
-__global__ void k_contour_count(const int* __restrict__ tri, int nf, const double* __restrict__ dist,
-                                const double* __restrict__ levels, int n_levels, int* count,
-                                unsigned long long* total) {
+// Both kernels give block b the faces [b C, (b + 1) C), C = ceil(nf / gridDim.x), 256 at a
+// time.  Bound by memory: 12 bytes of vertex ids and three distance gathers (L2) a face,
+// 32 bytes a segment.
+__device__ __forceinline__ int crossed_levels(const int* __restrict__ tri, const double* __restrict__ dist,
+                                              const double* __restrict__ levels, int n_levels, int f, double d[3]) {
+    face_dist(tri, dist, f, d);
+    int c = 0;
+    for (int l = 0; l < n_levels; ++l) c += face_mask(d, levels[l]) != 0;
+    return c;
+}
+
+// Segments of every block's faces, and of all.
+__global__ void __launch_bounds__(256) k_contour_count(const int* __restrict__ tri, int nf, const double* __restrict__ dist,
+                                                       const double* __restrict__ levels, int n_levels,
+                                                       unsigned long long* __restrict__ block_count,
+                                                       unsigned long long* total) {
+    const long long C = ((long long)nf + gridDim.x - 1) / gridDim.x;
+    const int f0 = (int)min((long long)nf, C * blockIdx.x), f1 = (int)min((long long)nf, C * (blockIdx.x + 1));
     unsigned long long t = 0;
-    for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += gridDim.x * blockDim.x) {
+    for (int f = f0 + threadIdx.x; f < f1; f += blockDim.x) {
         double d[3];
-        face_dist(tri, dist, f, d);
-        int c = 0;
-        for (int l = 0; l < n_levels; ++l) c += face_mask(d, levels[l]) != 0;
-        count[f] = c;
-        t += (unsigned long long)c;
+        t += (unsigned long long)crossed_levels(tri, dist, levels, n_levels, f, d);
     }
-    if (t) atomicAdd(total, t);
+    __shared__ unsigned long long sh[8];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x / 32] = t;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int q = 1; q < 8; ++q) t += sh[q];
+        block_count[blockIdx.x] = t;
+        if (t) atomicAdd(total, t);
+    }
 }
 
 // Segment endpoints: from the crossing on the edge whose start corner is inside to the
 // crossing on the edge whose start corner is outside, so that the inside (distance
 // below L) lies to the left of the segment seen from the face's front side (corners
 // counter-clockwise).
-__global__ void k_contour_write(const int* __restrict__ tri, int nf, const double* __restrict__ dist,
-                                const double* __restrict__ levels, int n_levels, const int* __restrict__ offset,
-                                long long capacity, pch_contour_segment* __restrict__ out) {
-    for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += gridDim.x * blockDim.x) {
-        double d[3];
-        face_dist(tri, dist, f, d);
-        long long o = offset[f];
+//
+// A block adds up the counts of the blocks before it and scans its own faces, so that no
+// array of per-face offsets is written and scanned between the two kernels.
+__global__ void __launch_bounds__(256) k_contour_write(const int* __restrict__ tri, int nf, const double* __restrict__ dist,
+                                                       const double* __restrict__ levels, int n_levels,
+                                                       const unsigned long long* __restrict__ block_count,
+                                                       long long capacity, pch_contour_segment* __restrict__ out) {
+    const long long C = ((long long)nf + gridDim.x - 1) / gridDim.x;
+    const int f0 = (int)min((long long)nf, C * blockIdx.x), f1 = (int)min((long long)nf, C * (blockIdx.x + 1));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x / 32;
+    __shared__ unsigned long long sh[8];
+    __shared__ int wsum[8];
+    unsigned long long before = 0;
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += blockDim.x) before += block_count[b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    if (lane == 0) sh[warp] = before;
+    __syncthreads();
+    long long base = 0;
+    for (int q = 0; q < 8; ++q) base += (long long)sh[q];
+    for (int tile = f0; tile < f1 && base < capacity; tile += blockDim.x) {
+        const int f = tile + threadIdx.x;
+        double d[3] = {0.0, 0.0, 0.0};
+        const int c = f < f1 ? crossed_levels(tri, dist, levels, n_levels, f, d) : 0;
+        int incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        long long o = base + incl - c;
+        for (int q = 0; q < 8; ++q) {
+            if (q < warp) o += wsum[q];
+            base += wsum[q];
+        }
+        __syncthreads();
+        if (c == 0) continue;
         for (int l = 0; l < n_levels; ++l) {
             const double L = levels[l];
             const int m = face_mask(d, L);
@@ -99,46 +151,64 @@ extern "C" pch_status pch_iso_contours(const pch_mesh* m, const double* dist, in
     for (int l = 0; l < n_levels; ++l)
         if (!std::isfinite(levels[l])) return set_error(PCH_ERR_INVALID_ARG, "level %d is not finite", l);
     const int nf = m->dm.nf, nv = m->dm.nv;
-    double *ddist = nullptr, *dlev = nullptr;
-    int *cnt = nullptr, *off = nullptr, *tmp = nullptr;
-    unsigned long long* dtotal = nullptr;
-    pch_contour_segment* dseg = nullptr;
-    const size_t ntmp = scan_tmp_ints(nf);
-    cudaStream_t s = 0;
+    // one temporary: levels, block counts, total, the distances (host fields) and, when the
+    // bound on their number is small, the segments; else these are allocated once counted
+    struct {
+        double *dist, *lev;
+        unsigned long long *count, *total;
+        pch_contour_segment* seg;
+    } t{};
+    const cudaStream_t s = 0;
+    const int grid = sm_count() * 8;
+    const long long most = std::min<long long>(capacity, (long long)nf * n_levels);
+    const bool at_once = most <= (64ll << 20) / (long long)sizeof(pch_contour_segment);
+    auto carve = [&](Carver& c) {
+        c.take(&t.lev, n_levels);
+        c.take(&t.count, grid);
+        c.take(&t.total, 1);
+        if (!dist_on_device) c.take(&t.dist, nv);
+        if (at_once) c.take(&t.seg, most);
+    };
+    Carver c;
+    carve(c);
+    void *tmp = nullptr, *seg_tmp = nullptr;
     unsigned long long total = 0;
     pch_status st = PCH_OK;
-    cudaError_t e = cudaSuccess;
-    if (!dist_on_device) {
-        e = cudaMalloc(&ddist, sizeof(double) * (size_t)nv);
-        if (!e) e = cudaMemcpy(ddist, dist, sizeof(double) * (size_t)nv, cudaMemcpyHostToDevice);
-    }
-    if (!e) e = cudaMalloc(&dlev, sizeof(double) * (size_t)n_levels);
-    if (!e) e = cudaMemcpy(dlev, levels, sizeof(double) * (size_t)n_levels, cudaMemcpyHostToDevice);
-    if (!e) e = cudaMalloc(&cnt, sizeof(int) * (size_t)nf);
-    if (!e) e = cudaMalloc(&off, sizeof(int) * (size_t)nf);
-    if (!e) e = cudaMalloc(&tmp, sizeof(int) * std::max<size_t>(ntmp, 1));
-    if (!e) e = cudaMalloc(&dtotal, sizeof(unsigned long long));
-    if (!e) e = cudaMemset(dtotal, 0, sizeof(unsigned long long));
-    const double* dd = dist_on_device ? dist : ddist;
-    const int grid = sm_count() * 4;
+    cudaError_t e = tmp_alloc(&tmp, c.off, s);
     if (!e) {
-        k_contour_count<<<grid, 256, 0, s>>>(m->dm.tri, nf, dd, dlev, n_levels, cnt, dtotal);
-        e = cudaGetLastError();
+        c = Carver{static_cast<char*>(tmp), 0};
+        carve(c);
+        e = cudaMemcpyAsync(t.lev, levels, sizeof(double) * (size_t)n_levels, cudaMemcpyHostToDevice, s);
+        if (!e && !dist_on_device) e = cudaMemcpyAsync(t.dist, dist, sizeof(double) * (size_t)nv, cudaMemcpyHostToDevice, s);
+        if (!e) e = cudaMemsetAsync(t.total, 0, sizeof(unsigned long long), s);
     }
-    if (!e) e = cudaMemcpy(&total, dtotal, sizeof(unsigned long long), cudaMemcpyDeviceToHost);
+    const double* dd = dist_on_device ? dist : t.dist;
+    auto write = [&](long long room, pch_contour_segment* seg) {
+        k_contour_write<<<grid, 256, 0, s>>>(m->dm.tri, nf, dd, t.lev, n_levels, t.count, room, seg);
+        return cudaGetLastError();
+    };
+    if (!e) {
+        k_contour_count<<<grid, 256, 0, s>>>(m->dm.tri, nf, dd, t.lev, n_levels, t.count, t.total);
+        e = cudaGetLastError();
+        if (!e && at_once && most > 0) e = write(most, t.seg);
+    }
+    if (!e) e = cudaMemcpyAsync(&total, t.total, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
+    if (!e) e = cudaStreamSynchronize(s);
     if (!e && total > (unsigned long long)INT_MAX) {
         st = set_error(PCH_ERR_CAPACITY, "%llu contour segments exceed 2^31 - 1", total);
     } else if (!e) {
         const long long keep = std::min<long long>(capacity, (long long)total);
-        e = exclusive_scan(cnt, off, nf, tmp, s);
-        if (!e && keep > 0) e = cudaMalloc(&dseg, sizeof(pch_contour_segment) * (size_t)keep);
-        if (!e && keep > 0) {
-            k_contour_write<<<grid, 256, 0, s>>>(m->dm.tri, nf, dd, dlev, n_levels, off, keep, dseg);
-            e = cudaGetLastError();
+        if (!at_once && keep > 0) {
+            e = tmp_alloc(&seg_tmp, sizeof(pch_contour_segment) * (size_t)keep, s);
+            t.seg = static_cast<pch_contour_segment*>(seg_tmp);
+            if (!e) e = write(keep, t.seg);
         }
-        if (!e && keep > 0) e = cudaMemcpy(segments, dseg, sizeof(pch_contour_segment) * (size_t)keep, cudaMemcpyDeviceToHost);
+        if (!e && keep > 0)
+            e = cudaMemcpyAsync(segments, t.seg, sizeof(pch_contour_segment) * (size_t)keep, cudaMemcpyDeviceToHost, s);
+        if (!e) e = cudaStreamSynchronize(s);
     }
-    cudaFree(ddist); cudaFree(dlev); cudaFree(cnt); cudaFree(off); cudaFree(tmp); cudaFree(dtotal); cudaFree(dseg);
+    if (tmp) cudaFreeAsync(tmp, s);
+    if (seg_tmp) cudaFreeAsync(seg_tmp, s);
     if (e) return set_error(e == cudaErrorMemoryAllocation ? PCH_ERR_OOM : PCH_ERR_CUDA, "iso-contours: %s",
                             cudaGetErrorString(e));
     if (st != PCH_OK) return st;

@@ -413,7 +413,7 @@ extern "C" pch_status pch_mlp_backward(const float* params_dev, const float* x_d
         return set_error(PCH_ERR_INVALID_ARG, "bad arguments");
     cudaStream_t s = (cudaStream_t)stream;
     void* scratch = nullptr;
-    PCH_CUDA(cudaMallocAsync(&scratch, backward_bytes(mlp_blocks(n)), s));
+    PCH_CUDA(tmp_alloc(&scratch, backward_bytes(mlp_blocks(n)), s));
     cudaError_t e = launch_backward(params_dev, x_dev, target_dev, n, grad_dev, loss_dev, scratch, s);
     cudaFreeAsync(scratch, s);
     PCH_CUDA(e);

@@ -2,7 +2,7 @@
 // per-half-edge unfolding frames, one-ring order, total angles and the saddle /
 // boundary classification of Section 3.  Entry points pch_create_mesh, pch_mesh_info,
 // pch_destroy, pch_last_error.
-#include <cmath>
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -63,6 +63,82 @@ unsigned long long current_context_id() {
     if (get_current(&ctx) != 0 || !ctx) return 0;
     unsigned long long id = 0;
     return get_id(ctx, &id) == 0 ? id : 0;
+}
+
+// ---------------------------------------------------------------- device memory
+struct PoolSlot {
+    unsigned long long ctx = 0;       // current_context_id() when the pool was made; 0 = empty
+    cudaMemPool_t pool = nullptr;
+    cudaStream_t stream = nullptr;    // orders the allocations of blocks that any stream uses
+};
+constexpr int kMaxPoolDevices = 64;
+static PoolSlot g_pool_slot[kMaxPoolDevices];
+static std::mutex g_pool_mu;
+
+// The current device's pool in its current context (a pool of an earlier, destroyed
+// context is gone with it).
+static cudaError_t current_pool(PoolSlot* out) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e) return e;
+    if (dev < 0 || dev >= kMaxPoolDevices) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    PoolSlot& sl = g_pool_slot[dev];
+    unsigned long long ctx = current_context_id();
+    if (ctx == 0) {                   // make the device's primary context current
+        if ((e = cudaFree(nullptr))) return e;
+        ctx = current_context_id();
+    }
+    if (sl.ctx != ctx || ctx == 0) {
+        PoolSlot fresh;
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        if ((e = cudaMemPoolCreate(&fresh.pool, &props))) return e;
+        unsigned long long keep = kPoolKeep;
+        e = cudaMemPoolSetAttribute(fresh.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (!e) e = cudaStreamCreateWithFlags(&fresh.stream, cudaStreamNonBlocking);
+        if (e) {
+            cudaMemPoolDestroy(fresh.pool);
+            return e;
+        }
+        fresh.ctx = ctx;
+        sl = fresh;
+    }
+    *out = sl;
+    return cudaSuccess;
+}
+
+cudaError_t dev_alloc(DevMem& m, size_t bytes) {
+    m.bytes = bytes ? bytes : 1;
+    m.pooled = m.bytes <= kPoolKeep / 2;
+    cudaError_t e = cudaSuccess;
+    if (m.pooled) {
+        PoolSlot ps;
+        e = current_pool(&ps);
+        if (!e) e = cudaMallocFromPoolAsync(&m.p, m.bytes, ps.pool, ps.stream);
+        if (!e) e = cudaStreamSynchronize(ps.stream);
+    } else {
+        e = cudaMalloc(&m.p, m.bytes);
+    }
+    if (e) m = DevMem{};
+    return e;
+}
+
+void dev_free(DevMem& m) {
+    if (m.p) {
+        PoolSlot ps;
+        if (m.pooled && current_pool(&ps) == cudaSuccess) cudaFreeAsync(m.p, ps.stream);
+        else cudaFree(m.p);
+    }
+    m = DevMem{};
+}
+
+cudaError_t tmp_alloc(void** p, size_t bytes, cudaStream_t s) {
+    PoolSlot ps;
+    const cudaError_t e = current_pool(&ps);
+    return e ? e : cudaMallocFromPoolAsync(p, bytes ? bytes : 1, ps.pool, s);
 }
 
 // ---------------------------------------------------------------- exclusive scan
@@ -329,9 +405,10 @@ __global__ void k_morton(int nf, const double* __restrict__ xyz, const int* __re
 }
 
 __global__ void k_permute_faces(int nf, const int* __restrict__ tri, const int* __restrict__ perm, int* tri_out,
-                                int* finv) {
+                                int* fperm, int* finv) {
     for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += gridDim.x * blockDim.x) {
         const int o = perm[f];
+        fperm[f] = o;
         finv[o] = f;
         for (int c = 0; c < 3; ++c) tri_out[3 * f + c] = tri[3 * o + c];
     }
@@ -381,11 +458,67 @@ __global__ void __launch_bounds__(256) k_stats_final(const double* part_l, const
     if (threadIdx.x == 0) { *out_lsum = s; out_counts[0] = nb; out_counts[1] = np; }
 }
 
-static void free_mesh(DevMesh& d) {
-    cudaFree(d.rec); cudaFree(d.vstart); cudaFree(d.vlist); cudaFree(d.hang);
-    cudaFree(d.tri); cudaFree(d.fperm); cudaFree(d.finv);
-    cudaFree(d.vtheta); cudaFree(d.vphi); cudaFree(d.vflag); cudaFree(d.vrot); cudaFree(d.vtrot);
-    d = DevMesh{};
+// Lays out the arrays of a mesh.
+static void carve_mesh(Carver& c, DevMesh& d, bool reorder) {
+    c.take(&d.rec, d.nh);
+    c.take(&d.vrot, d.nh);
+    c.take(&d.vtrot, d.nv);
+    c.take(&d.tri, d.nh);
+    c.take(&d.vlist, d.nh);
+    c.take(&d.hang, d.nh);
+    c.take(&d.vphi, d.nh);
+    c.take(&d.vstart, d.nv + 1);
+    c.take(&d.vtheta, d.nv);
+    c.take(&d.vflag, d.nv);
+    if (reorder) {
+        c.take(&d.fperm, d.nf);
+        c.take(&d.finv, d.nf);
+    }
+}
+
+// Temporaries of the mesh preparation.
+struct MeshTmp {
+    double *xyz, *hang64, *lsum;
+    unsigned long long* hkeys;
+    long long* box;
+    int *twin, *vcount, *vout, *hvals, *counts, *scan_tmp, *tri_sorted, *fval[2], *fhist;
+    unsigned* fkey[2];
+    int* err;               // kMeshErr* flags
+    unsigned long long* bad; // first non-finite coordinate, first vertex id out of range
+};
+static void carve_tmp(Carver& c, MeshTmp& t, int nv, int nf, unsigned long long cap, bool reorder, int sort_blocks) {
+    const int nh = 3 * nf;
+    c.take(&t.xyz, 3 * (size_t)nv);
+    c.take(&t.hang64, nh);
+    c.take(&t.lsum, 1 + kStatBlocks);
+    c.take(&t.hkeys, cap);
+    c.take(&t.hvals, cap);
+    c.take(&t.twin, nh);
+    c.take(&t.vcount, nv + 1);
+    c.take(&t.vout, nv);
+    c.take(&t.counts, 2 + 2 * kStatBlocks);
+    c.take(&t.scan_tmp, scan_tmp_ints(nv + 1));
+    c.take(&t.err, 1);
+    c.take(&t.bad, 2);
+    if (reorder) {
+        c.take(&t.tri_sorted, nh);
+        for (int j = 0; j < 2; ++j) {
+            c.take(&t.fkey[j], nf);
+            c.take(&t.fval[j], nf);
+        }
+        c.take(&t.fhist, kRsDigits * sort_blocks + 1);
+        c.take(&t.box, 6);
+    }
+}
+
+// First coordinate that is not finite and first vertex id out of range (~0: none).
+__global__ void k_check(int nv, int nf, const double* __restrict__ xyz, const int* __restrict__ tri,
+                        unsigned long long* bad) {
+    const long long n = max(3ll * nv, 3ll * nf);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        if (i < 3ll * nv && !(fabs(xyz[i]) <= 1.7976931348623157e308)) atomicMin(bad, (unsigned long long)i);
+        if (i < 3ll * nf && (unsigned)tri[i] >= (unsigned)nv) atomicMin(bad + 1, (unsigned long long)i);
+    }
 }
 
 void destroy_workspace(Workspace* w);   // solver.cu
@@ -402,28 +535,21 @@ extern "C" pch_status pch_create_mesh(const double* vertices, int32_t n_vertices
     if (!vertices || !faces || !out) return set_error(PCH_ERR_INVALID_ARG, "null pointer argument");
     if (n_vertices < 3 || n_faces < 1) return set_error(PCH_ERR_INVALID_ARG, "need >= 3 vertices and >= 1 face");
     if ((long long)n_faces * 3 >= (1LL << 31) - 1) return set_error(PCH_ERR_CAPACITY, "too many faces");
-    for (long long i = 0; i < 3LL * n_vertices; ++i)
-        if (!std::isfinite(vertices[i])) return set_error(PCH_ERR_INVALID_ARG, "non-finite coordinate at vertex %lld", i / 3);
-    for (long long i = 0; i < 3LL * n_faces; ++i)
-        if (faces[i] < 0 || faces[i] >= n_vertices)
-            return set_error(PCH_ERR_INVALID_ARG, "face %lld references vertex %d out of range", i / 3, faces[i]);
 
     const int nv = n_vertices, nf = n_faces, nh = 3 * n_faces;
-    DevMesh d{};
-    d.nv = nv; d.nf = nf; d.nh = nh;
-    double* xyz = nullptr;
-    int *tri = nullptr, *tri_sorted = nullptr, *fval[2] = {nullptr, nullptr}, *fhist = nullptr, *twin = nullptr, *vcount = nullptr, *vout = nullptr, *err = nullptr, *scan_tmp = nullptr,
-        *hvals = nullptr, *counts = nullptr;
-    unsigned long long* hkeys = nullptr;
-    double* lsum = nullptr;
-    double* hang64 = nullptr;
-    unsigned* fkey[2] = {nullptr, nullptr};
-    long long* box = nullptr;
+    const bool reorder = nf >= kReorderFaces;
     const int sort_blocks = 2 * sm_count();
+    const cudaStream_t s = 0;         // the legacy default stream, as the callers' copies
     unsigned long long cap = 1;
     while (cap < 2ull * (unsigned long long)nh) cap <<= 1;
+    DevMesh d{};
+    d.nv = nv; d.nf = nf; d.nh = nh;
+    DevMem mem;
+    MeshTmp t{};
+    void* tmp = nullptr;
     pch_status st = PCH_OK;
     int herr = 0;
+    unsigned long long hbad[2] = {~0ull, ~0ull};
     double hl = 0.0;
     int hc[2] = {0, 0};
     auto fail = [&](pch_status s) { st = s; };
@@ -437,71 +563,64 @@ extern "C" pch_status pch_create_mesh(const double* vertices, int32_t n_vertices
         }                                                                                       \
     } while (0)
     {
-        MCHK(cudaMalloc(&xyz, sizeof(double) * 3 * nv));
-        MCHK(cudaMalloc(&d.tri, sizeof(int) * nh));
-        MCHK(cudaMalloc(&d.rec, sizeof(HERec) * nh));
-        MCHK(cudaMalloc(&hang64, sizeof(double) * nh));
-        MCHK(cudaMalloc(&d.hang, sizeof(float) * nh));
-        MCHK(cudaMalloc(&d.vphi, sizeof(float) * nh));
-        MCHK(cudaMalloc(&d.vlist, sizeof(int) * nh));
-        MCHK(cudaMalloc(&d.vstart, sizeof(int) * (nv + 1)));
-        MCHK(cudaMalloc(&d.vtheta, sizeof(float) * nv));
-        MCHK(cudaMalloc(&d.vrot, sizeof(double2) * nh));
-        MCHK(cudaMalloc(&d.vtrot, sizeof(double2) * nv));
-        MCHK(cudaMalloc(&d.vflag, nv));
-        MCHK(cudaMalloc(&twin, sizeof(int) * nh));
-        MCHK(cudaMalloc(&vcount, sizeof(int) * (nv + 1)));
-        MCHK(cudaMalloc(&vout, sizeof(int) * nv));
-        MCHK(cudaMalloc(&err, sizeof(int)));
-        MCHK(cudaMalloc(&counts, sizeof(int) * (2 + 2 * kStatBlocks)));
-        MCHK(cudaMalloc(&lsum, sizeof(double) * (1 + kStatBlocks)));
-        MCHK(cudaMalloc(&scan_tmp, sizeof(int) * scan_tmp_ints(nv + 1)));
-        MCHK(cudaMalloc(&hkeys, sizeof(unsigned long long) * cap));
-        MCHK(cudaMalloc(&hvals, sizeof(int) * cap));
-        MCHK(cudaMemcpy(xyz, vertices, sizeof(double) * 3 * nv, cudaMemcpyHostToDevice));
-        MCHK(cudaMemcpy(d.tri, faces, sizeof(int) * nh, cudaMemcpyHostToDevice));
-        tri = d.tri;
-        MCHK(cudaMemset(err, 0, sizeof(int)));
-        MCHK(cudaMemset(vcount, 0, sizeof(int) * (nv + 1)));
-        MCHK(cudaMemset(vout, 0x7f, sizeof(int) * nv));
-        MCHK(cudaMemset(hkeys, 0xff, sizeof(unsigned long long) * cap));
+        Carver cm, ct;
+        carve_mesh(cm, d, reorder);
+        MCHK(dev_alloc(mem, cm.off));
+        cm = Carver{static_cast<char*>(mem.p), 0};
+        carve_mesh(cm, d, reorder);
+        carve_tmp(ct, t, nv, nf, cap, reorder, sort_blocks);
+        MCHK(tmp_alloc(&tmp, ct.off, s));
+        ct = Carver{static_cast<char*>(tmp), 0};
+        carve_tmp(ct, t, nv, nf, cap, reorder, sort_blocks);
+        MCHK(cudaMemcpyAsync(t.xyz, vertices, sizeof(double) * 3 * nv, cudaMemcpyHostToDevice, s));
+        MCHK(cudaMemcpyAsync(d.tri, faces, sizeof(int) * nh, cudaMemcpyHostToDevice, s));
+        MCHK(cudaMemsetAsync(t.bad, 0xff, sizeof(unsigned long long) * 2, s));
+        MCHK(cudaMemsetAsync(t.err, 0, sizeof(int), s));
+        MCHK(cudaMemsetAsync(t.vcount, 0, sizeof(int) * (nv + 1), s));
+        MCHK(cudaMemsetAsync(t.vout, 0x7f, sizeof(int) * nv, s));
+        MCHK(cudaMemsetAsync(t.hkeys, 0xff, sizeof(unsigned long long) * cap, s));
         const int tb = 256;
         const int gb = std::max(1, std::min((nh + tb - 1) / tb, sm_count() * 8));
         const int gv = std::max(1, std::min((nv + tb - 1) / tb, sm_count() * 8));
-        if (nf >= kReorderFaces) {
-            MCHK(cudaMalloc(&tri_sorted, sizeof(int) * nh));
-            MCHK(cudaMalloc(&d.finv, sizeof(int) * nf));
-            for (int j = 0; j < 2; ++j) {
-                MCHK(cudaMalloc(&fkey[j], sizeof(unsigned) * nf));
-                MCHK(cudaMalloc(&fval[j], sizeof(int) * nf));
-            }
-            MCHK(cudaMalloc(&fhist, sizeof(int) * (kRsDigits * sort_blocks + 1)));
-            MCHK(cudaMalloc(&box, sizeof(long long) * 6));
-            MCHK(cudaMemset(box, 0x7f, sizeof(long long) * 6));
-            MCHK(cudaMemcpy(fhist + kRsDigits * sort_blocks, &nf, sizeof(int), cudaMemcpyHostToDevice));
-            k_bounds<<<gv, tb>>>(nv, xyz, box);
-            k_morton<<<gb, tb>>>(nf, xyz, tri, box, fkey[0]);
-            const int r = launch_sort_keys(fhist + kRsDigits * sort_blocks, nf, kMortonBits, fkey, fval, fhist, sort_blocks, 0);
-            d.fperm = fval[r];
-            fval[r] = nullptr;
-            k_permute_faces<<<gb, tb>>>(nf, tri, d.fperm, tri_sorted, d.finv);
-            MCHK(cudaGetLastError());
-            tri = tri_sorted;
+        k_check<<<std::max(gb, gv), tb, 0, s>>>(nv, nf, t.xyz, d.tri, t.bad);
+        MCHK(cudaMemcpyAsync(hbad, t.bad, sizeof hbad, cudaMemcpyDeviceToHost, s));
+        MCHK(cudaStreamSynchronize(s));
+        if (hbad[0] != ~0ull) {
+            fail(set_error(PCH_ERR_INVALID_ARG, "non-finite coordinate at vertex %lld", (long long)hbad[0] / 3));
+            goto cleanup;
         }
-        k_frames<<<gb, tb>>>(nh, xyz, tri, d.rec, hang64, err);
-        k_hash_insert<<<gb, tb>>>(nh, tri, hkeys, hvals, cap - 1, err);
-        k_twins<<<gb, tb>>>(nh, tri, hkeys, hvals, cap - 1, twin, vcount, vout);
+        if (hbad[1] != ~0ull) {
+            fail(set_error(PCH_ERR_INVALID_ARG, "face %lld references vertex %d out of range", (long long)hbad[1] / 3,
+                           faces[hbad[1]]));
+            goto cleanup;
+        }
+        const int* tri = d.tri;
+        if (reorder) {
+            MCHK(cudaMemsetAsync(t.box, 0x7f, sizeof(long long) * 6, s));
+            MCHK(cudaMemcpyAsync(t.fhist + kRsDigits * sort_blocks, &nf, sizeof(int), cudaMemcpyHostToDevice, s));
+            k_bounds<<<gv, tb, 0, s>>>(nv, t.xyz, t.box);
+            k_morton<<<gb, tb, 0, s>>>(nf, t.xyz, tri, t.box, t.fkey[0]);
+            const int r = launch_sort_keys(t.fhist + kRsDigits * sort_blocks, nf, kMortonBits, t.fkey, t.fval, t.fhist,
+                                           sort_blocks, s);
+            k_permute_faces<<<gb, tb, 0, s>>>(nf, tri, t.fval[r], t.tri_sorted, d.fperm, d.finv);
+            MCHK(cudaGetLastError());
+            tri = t.tri_sorted;
+        }
+        k_frames<<<gb, tb, 0, s>>>(nh, t.xyz, tri, d.rec, t.hang64, t.err);
+        k_hash_insert<<<gb, tb, 0, s>>>(nh, tri, t.hkeys, t.hvals, cap - 1, t.err);
+        k_twins<<<gb, tb, 0, s>>>(nh, tri, t.hkeys, t.hvals, cap - 1, t.twin, t.vcount, t.vout);
         MCHK(cudaGetLastError());
-        MCHK(exclusive_scan(vcount, d.vstart, nv + 1, scan_tmp, 0));
-        k_rings<<<gv, tb>>>(nv, twin, vout, d.vstart, hang64, d.vlist, d.vphi, d.vtheta, d.hang, d.vrot, d.vtrot,
-                            d.vflag, err);
-        k_rec_ids<<<gb, tb>>>(nh, twin, d.vflag, d.rec);
-        k_stats<<<kStatBlocks, 256>>>(nh, nv, d.rec, twin, d.vflag, lsum + 1, counts + 2);
-        k_stats_final<<<1, kStatBlocks>>>(lsum + 1, counts + 2, lsum, counts);
+        MCHK(exclusive_scan(t.vcount, d.vstart, nv + 1, t.scan_tmp, s));
+        k_rings<<<gv, tb, 0, s>>>(nv, t.twin, t.vout, d.vstart, t.hang64, d.vlist, d.vphi, d.vtheta, d.hang, d.vrot, d.vtrot,
+                                  d.vflag, t.err);
+        k_rec_ids<<<gb, tb, 0, s>>>(nh, t.twin, d.vflag, d.rec);
+        k_stats<<<kStatBlocks, 256, 0, s>>>(nh, nv, d.rec, t.twin, d.vflag, t.lsum + 1, t.counts + 2);
+        k_stats_final<<<1, kStatBlocks, 0, s>>>(t.lsum + 1, t.counts + 2, t.lsum, t.counts);
         MCHK(cudaGetLastError());
-        MCHK(cudaMemcpy(&herr, err, sizeof(int), cudaMemcpyDeviceToHost));
-        MCHK(cudaMemcpy(&hl, lsum, sizeof(double), cudaMemcpyDeviceToHost));
-        MCHK(cudaMemcpy(hc, counts, sizeof(int) * 2, cudaMemcpyDeviceToHost));
+        MCHK(cudaMemcpyAsync(&herr, t.err, sizeof(int), cudaMemcpyDeviceToHost, s));
+        MCHK(cudaMemcpyAsync(&hl, t.lsum, sizeof(double), cudaMemcpyDeviceToHost, s));
+        MCHK(cudaMemcpyAsync(hc, t.counts, sizeof(int) * 2, cudaMemcpyDeviceToHost, s));
+        MCHK(cudaStreamSynchronize(s));
         if (herr & kMeshErrDup) { fail(set_error(PCH_ERR_NONMANIFOLD, "an oriented edge appears in two faces (non-manifold or inconsistent orientation)")); goto cleanup; }
         if (herr & kMeshErrDegenerate) { fail(set_error(PCH_ERR_DEGENERATE, "a face has a repeated vertex or (near) zero area")); goto cleanup; }
         if (herr & kMeshErrFan) { fail(set_error(PCH_ERR_NONMANIFOLD, "a vertex whose faces do not form a single fan")); goto cleanup; }
@@ -509,6 +628,7 @@ extern "C" pch_status pch_create_mesh(const double* vertices, int32_t n_vertices
         d.lbar = hl / nh;
         pch_mesh* m = new pch_mesh();
         m->dm = d;
+        m->mem = mem;
         cudaGetDevice(&m->device);
         m->n_boundary_he = hc[0];
         m->n_pseudo = hc[1];
@@ -517,11 +637,9 @@ extern "C" pch_status pch_create_mesh(const double* vertices, int32_t n_vertices
     }
 cleanup:
 #undef MCHK
-    cudaFree(xyz); cudaFree(tri_sorted); cudaFree(twin); cudaFree(box); cudaFree(fhist);
-    for (int j = 0; j < 2; ++j) { cudaFree(fkey[j]); cudaFree(fval[j]); }
-    cudaFree(vcount); cudaFree(vout); cudaFree(err);
-    cudaFree(scan_tmp); cudaFree(hkeys); cudaFree(hvals); cudaFree(counts); cudaFree(lsum); cudaFree(hang64);
-    if (st != PCH_OK) free_mesh(d);
+    if (st != PCH_OK) cudaStreamSynchronize(s);   // nothing is in flight on what is freed below
+    if (tmp) cudaFreeAsync(tmp, s);
+    if (st != PCH_OK) dev_free(mem);
     return st;
 }
 
@@ -540,8 +658,9 @@ extern "C" void pch_destroy(pch_mesh* m) {
     int cur = 0;
     cudaGetDevice(&cur);
     cudaSetDevice(m->device);
+    cudaDeviceSynchronize();          // work of asynchronous calls may still use the memory
     if (m->ws) destroy_workspace(m->ws);
-    free_mesh(m->dm);
+    dev_free(m->mem);
     cudaSetDevice(cur);
     delete m;
 }

@@ -18,8 +18,50 @@ struct Workspace;   // solver.cu
 
 }  // namespace pch
 
+namespace pch {
+
+// ---- device memory -------------------------------------------------------------------
+// The library's own stream-ordered pool, one per device and context (safe for several
+// threads and streams, as the driver's pools are): up to kPoolKeep bytes of freed memory
+// stay with it for the next mesh, workspace or temporary, the rest goes back to the
+// driver at the next synchronisation.  (cudaMalloc / cudaFree of a mesh and its workspace
+// took 4 ms a mesh, and temporaries of the default pool, which keeps nothing, were mapped
+// anew after every synchronising call.)
+constexpr unsigned long long kPoolKeep = 512ull << 20;
+
+// A block of memory that any stream may use once dev_alloc returns.  Blocks above half of
+// kPoolKeep come from cudaMalloc.
+struct DevMem {
+    void* p = nullptr;
+    size_t bytes = 0;
+    bool pooled = false;
+};
+cudaError_t dev_alloc(DevMem& m, size_t bytes);
+// The caller has made sure that no work on the device uses the block any more (cudaFree, for
+// the large ones, waits for the device itself).
+void dev_free(DevMem& m);
+
+// Stream-ordered temporaries; released with cudaFreeAsync.
+cudaError_t tmp_alloc(void** p, size_t bytes, cudaStream_t s);
+
+// Lays arrays out in one block: a first pass over the take() calls with base = nullptr
+// gives the size.
+struct Carver {
+    char* base = nullptr;
+    size_t off = 0;
+    template <class T>
+    void take(T** p, size_t n) {
+        off = (off + 255) & ~(size_t)255;
+        *p = base ? reinterpret_cast<T*>(base + off) : nullptr;
+        off += sizeof(T) * n;
+    }
+};
+
+}  // namespace pch
+
 struct pch_mesh {
     pch::DevMesh dm;
+    pch::DevMem mem;        // every array of dm
     int device;
     int n_boundary_he;
     int n_pseudo;

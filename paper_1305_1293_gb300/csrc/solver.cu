@@ -257,10 +257,21 @@ __device__ __forceinline__ bool stale_source(const Inst& I, int src, double d) {
 }
 
 // ====================================================================== init
-__global__ void k_fill_inf(unsigned long long* g, long long n) {
-    const unsigned long long inf = 0x7FF0000000000000ull;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        g[i] = inf;
+// The state of a solve before its sources: every distance +inf, no angle_split, no fan
+// (stamp 0, direction NaN), empty histograms and counters.
+__global__ void __launch_bounds__(256) k_reset(Work w, unsigned long long* g, long long n_g, unsigned long long* ang,
+                                               long long n_ang, unsigned* stamp, float* fan_phi) {
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    for (long long i = t; i < n_ang; i += step) ang[i] = kEmptyAngle;
+    for (long long i = t; i < n_g; i += step) {
+        g[i] = 0x7FF0000000000000ull;
+        stamp[i] = 0u;
+        fan_phi[i] = __uint_as_float(0xffffffffu);
+    }
+    for (long long i = t; i < (long long)w.n_inst * kBins; i += step) w.hist[0][i] = w.hist[1][i] = 0u;
+    static_assert(sizeof(Counters) % 4 == 0, "cleared by words");
+    if (t < (long long)(sizeof(Counters) / 4)) reinterpret_cast<int*>(w.cnt)[t] = 0;
+    if (t == 0 && w.trace_rows) *w.trace_rows = 0;
 }
 
 // Algorithm 1, initialisation: geod_dist = 0 at the sources; a window on every edge
@@ -275,18 +286,10 @@ __global__ void k_init_sources(Work w, const SrcDev* __restrict__ srcs, int n_sr
             I.g[s.vertex] = 0ull;
             // the source's fan covers every direction
             push_fan(w.req[0], &cnt->n_req, w.req_cap, &cnt->error, s.inst, (unsigned)s.vertex, 0.0, -1, 0.0, 0.0);
+            continue;
         }
-    }
-}
-
-// Face-point sources (one thread each, after k_init_sources): corner distances and the
-// three windows, written to the child arena of iteration 0.
-__global__ void k_init_face_sources(Work w, const SrcDev* __restrict__ srcs, int n_src) {
-    Counters* cnt = w.cnt;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_src; i += gridDim.x * blockDim.x) {
-        SrcDev s = srcs[i];
-        if (s.kind != 1) continue;
-        const Inst& I = w.inst[s.inst];
+        // a point inside a face: corner distances and three windows, to the child arena of
+        // iteration 0
         const int face = I.finv ? I.finv[s.face] : s.face;
         for (int k = 0; k < 3; ++k) {
             int h = 3 * face + k;
@@ -1284,23 +1287,6 @@ __global__ void k_min_into(const unsigned long long* __restrict__ g, unsigned lo
 }
 
 // ====================================================================== host side
-struct Alloc {
-    std::vector<void*> ptrs;
-    size_t bytes = 0;
-    template <class T>
-    cudaError_t get(T** p, size_t n) {
-        if (n == 0) n = 1;
-        cudaError_t e = cudaMalloc((void**)p, sizeof(T) * n);
-        if (e == cudaSuccess) { ptrs.push_back(*p); bytes += sizeof(T) * n; }
-        return e;
-    }
-    void release() {
-        for (void* p : ptrs) cudaFree(p);
-        ptrs.clear();
-        bytes = 0;
-    }
-};
-
 struct GraphKey {
     SolveCfg cfg;
     Work w;
@@ -1308,18 +1294,21 @@ struct GraphKey {
 
 struct Workspace {
     int device = 0;
-    Alloc pools;            // pools, arena, sort buffers, requests (sized by caps)
-    Alloc inst_mem;         // g / angle_split / stamps (sized by the instances)
-    Alloc fixed;            // counters, tables
-    Alloc sthr;             // strided-selection thresholds (PCH_CONTROL_STRIDED)
+    DevMem pools;           // pools, arena, sort buffers, requests (sized by caps)
+    DevMem inst_mem;        // g / angle_split / stamps, counters, tables (sized by the instances)
+    DevMem trace_mem;       // controller traces
+    DevMem sthr;            // strided-selection thresholds (PCH_CONTROL_STRIDED)
     int sthr_cap = 0;
-    Alloc plog_mem;         // distance-event records (geodesic paths)
+    DevMem plog_mem;        // distance-event records (geodesic paths)
     int plog_cap = 0;
     ProvRec* plog = nullptr;
     Work w{};
     int pool_cap = 0, sel_cap = 0, arena_cap = 0, req_cap = 0;
     long long g_cap = 0, ang_cap = 0, st_cap = 0;
-    int inst_cap = 0;
+    int inst_cap = 0, src_cap = 0;
+    size_t setup_cap = 0;             // bytes of the set-up block: instances, controls, sources
+    char* setup = nullptr;            // device
+    char* setup_host = nullptr;       // pinned
     unsigned long long* g_all = nullptr;
     unsigned long long* ang_all = nullptr;
     unsigned* stamp_all = nullptr;
@@ -1341,12 +1330,13 @@ void destroy_workspace(Workspace* ws) {
     if (!ws) return;
     if (ws->exec) cudaGraphExecDestroy(ws->exec);
     if (ws->graph) cudaGraphDestroy(ws->graph);
-    ws->pools.release();
-    ws->inst_mem.release();
-    ws->fixed.release();
-    ws->sthr.release();
-    ws->plog_mem.release();
+    dev_free(ws->pools);
+    dev_free(ws->inst_mem);
+    dev_free(ws->trace_mem);
+    dev_free(ws->sthr);
+    dev_free(ws->plog_mem);
     if (ws->cnt_host) cudaFreeHost(ws->cnt_host);
+    if (ws->setup_host) cudaFreeHost(ws->setup_host);
     for (auto& e : ws->ev) if (e) cudaEventDestroy(e);
     delete ws;
 }
@@ -1359,17 +1349,28 @@ static void drop_graph(Workspace* ws) {
 }
 
 // `keyed`: the pending pools; the work list and the arena hold no keys.
-static cudaError_t alloc_soa(Alloc& a, WinSoA& s, int cap, bool keyed) {
-    cudaError_t e;
-    if ((e = a.get(&s.he, cap))) return e;
-    if ((e = a.get(&s.inst, cap))) return e;
-    if ((e = a.get(&s.d, cap))) return e;
-    if ((e = a.get(&s.A, cap))) return e;
-    if ((e = a.get(&s.B, cap))) return e;
-    if ((e = a.get(&s.px, cap))) return e;
-    if ((e = a.get(&s.py, cap))) return e;
-    if (keyed && (e = a.get(&s.key, cap))) return e;
-    return a.get(&s.src, cap);
+static void carve_soa(Carver& c, WinSoA& s, size_t cap, bool keyed) {
+    c.take(&s.d, cap);
+    c.take(&s.A, cap);
+    c.take(&s.B, cap);
+    c.take(&s.px, cap);
+    c.take(&s.py, cap);
+    if (keyed) c.take(&s.key, cap);
+    c.take(&s.he, cap);
+    c.take(&s.inst, cap);
+    c.take(&s.src, cap);
+}
+static void carve_pools(Carver& c, Work& w, int pool_cap, int sel_cap, int arena_cap, int req_cap, int sort_blocks) {
+    carve_soa(c, w.pool[0], pool_cap, true);
+    carve_soa(c, w.pool[1], pool_cap, true);
+    carve_soa(c, w.sel, sel_cap, false);
+    carve_soa(c, w.arena, arena_cap, false);
+    for (int j = 0; j < 2; ++j) {
+        c.take(&w.req[j], req_cap);
+        c.take(&w.sort_key[j], arena_cap);
+        c.take(&w.sort_val[j], arena_cap);
+    }
+    c.take(&w.sort_hist, (size_t)kRsDigits * sort_blocks);
 }
 
 // Capacities: the work list holds sel_cap windows (more selected windows simply stay
@@ -1388,29 +1389,20 @@ static pch_status ensure_pools(Workspace* ws, int sel_cap, int pool_cap, int req
     sel_cap = std::max(sel_cap, ws->sel_cap);
     pool_cap = std::max(pool_cap, ws->pool_cap);
     arena_cap = arena_for(sel_cap);
-    const int req_cap = std::max({4 * sel_cap + (1 << 20), req_min, ws->req_cap});
+    const int req_cap = std::max({4 * sel_cap + (1 << 18), req_min, ws->req_cap});
     const int sort_blocks = 2 * sm_count();
     drop_graph(ws);
     Work& w = ws->w;
     Work nw = w;
-    Alloc fresh;
-    cudaError_t e = cudaSuccess;
-    if (!e) e = alloc_soa(fresh, nw.pool[0], pool_cap, true);
-    if (!e) e = alloc_soa(fresh, nw.pool[1], pool_cap, true);
-    if (!e) e = alloc_soa(fresh, nw.sel, sel_cap, false);
-    if (!e) e = alloc_soa(fresh, nw.arena, arena_cap, false);
-    if (!e) e = fresh.get(&nw.req[0], req_cap);
-    if (!e) e = fresh.get(&nw.req[1], req_cap);
-    if (!e) e = fresh.get(&nw.sort_key[0], arena_cap);
-    if (!e) e = fresh.get(&nw.sort_key[1], arena_cap);
-    if (!e) e = fresh.get(&nw.sort_val[0], arena_cap);
-    if (!e) e = fresh.get(&nw.sort_val[1], arena_cap);
-    if (!e) e = fresh.get(&nw.sort_hist, (size_t)kRsDigits * sort_blocks);
-    if (e) {
-        fresh.release();
+    DevMem fresh;
+    Carver c;
+    carve_pools(c, nw, pool_cap, sel_cap, arena_cap, req_cap, sort_blocks);
+    cudaError_t e = dev_alloc(fresh, c.off);
+    if (e)
         return set_error(e == cudaErrorMemoryAllocation ? PCH_ERR_OOM : PCH_ERR_CUDA, "workspace allocation: %s",
                          cudaGetErrorString(e));
-    }
+    c = Carver{static_cast<char*>(fresh.p), 0};
+    carve_pools(c, nw, pool_cap, sel_cap, arena_cap, req_cap, sort_blocks);
     if (ws->pool_cap > 0) {
         // growth between iterations: keep the pending pools and the fan requests
         const size_t n = (size_t)ws->pool_cap;
@@ -1427,9 +1419,9 @@ static pch_status ensure_pools(Workspace* ws, int sel_cap, int pool_cap, int req
             cudaMemcpy(nw.req[p], w.req[p], sizeof(FanReq) * (size_t)ws->req_cap, cudaMemcpyDeviceToDevice);
         }
         e = cudaDeviceSynchronize();
-        if (e) { fresh.release(); return set_error(PCH_ERR_CUDA, "pool growth copy: %s", cudaGetErrorString(e)); }
+        if (e) { dev_free(fresh); return set_error(PCH_ERR_CUDA, "pool growth copy: %s", cudaGetErrorString(e)); }
     }
-    ws->pools.release();
+    dev_free(ws->pools);
     ws->pools = fresh;
     w = nw;
     ws->pool_cap = w.pool_cap = pool_cap;
@@ -1456,42 +1448,56 @@ static pch_status ensure_workspace(pch_mesh* owner, Workspace** out) {
         }
         cudaEventCreate(&ws->ev[0]);
         cudaEventCreate(&ws->ev[1]);
-        if (ws->fixed.get(&ws->w.cnt, 1) != cudaSuccess) {
-            destroy_workspace(ws);
-            return set_error(PCH_ERR_OOM, "counter allocation failed");
-        }
         owner->ws = ws;
     }
     *out = owner->ws;
     return PCH_OK;
 }
 
-static pch_status ensure_instances(Workspace* ws, int n_inst, long long g_total, long long a_total) {
-    if (n_inst <= ws->inst_cap && g_total <= ws->g_cap && a_total <= ws->ang_cap) return PCH_OK;
-    drop_graph(ws);
-    ws->inst_mem.release();
-    Work& w = ws->w;
-    int ic = std::max(n_inst, ws->inst_cap);
-    long long gc = std::max(g_total, ws->g_cap), ac = std::max(a_total, ws->ang_cap);
-    cudaError_t e = cudaSuccess;
-    if (!e) e = ws->inst_mem.get(&ws->g_all, gc);
-    if (!e) e = ws->inst_mem.get(&ws->ang_all, ac);
-    if (!e) e = ws->inst_mem.get(&ws->stamp_all, gc);
-    if (!e) e = ws->inst_mem.get(&ws->fanphi_all, gc);
-    if (!e) e = ws->inst_mem.get(&ws->fandir_all, gc);
-    if (!e) e = ws->inst_mem.get(&w.inst, ic);
-    if (!e) e = ws->inst_mem.get(&w.ctl, ic);
-    if (!e) e = ws->inst_mem.get(&w.hist[0], (size_t)ic * kBins);
-    if (!e) e = ws->inst_mem.get(&w.hist[1], (size_t)ic * kBins);
-    if (e) {
-        ws->inst_mem.release();
-        ws->inst_cap = 0; ws->g_cap = ws->ang_cap = 0;
-        return set_error(e == cudaErrorMemoryAllocation ? PCH_ERR_OOM : PCH_ERR_CUDA, "instance allocation: %s",
-                         cudaGetErrorString(e));
+static size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
+// The set-up block, one copy from pinned memory: Inst[n_inst], InstCtl[n_inst], SrcDev[n_src].
+static size_t setup_bytes(int n_inst, int n_src) {
+    return align_up(sizeof(Inst) * n_inst) + align_up(sizeof(InstCtl) * n_inst) + sizeof(SrcDev) * (size_t)n_src;
+}
+
+static pch_status ensure_instances(Workspace* ws, int n_inst, long long g_total, long long a_total, int n_src) {
+    if (n_inst > ws->inst_cap || n_src > ws->src_cap || g_total > ws->g_cap || a_total > ws->ang_cap) {
+        drop_graph(ws);
+        PCH_CUDA(cudaDeviceSynchronize());
+        dev_free(ws->inst_mem);
+        Work& w = ws->w;
+        const int ic = std::max(n_inst, ws->inst_cap), sc = std::max(n_src, std::max(ws->src_cap, 64));
+        const long long gc = std::max(g_total, ws->g_cap), ac = std::max(a_total, ws->ang_cap);
+        ws->inst_cap = ws->src_cap = 0;
+        ws->g_cap = ws->ang_cap = 0;
+        if (ws->setup_host) cudaFreeHost(ws->setup_host);
+        ws->setup_host = nullptr;
+        ws->setup_cap = setup_bytes(ic, sc);
+        cudaError_t e = cudaMallocHost(&ws->setup_host, ws->setup_cap);
+        for (int pass = 0; pass < 2 && !e; ++pass) {
+            Carver c;
+            c.base = static_cast<char*>(ws->inst_mem.p);
+            c.take(&ws->g_all, gc);
+            c.take(&ws->ang_all, ac);
+            c.take(&ws->fandir_all, gc);
+            c.take(&ws->stamp_all, gc);
+            c.take(&ws->fanphi_all, gc);
+            c.take(&w.hist[0], (size_t)ic * kBins);
+            c.take(&w.hist[1], (size_t)ic * kBins);
+            c.take(&w.cnt, 1);
+            c.take(&ws->setup, ws->setup_cap);
+            if (pass == 0) e = dev_alloc(ws->inst_mem, c.off);
+        }
+        if (e) {
+            dev_free(ws->inst_mem);
+            return set_error(e == cudaErrorMemoryAllocation ? PCH_ERR_OOM : PCH_ERR_CUDA, "instance allocation: %s",
+                             cudaGetErrorString(e));
+        }
+        ws->inst_cap = ic;
+        ws->src_cap = sc;
+        ws->g_cap = gc;
+        ws->ang_cap = ac;
     }
-    ws->inst_cap = ic;
-    ws->g_cap = gc;
-    ws->ang_cap = ac;
     return PCH_OK;
 }
 
@@ -1635,6 +1641,7 @@ static pch_status run_solve(Workspace* ws, cudaStream_t s, const SolveCfg& cfg_i
                 ws->gkey = key;
             }
             PCH_CUDA(cudaGraphLaunch(ws->exec, s));
+            PCH_CUDA(cudaEventRecord(ws->ev[1], s));
             PCH_CUDA(cudaMemcpyAsync(ws->cnt_host, w.cnt, sizeof(Counters), cudaMemcpyDeviceToHost, s));
             PCH_CUDA(cudaStreamSynchronize(s));
             const Counters& c = *ws->cnt_host;
@@ -1650,8 +1657,10 @@ static pch_status run_solve(Workspace* ws, cudaStream_t s, const SolveCfg& cfg_i
         const long long it = ws->cnt_host->iter;
         launches += ((it + cfg.unroll - 1) / cfg.unroll) * cfg.unroll * kernels_per_iteration(cfg);
     }
-    PCH_CUDA(cudaEventRecord(ws->ev[1], s));
-    PCH_CUDA(cudaEventSynchronize(ws->ev[1]));
+    if (cfg.loop == PCH_LOOP_HOST || cfg.profile) {
+        PCH_CUDA(cudaEventRecord(ws->ev[1], s));
+        PCH_CUDA(cudaEventSynchronize(ws->ev[1]));
+    }
     const Counters& c = *ws->cnt_host;
     if (c.error) return status_from_error(c.error);
     if (stats) {
@@ -1662,7 +1671,7 @@ static pch_status run_solve(Workspace* ws, cudaStream_t s, const SolveCfg& cfg_i
         stats->windows_propagated = (int64_t)c.propagated;
         stats->peak_pending = (int64_t)c.peak_pending;
         stats->ms_total = ms;
-        stats->bytes_workspace = (int64_t)(ws->pools.bytes + ws->inst_mem.bytes + ws->fixed.bytes + ws->sthr.bytes);
+        stats->bytes_workspace = (int64_t)(ws->pools.bytes + ws->inst_mem.bytes + ws->trace_mem.bytes + ws->sthr.bytes);
         stats->kernel_launches += launches;
         stats->fans = (int64_t)c.fans;
         stats->fan_windows = (int64_t)c.fan_windows;
@@ -1741,14 +1750,13 @@ static pch_status ensure_plog(Workspace* ws, long long cap) {
     cap = std::min<long long>(cap, 1LL << 30);
     if (cap <= ws->plog_cap) return PCH_OK;
     drop_graph(ws);
-    ws->plog_mem.release();
+    PCH_CUDA(cudaDeviceSynchronize());
+    dev_free(ws->plog_mem);
     ws->plog_cap = 0;
     ws->plog = nullptr;
-    if (ws->plog_mem.get(&ws->plog, (size_t)cap) != cudaSuccess) {
-        ws->plog_mem.release();
-        ws->plog = nullptr;
+    if (dev_alloc(ws->plog_mem, sizeof(ProvRec) * (size_t)cap) != cudaSuccess)
         return set_error(PCH_ERR_OOM, "distance-event records: allocation of %lld failed", cap);
-    }
+    ws->plog = static_cast<ProvRec*>(ws->plog_mem.p);
     ws->plog_cap = (int)cap;
     return PCH_OK;
 }
@@ -1785,8 +1793,6 @@ pch_status solve_instances(pch_mesh* const* meshes, int n_inst, const SrcDev* sr
     pch_status st = ensure_workspace(meshes[0], &ws);
     if (st != PCH_OK) return st;
     // instance layout
-    std::vector<Inst> hinst(n_inst);
-    std::vector<InstCtl> hctl(n_inst);
     long long goff = 0, aoff = 0, kbase = 0;
     std::vector<long long> gofs(n_inst), aofs(n_inst);
     for (int i = 0; i < n_inst; ++i) {
@@ -1795,8 +1801,15 @@ pch_status solve_instances(pch_mesh* const* meshes, int n_inst, const SrcDev* sr
         goff += meshes[i]->dm.nv;
         aoff += meshes[i]->dm.nh;
     }
-    st = ensure_instances(ws, n_inst, goff, aoff);
+    st = ensure_instances(ws, n_inst, goff, aoff, n_src);
     if (st != PCH_OK) return st;
+    const size_t ctl_at = align_up(sizeof(Inst) * n_inst), src_at = ctl_at + align_up(sizeof(InstCtl) * n_inst);
+    Inst* hinst = reinterpret_cast<Inst*>(ws->setup_host);
+    InstCtl* hctl = reinterpret_cast<InstCtl*>(ws->setup_host + ctl_at);
+    std::memcpy(ws->setup_host + src_at, srcs, sizeof(SrcDev) * n_src);
+    ws->w.inst = reinterpret_cast<Inst*>(ws->setup);
+    ws->w.ctl = reinterpret_cast<InstCtl*>(ws->setup + ctl_at);
+    const SrcDev* dsrc = reinterpret_cast<const SrcDev*>(ws->setup + src_at);
     SolveCfg cfg = make_cfg(opt, n_inst, aoff);
     for (int i = 0; i < n_inst; ++i) {
         const DevMesh& dm = meshes[i]->dm;
@@ -1835,12 +1848,16 @@ pch_status solve_instances(pch_mesh* const* meshes, int n_inst, const SrcDev* sr
     w.n_inst = n_inst;
     if (cfg.stride_T > ws->sthr_cap) {
         drop_graph(ws);
-        ws->sthr.release();
+        PCH_CUDA(cudaDeviceSynchronize());
+        dev_free(ws->sthr);
         ws->sthr_cap = 0;
-        if (ws->sthr.get(&w.sthr_key, (size_t)cfg.stride_T) != cudaSuccess ||
-            ws->sthr.get(&w.sthr_idx, (size_t)cfg.stride_T) != cudaSuccess) {
-            ws->sthr.release();
-            return set_error(PCH_ERR_OOM, "strided selection thresholds: allocation failed");
+        for (int pass = 0; pass < 2; ++pass) {
+            Carver c;
+            c.base = static_cast<char*>(ws->sthr.p);
+            c.take(&w.sthr_key, (size_t)cfg.stride_T);
+            c.take(&w.sthr_idx, (size_t)cfg.stride_T);
+            if (pass == 0 && dev_alloc(ws->sthr, c.off) != cudaSuccess)
+                return set_error(PCH_ERR_OOM, "strided selection thresholds: allocation failed");
         }
         ws->sthr_cap = cfg.stride_T;
     }
@@ -1853,9 +1870,14 @@ pch_status solve_instances(pch_mesh* const* meshes, int n_inst, const SrcDev* sr
     ws->trace_on = opt && (opt->flags & PCH_FLAG_TRACE);
     if (ws->trace_on && !ws->trace_buf) {
         ws->trace_cap = 1 << 18;
-        if (ws->fixed.get(&ws->trace_buf, (size_t)ws->trace_cap * (kFeatures + 2)) != cudaSuccess ||
-            ws->fixed.get(&ws->trace_rows, 1) != cudaSuccess)
-            return set_error(PCH_ERR_OOM, "trace buffer allocation failed");
+        for (int pass = 0; pass < 2; ++pass) {
+            Carver c;
+            c.base = static_cast<char*>(ws->trace_mem.p);
+            c.take(&ws->trace_buf, (size_t)ws->trace_cap * (kFeatures + 2));
+            c.take(&ws->trace_rows, 1);
+            if (pass == 0 && dev_alloc(ws->trace_mem, c.off) != cudaSuccess)
+                return set_error(PCH_ERR_OOM, "trace buffer allocation failed");
+        }
     }
     w.trace = ws->trace_on ? ws->trace_buf : nullptr;
     w.trace_cap = ws->trace_cap;
@@ -1868,25 +1890,12 @@ pch_status solve_instances(pch_mesh* const* meshes, int n_inst, const SrcDev* sr
         w.plog = prov ? ws->plog : nullptr;
         w.plog_cap = prov ? ws->plog_cap : 0;
         // upload tables, clear state
-        PCH_CUDA(cudaMemcpyAsync(w.inst, hinst.data(), sizeof(Inst) * n_inst, cudaMemcpyHostToDevice, s));
-        PCH_CUDA(cudaMemcpyAsync(w.ctl, hctl.data(), sizeof(InstCtl) * n_inst, cudaMemcpyHostToDevice, s));
-        PCH_CUDA(cudaMemsetAsync(w.cnt, 0, sizeof(Counters), s));
-        PCH_CUDA(cudaMemsetAsync(w.hist[0], 0, sizeof(unsigned) * kBins * n_inst, s));
-        PCH_CUDA(cudaMemsetAsync(w.hist[1], 0, sizeof(unsigned) * kBins * n_inst, s));
-        PCH_CUDA(cudaMemsetAsync(ws->ang_all, 0xff, sizeof(unsigned long long) * aoff, s));
-        PCH_CUDA(cudaMemsetAsync(ws->stamp_all, 0, sizeof(unsigned) * goff, s));
-        PCH_CUDA(cudaMemsetAsync(ws->fanphi_all, 0xff, sizeof(float) * goff, s));   // NaN: no fan yet
-        if (w.trace_rows) PCH_CUDA(cudaMemsetAsync(w.trace_rows, 0, sizeof(int), s));
+        PCH_CUDA(cudaMemcpyAsync(ws->setup, ws->setup_host, src_at + sizeof(SrcDev) * n_src, cudaMemcpyHostToDevice, s));
         if (stats) std::memset(stats, 0, sizeof(pch_stats));
-        k_fill_inf<<<grid_for(4), 256, 0, s>>>(ws->g_all, goff);
-        SrcDev* dsrc = nullptr;
-        PCH_CUDA(cudaMallocAsync(&dsrc, sizeof(SrcDev) * n_src, s));
-        PCH_CUDA(cudaMemcpyAsync(dsrc, srcs, sizeof(SrcDev) * n_src, cudaMemcpyHostToDevice, s));
+        k_reset<<<grid_for(4), 256, 0, s>>>(w, ws->g_all, goff, ws->ang_all, aoff, ws->stamp_all, ws->fanphi_all);
         k_init_sources<<<(n_src + 127) / 128, 128, 0, s>>>(w, dsrc, n_src);
-        k_init_face_sources<<<(n_src + 127) / 128, 128, 0, s>>>(w, dsrc, n_src);
         PCH_CUDA(cudaGetLastError());
-        PCH_CUDA(cudaFreeAsync(dsrc, s));
-        if (stats) stats->kernel_launches = 3;
+        if (stats) stats->kernel_launches = 2;
         st = run_solve(ws, s, cfg, stats);
         if (st == PCH_ERR_CAPACITY && (ws->cnt_host->error & kErrReqFull) && attempt < 4) {
             st = ensure_pools(ws, ws->sel_cap, ws->pool_cap, 2 * ws->req_cap);
@@ -2107,10 +2116,10 @@ static pch_status trace_paths(pch_mesh* m, const SrcDev* sd, int n_src, const pc
     int *dpick = nullptr, *dtg = nullptr, *dn = nullptr;
     pch_path_point* dpts = nullptr;
     const size_t npts = (size_t)std::max(n_targets, 1) * (size_t)max_points;
-    cudaError_t e = cudaMallocAsync(&dpick, sizeof(int) * (size_t)nv, s);
-    if (!e) e = cudaMallocAsync(&dtg, sizeof(int) * (size_t)std::max(n_targets, 1), s);
-    if (!e) e = cudaMallocAsync(&dn, sizeof(int) * (size_t)std::max(n_targets, 1), s);
-    if (!e) e = cudaMallocAsync(&dpts, sizeof(pch_path_point) * npts, s);
+    cudaError_t e = tmp_alloc((void**)&dpick, sizeof(int) * (size_t)nv, s);
+    if (!e) e = tmp_alloc((void**)&dtg, sizeof(int) * (size_t)std::max(n_targets, 1), s);
+    if (!e) e = tmp_alloc((void**)&dn, sizeof(int) * (size_t)std::max(n_targets, 1), s);
+    if (!e) e = tmp_alloc((void**)&dpts, sizeof(pch_path_point) * npts, s);
     if (!e && n_targets > 0) e = cudaMemcpyAsync(dtg, targets, sizeof(int) * (size_t)n_targets, cudaMemcpyHostToDevice, s);
     if (!e) e = cudaMemsetAsync(dpick, 0x7f, sizeof(int) * (size_t)nv, s);
     if (!e) e = cudaStreamSynchronize(s);   // I (the instance table) is needed by value
@@ -2197,10 +2206,10 @@ static pch_status voronoi(pch_mesh* m, const SrcDev* sd, int n_src, const pch_op
     PCH_CUDA(cudaMemcpyAsync(&I, ws->w.inst, sizeof(Inst), cudaMemcpyDeviceToHost, s));
     int *dpick = nullptr, *dvsrc = nullptr, *dlab = nullptr;
     SrcDev* dsd = nullptr;
-    cudaError_t e = cudaMallocAsync(&dpick, sizeof(int) * (size_t)nv, s);
-    if (!e) e = cudaMallocAsync(&dvsrc, sizeof(int) * (size_t)nv, s);
-    if (!e) e = cudaMallocAsync(&dlab, sizeof(int) * (size_t)nv, s);
-    if (!e) e = cudaMallocAsync(&dsd, sizeof(SrcDev) * (size_t)n_src, s);
+    cudaError_t e = tmp_alloc((void**)&dpick, sizeof(int) * (size_t)nv, s);
+    if (!e) e = tmp_alloc((void**)&dvsrc, sizeof(int) * (size_t)nv, s);
+    if (!e) e = tmp_alloc((void**)&dlab, sizeof(int) * (size_t)nv, s);
+    if (!e) e = tmp_alloc((void**)&dsd, sizeof(SrcDev) * (size_t)n_src, s);
     if (!e) e = cudaMemcpyAsync(dsd, sd, sizeof(SrcDev) * (size_t)n_src, cudaMemcpyHostToDevice, s);
     if (!e) e = cudaMemsetAsync(dpick, 0x7f, sizeof(int) * (size_t)nv, s);
     if (!e) e = cudaMemsetAsync(dvsrc, 0x7f, sizeof(int) * (size_t)nv, s);   // 0x7f7f7f7f: no source
