@@ -274,7 +274,7 @@ def iso_contours(mesh: Mesh, dist, levels, capacity: int | None = None):
         _check(lib.pch_iso_contours(mesh.handle, _ptr(d), int(on_dev), lev.ctypes.data, lev.size, None, 0,
                                     ctypes.byref(n)))
         capacity = n.value
-    out = np.zeros(max(int(capacity), 1), dtype=CONTOUR_DTYPE)
+    out = np.empty(max(int(capacity), 1), dtype=CONTOUR_DTYPE)
     _check(lib.pch_iso_contours(mesh.handle, _ptr(d), int(on_dev), lev.ctypes.data, lev.size, out.ctypes.data,
                                 int(capacity), ctypes.byref(n)))
     return out[:min(n.value, int(capacity))]
