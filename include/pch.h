@@ -115,8 +115,9 @@ enum {
                                  (pch_stats.ms_phase); slower, for measurement only */
     PCH_FLAG_EDGE_SORT = 16   /* organise new windows by (instance, half-edge) with a radix
                                  sort and drop windows another window on the same edge
-                                 dominates (per-edge trimming); by default they are only
-                                 grouped by instance (Algorithm 3's gap-free copy) */
+                                 dominates (per-edge trimming); by default the next
+                                 iteration's selection reads them in the order they were
+                                 made (Algorithm 3's gap-free copy) */
 };
 
 /* Per-call statistics (the columns of Table `tab:speedup`: time, windows, peak windows). */

@@ -33,22 +33,22 @@ constexpr int kMlpParams = kMlpB4 + 1;
 //  f21     log2(1 + front distance / mean edge length) / 16
 //  f22     log2(1 + pending / faces) / 8
 //  f23     1
-__device__ __forceinline__ void controller_features(const InstCtl& c, const Inst& I, const unsigned* hist, int np,
+// `prefix`: inclusive sums of the 256-bin histogram.  Called by the first kFeatures threads
+// of a block.
+__device__ __forceinline__ void controller_features(const InstCtl& c, const Inst& I, const unsigned* prefix, int np,
                                                     int it, float* f) {
-    f[0] = log2f(1.f + (float)np) / 20.f;
-    unsigned run = 0;
-    for (int j = 0; j < 16; ++j) {
-        for (int b = j * 16; b < (j + 1) * 16; ++b) run += hist[b];
-        f[1 + j] = np > 0 ? (float)run / (float)np : 0.f;
-    }
-    float faces = (float)(I.nh / 3);
-    f[17] = log2f(faces) / 24.f;
-    f[18] = log2f((float)I.lbar) / 8.f;
-    f[19] = log2f(1.f + (float)it) / 16.f;
-    f[20] = c.last_ratio / 4.f;
-    f[21] = log2f(1.f + (float)(c.ref * I.ilbar)) / 16.f;
-    f[22] = log2f(1.f + (float)np / faces) / 8.f;
-    f[23] = 1.f;
+    const int j = threadIdx.x;
+    const float faces = (float)(I.nh / 3);
+    float v = 1.f;
+    if (j == 0) v = log2f(1.f + (float)np) / 20.f;
+    else if (j <= 16) v = np > 0 ? (float)prefix[16 * j - 1] / (float)np : 0.f;
+    else if (j == 17) v = log2f(faces) / 24.f;
+    else if (j == 18) v = log2f((float)I.lbar) / 8.f;
+    else if (j == 19) v = log2f(1.f + (float)it) / 16.f;
+    else if (j == 20) v = c.last_ratio / 4.f;
+    else if (j == 21) v = log2f(1.f + (float)(c.ref * I.ilbar)) / 16.f;
+    else if (j == 22) v = log2f(1.f + (float)np / faces) / 8.f;
+    f[j] = v;
 }
 
 // Block-cooperative forward pass (threads 0..63 compute one neuron each per layer).

@@ -80,8 +80,9 @@ struct WinSoA {
     double* B;
     double* px;     // pseudo-source position in the edge frame (py < 0)
     double* py;
-    double* key;    // d + dist(I, [A, B]): the window's distance back to the source (pools; the
-                    // append computes it, so that propagation does not)
+    double* key;    // d + dist(I, [A, B]): the window's distance back to the source (pools only:
+                    // the compaction computes it, so that propagation does not)
+    float* keyf;    // its FP32 image (the arena's windows from propagation)
     int* src;       // mesh vertex at the pseudo-source (-1 for a point inside a face)
 };
 // Endpoint events still to be made: the window's end A (or B) may lie at the edge's start
@@ -113,16 +114,17 @@ struct Inst {
     long long keybase;          // sort key = keybase + half-edge
     double lbar;
     double ilbar;
+    float ilbarf;               // 1 / lbar's FP32 image
     unsigned fbias;             // exponent offset of FP32 images: lbar's binade becomes [1, 2)
-    unsigned pad;
 };
 
 struct InstCtl {
     double tau;                 // selection threshold of the current iteration
     double ref;                 // histogram reference (a lower bound of every pending key)
-    unsigned long long kmin;    // running min of the keys written to the next pool (bits)
-    int n_pending;              // pending windows of this instance in the current pool
-    int n_next;                 // pending windows written to the next pool
+    unsigned kminf;             // running min of the pending keys' FP32 images (bits; ~0: none)
+    float reff;                 // ref as an FP32 image
+    int n_pending;              // pending windows of this instance
+    int n_next;                 // windows pending for the next iteration: left in the pool, or created
     int n_sel;                  // selected this iteration
     int n_child;                // children written this iteration
     long long k_target;         // plain control: windows to select
@@ -134,18 +136,22 @@ struct InstCtl {
 
 // ---- global counters of one solve -------------------------------------------------
 struct Counters {
-    int n_pending;          // windows in the current pool
+    int n_pending;          // pending windows: in the current pool and in the arena
+    int n_pool;             // windows in the current pool
+    int n_new;              // arena slots the last iteration's propagation and fans filled
     int n_rest;             // not-selected windows copied to the next pool
     int n_sel;              // selected windows (work list)
-    int n_child;            // slots used in the child arena
+    int n_child;            // arena slots used by the propagation
+    int n_fan;              // arena slots used by the fans, after those
     int n_req;              // fan requests for this iteration
     int n_req_next;         // fan requests for the next iteration
-    int n_app;              // windows appended to the next pool
+    int n_app;              // windows k_append added to the next pool
     int iter;
+    int ticket;             // blocks of k_ctrl that are done
     int error;              // bitmask of kErr*
     int done;
     int sort_bits;          // bits of the sort key
-    int halt;               // set by k_finish when the loop must stop; every kernel no-ops
+    int halt;               // set by k_ctrl when the loop must stop; every kernel no-ops
     unsigned long long created, propagated, filtered, trimmed, peak_pending;
     unsigned long long fans, fan_windows, fan_cand, chained;
     unsigned long long examined, occupied, children, rays;   // propagation path counts (FP64 op tally)
@@ -207,6 +213,7 @@ struct Work {
     Inst* inst;
     InstCtl* ctl;
     int n_inst;
+    int append;             // new windows reach the pool through k_append, not from the arena
     Counters* cnt;
     float* trace;           // controller trace rows
     int trace_cap;

@@ -1,8 +1,7 @@
-// Data organisation (Step 3 of Section 4.2, Algorithm 3): the windows a propagation
-// step produced are gathered into a gap-free pool, grouped by instance (so that the
-// append and the selection see one instance per warp), or on request in the order of
-// their edge key (instance key base + half-edge id) so that windows on one edge are
-// adjacent for the per-edge trimming of Step 4.  A single instance needs no sort.
+// Radix sort of the windows a propagation step produced (Step 3 of Section 4.2, Algorithm
+// 3) by their edge key (instance key base + half-edge id), on request: windows on one edge
+// are then adjacent for the per-edge trimming of Step 4.  Also of the faces by their Morton
+// code (mesh preparation).
 //
 // Hand-written stable LSD radix sort of (32-bit key, 32-bit index) pairs, 8-bit digits.
 // The element count n lives in device memory, so every launch has a fixed grid (graph
@@ -45,7 +44,7 @@ __device__ __forceinline__ unsigned rs_key(const RsIn& in, int i) {
     int h = in.he[i];
     if (h < 0) return ~0u;
     const int inst = in.inst[i] & kInstMask;
-    return in.by_edge ? (unsigned)(in.insts[inst].keybase + h) : (unsigned)inst;
+    return (unsigned)(in.insts[inst].keybase + h);
 }
 
 __global__ void __launch_bounds__(kRsThreads) k_rs_hist(RsIn in, const int* n_ptr, int cap, int shift, int* hist) {
@@ -136,7 +135,7 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(RsIn in, unsigned* __
 
 // Sort the child arena by edge key.  Leaves the sorted (key, index) pairs in
 // key_buf[r] / val_buf[r] and returns r.
-int launch_sort_children(const WinSoA& arena, const Inst* insts, const int* n_ptr, int cap, int key_bits, int by_edge,
+int launch_sort_children(const WinSoA& arena, const Inst* insts, const int* n_ptr, int cap, int key_bits,
                          unsigned* key_buf[2], int* val_buf[2], int* hist, int blocks, cudaStream_t s) {
     int passes = (key_bits + kRsDigitBits - 1) / kRsDigitBits;
     if (passes < 1) passes = 1;
@@ -148,7 +147,6 @@ int launch_sort_children(const WinSoA& arena, const Inst* insts, const int* n_pt
         in.he = arena.he;
         in.inst = arena.inst;
         in.insts = insts;
-        in.by_edge = by_edge;
         if (src >= 0) {
             in.keys = key_buf[src];
             in.vals = val_buf[src];

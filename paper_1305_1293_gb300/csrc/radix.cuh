@@ -15,10 +15,9 @@ struct RsIn {
     const int* he;
     const int* inst;
     const Inst* insts;
-    int by_edge;    // key = instance key base + half-edge; else the instance
 };
 
-int launch_sort_children(const WinSoA& arena, const Inst* insts, const int* n_ptr, int cap, int key_bits, int by_edge,
+int launch_sort_children(const WinSoA& arena, const Inst* insts, const int* n_ptr, int cap, int key_bits,
                          unsigned* key_buf[2], int* val_buf[2], int* hist, int blocks, cudaStream_t s);
 // Sort n_max (key, index) pairs by the low key_bits bits of key_buf[0] (n in device memory);
 // the sorted pairs are left in key_buf[r] / val_buf[r], r returned.

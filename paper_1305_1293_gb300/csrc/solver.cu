@@ -2,23 +2,25 @@
 //
 // One iteration, every phase a kernel over device-resident counts (fixed grids, so the
 // whole iteration can be replayed from a CUDA graph):
-//   k_tau        Step 1a: per-instance selection threshold from the key histogram
+//   k_ctrl       loop control (Algorithm 1's "until all windows are processed") and
+//                Step 1a: per-instance selection threshold from the key histogram
 //                (plain: the k-th nearest window, the paper's k; learned: MLP controller)
-//   k_compact    Step 1b: windows with key <= tau -> work list, the rest -> next pool
-//                (warp ballot / prefix compaction, structure-of-arrays copies)
+//   k_compact    Step 1b and Steps 3/4: pending windows (the pool and the windows created by
+//                the last iteration, re-filtered) with key <= tau -> work list, the rest ->
+//                next pool (Algorithm 3's gap-free copy; warp ballots, structure of arrays)
 //   k_propagate  Step 2, Algorithm 2: FP64 unfolding, endpoint / occupancy events,
 //                one angle one split, children, Xin-Wang filter
 //   k_fan        Step 2, Fig. `fig:propagation`(c): windows from improved pseudo-sources
-//   sort         Step 3, Algorithm 3: radix sort of the new windows by edge (radix.cu)
-//   k_append     Step 3/4: gap-free append in edge order with per-edge trimming and a
-//                re-filter against the updated distances
-//   k_finish     loop control (Algorithm 1's "until all windows are processed")
+// With PCH_FLAG_EDGE_SORT (radix sort of the new windows by edge, radix.cu, and per-edge
+// trimming) and under the strided control (whose selection reads every pending key) the new
+// windows are appended to the pool at the end of the iteration instead (k_append).
 // Events of Algorithm 4 are applied as they are produced: the vertex distance is an
 // atomicMin on the ordered 64-bit image of the nonnegative double, which keeps exactly
 // the first event of Algorithm 4's (key, value) order; angle_split is one packed 64-bit
 // word per half-edge (rounded-up distance | crossing position), also updated by atomicMin.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <vector>
 
@@ -63,33 +65,14 @@ __device__ __forceinline__ unsigned long long pack_angle(double D, long long pos
 // kEpsSnap (2^-40 of the edge) in position units.
 constexpr long long kSplitTol = 1ll << (kPosBits - 40);
 
-struct WarpScan {
-    int excl, total;
-};
-__device__ __forceinline__ WarpScan warp_scan(int x) {
+// Warp-aggregated reservation of one slot for every lane with `on` on counter `c` (called
+// by the whole warp); returns the lane's slot.
+__device__ __forceinline__ int warp_reserve(int* c, bool on) {
     const int lane = threadIdx.x & 31;
-    int incl = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    return {incl - x, __shfl_sync(0xffffffffu, incl, 31)};
-}
-
-// Warp-aggregated reservation of `x` slots per lane on counter `c`; returns the lane's
-// base.
-__device__ __forceinline__ int warp_reserve(int* c, int x) {
-    WarpScan s = warp_scan(x);
+    const unsigned m = __ballot_sync(0xffffffffu, on);
     int base = 0;
-    if ((threadIdx.x & 31) == 31 && s.total) base = atomicAdd(c, s.total);
-    base = __shfl_sync(0xffffffffu, base, 31);
-    return base + s.excl;
-}
-
-__device__ __forceinline__ void warp_add_ull(unsigned long long* c, int x) {
-    int t = warp_scan(x).total;
-    if ((threadIdx.x & 31) == 0 && t) atomicAdd(c, (unsigned long long)t);
+    if (lane == 0 && m) base = atomicAdd(c, __popc(m));
+    return __shfl_sync(0xffffffffu, base, 0) + __popc(m & ((1u << lane) - 1u));
 }
 
 // Where a distance event came from (kept only for geodesic paths): the window's half-edge
@@ -175,60 +158,86 @@ __device__ __forceinline__ void push_fan(FanReq* req, int* n, int cap, int* err,
     }
 }
 
-__device__ __forceinline__ int hist_bin(double key, double ref, double ilbar) {
-    float t = (float)((key - ref) * ilbar);
-    t = fmaxf(t, 0.f);
-    float b = kBinsPerOctave * __log2f(1.f + kBinScale * t);
-    int bi = (int)b;
-    return bi < 0 ? 0 : (bi >= kBins ? kBins - 1 : bi);
+__device__ __forceinline__ int hist_bin(float t) {      // t: distance of the key from ref, in lbar
+    const int b = (int)(kBinsPerOctave * __log2f(1.f + kBinScale * fmaxf(t, 0.f)));
+    return b < 0 ? 0 : (b >= kBins ? kBins - 1 : b);
 }
 
+// Upper edge of bin b (single-precision exponential: the FP64 one is a chain of some fifty
+// FP64 instructions, and tau only has to lie near the bin's edge).
 __device__ __forceinline__ double bin_upper(int b, double ref, double lbar) {
-    return ref + lbar * (exp2((double)(b + 1) / (double)kBinsPerOctave) - 1.0) / (double)kBinScale;
+    return ref + lbar * (double)((exp2f((float)(b + 1) / kBinsPerOctave) - 1.f) / kBinScale);
 }
 
-// Writes of windows into the next pool also feed the next iteration's selection
-// statistics: per-instance histogram (relative to ctl.ref), minimum key and count.
-struct PoolStats {
-    unsigned* sh_hist;   // shared-memory histogram (n_inst <= kShHistInst) or nullptr
-    unsigned* g_hist;
-    int n_inst;
-};
+// Every window that becomes pending for the next iteration feeds its selection statistics:
+// per-instance histogram (relative to ctl.ref), minimum key and count, from the FP32 image
+// of its key.  A block that reads many windows collects them in shared memory (up to
+// kShHistInst instances); a window just created adds to the global ones.
 constexpr int kShHistInst = 32;      // 32 KB of shared memory per block
-
-__device__ __forceinline__ void pool_stat(const Work& w, const PoolStats& ps, int inst, double key, bool on) {
-    // minimum key per instance: warp-reduce when the warp holds a single instance
-    const unsigned full = 0xffffffffu;
-    unsigned long long kb = on ? dbits(key) : ~0ull;
-    int inst0 = __shfl_sync(full, inst, 0);
-    bool uniform = __all_sync(full, !on || inst == inst0);
-    if (uniform) {
-        unsigned long long m = kb;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            unsigned long long t = __shfl_xor_sync(full, m, o);
-            m = t < m ? t : m;
+struct PoolStats {
+    unsigned hist[kShHistInst * kBins];
+    unsigned kminf[kShHistInst];
+    int n[kShHistInst];
+};
+__device__ __forceinline__ void stats_begin(PoolStats& ps, int n_inst) {
+    if (n_inst > kShHistInst) return;
+    for (int j = threadIdx.x; j < n_inst * kBins; j += blockDim.x) ps.hist[j] = 0u;
+    for (int j = threadIdx.x; j < n_inst; j += blockDim.x) { ps.kminf[j] = ~0u; ps.n[j] = 0; }
+    __syncthreads();
+}
+__device__ __forceinline__ void stats_end(const Work& w, PoolStats& ps, unsigned* g_hist) {
+    if (w.n_inst > kShHistInst) return;
+    __syncthreads();
+    for (int j = threadIdx.x; j < w.n_inst * kBins; j += blockDim.x)
+        if (ps.hist[j]) atomicAdd(&g_hist[j], ps.hist[j]);
+    for (int j = threadIdx.x; j < w.n_inst; j += blockDim.x)
+        if (ps.n[j]) {
+            atomicMin(&w.ctl[j].kminf, ps.kminf[j]);
+            atomicAdd(&w.ctl[j].n_next, ps.n[j]);
         }
-        int cntw = __popc(__ballot_sync(full, on));
-        if ((threadIdx.x & 31) == 0 && cntw) {
-            atomicMin(&w.ctl[inst0].kmin, m);
-            atomicAdd(&w.ctl[inst0].n_next, cntw);
+}
+// One window of a whole warp's (lanes with `on`), key as its image.
+__device__ __forceinline__ void stats_add(const Work& w, PoolStats& ps, unsigned* g_hist, int inst, float key, bool on) {
+    const unsigned full = 0xffffffffu, m = __ballot_sync(full, on);
+    if (!m) return;
+    const int lane = threadIdx.x & 31;
+    const bool shared = w.n_inst <= kShHistInst;
+    const int inst0 = __shfl_sync(full, inst, __ffs(m) - 1);
+    const unsigned kb = on ? __float_as_uint(key) : ~0u;
+    if (__all_sync(full, !on || inst == inst0)) {
+        const unsigned mn = __reduce_min_sync(full, kb);
+        if (lane == 0) {
+            atomicMin(shared ? &ps.kminf[inst0] : &w.ctl[inst0].kminf, mn);
+            atomicAdd(shared ? &ps.n[inst0] : &w.ctl[inst0].n_next, __popc(m));
         }
     } else if (on) {
-        atomicMin(&w.ctl[inst].kmin, kb);
-        atomicAdd(&w.ctl[inst].n_next, 1);
+        atomicMin(shared ? &ps.kminf[inst] : &w.ctl[inst].kminf, kb);
+        atomicAdd(shared ? &ps.n[inst] : &w.ctl[inst].n_next, 1);
     }
     if (on) {
-        const InstCtl& c = w.ctl[inst];
-        int b = hist_bin(key, c.ref, w.inst[inst].ilbar);
-        if (ps.sh_hist) {
-            atomicAdd(&ps.sh_hist[inst * kBins + b], 1u);
+        const int slot = inst * kBins + hist_bin((key - w.ctl[inst].reff) * w.inst[inst].ilbarf);
+        if (shared) {
+            atomicAdd(&ps.hist[slot], 1u);
         } else {
             // many instances: lanes that hit the same global bin add together
-            const int slot = inst * kBins + b;
             const unsigned peers = __match_any_sync(__activemask(), slot);
-            if ((threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&ps.g_hist[slot], (unsigned)__popc(peers));
+            if (lane == __ffs(peers) - 1) atomicAdd(&g_hist[slot], (unsigned)__popc(peers));
         }
+    }
+}
+// A window just written to the arena (the lanes that wrote one).
+__device__ __forceinline__ void stats_created(const Work& w, unsigned* g_hist, int inst, float key) {
+    atomicAdd(&g_hist[inst * kBins + hist_bin((key - w.ctl[inst].reff) * w.inst[inst].ilbarf)], 1u);
+    const unsigned m = __activemask();
+    if (w.n_inst == 1) {
+        const unsigned mn = __reduce_min_sync(m, __float_as_uint(key));
+        if ((threadIdx.x & 31) == __ffs(m) - 1) {
+            atomicMin(&w.ctl[0].kminf, mn);
+            atomicAdd(&w.ctl[0].n_next, __popc(m));
+        }
+    } else {
+        atomicMin(&w.ctl[inst].kminf, __float_as_uint(key));
+        atomicAdd(&w.ctl[inst].n_next, 1);
     }
 }
 
@@ -270,7 +279,8 @@ __global__ void __launch_bounds__(256) k_reset(Work w, unsigned long long* g, lo
     }
     for (long long i = t; i < (long long)w.n_inst * kBins; i += step) w.hist[0][i] = w.hist[1][i] = 0u;
     static_assert(sizeof(Counters) % 4 == 0, "cleared by words");
-    if (t < (long long)(sizeof(Counters) / 4)) reinterpret_cast<int*>(w.cnt)[t] = 0;
+    if (t < (long long)(sizeof(Counters) / 4))
+        reinterpret_cast<int*>(w.cnt)[t] = t == (long long)(offsetof(Counters, iter) / 4) ? -1 : 0;
     if (t == 0 && w.trace_rows) *w.trace_rows = 0;
 }
 
@@ -285,7 +295,7 @@ __global__ void k_init_sources(Work w, const SrcDev* __restrict__ srcs, int n_sr
         if (s.kind == 0) {
             I.g[s.vertex] = 0ull;
             // the source's fan covers every direction
-            push_fan(w.req[0], &cnt->n_req, w.req_cap, &cnt->error, s.inst, (unsigned)s.vertex, 0.0, -1, 0.0, 0.0);
+            push_fan(w.req[0], &cnt->n_req_next, w.req_cap, &cnt->error, s.inst, (unsigned)s.vertex, 0.0, -1, 0.0, 0.0);
             continue;
         }
         // a point inside a face: corner distances and three windows, to the child arena of
@@ -302,87 +312,157 @@ __global__ void k_init_sources(Work w, const SrcDev* __restrict__ srcs, int n_sr
             const EvSrc es{s.inst, h, -1 - s.label, 2, x, y};
             if (const int ev = w.plog ? vertex_event<true>(I, R.v0, dstart, gc, &w, &es) : vertex_event(I, R.v0, dstart, gc)) {
                 // incoming direction: from the corner towards the point, inside face(h)
-                push_fan(w.req[0], &cnt->n_req, w.req_cap, &cnt->error, s.inst, R.v0 & ~kPseudoBit, dstart, h, x, y, ev);
+                push_fan(w.req[0], &cnt->n_req_next, w.req_cap, &cnt->error, s.inst, R.v0 & ~kPseudoBit, dstart, h, x, y, ev);
             }
             if (R.twin < 0) continue;
             // window on twin(h) = (v1 -> v0): point at (L - x, -y), interval [0, L]
             double px = R.L - x, py = -y;
             int slot = atomicAdd(&cnt->n_child, 1);
-            if (slot < w.arena_cap)
+            if (slot < w.arena_cap) {
                 store_win(w.arena, slot, {R.twin, s.inst, -1 - s.label, kPendA | kPendB, 0.0, 0.0, R.L, px, py, 0.0});
+                if (!w.append) {
+                    const float fx = f_of(px < 0.0 ? px : (px > R.L ? px - R.L : 0.0), I.fbias), fy = f_of(py, I.fbias);
+                    stats_created(w, w.hist[0], s.inst, sqrtf(fmaf(fx, fx, fy * fy)));
+                }
+            }
         }
     }
 }
 
 // ====================================================================== Step 1: selection
-// Per instance: the plain control selects the k nearest windows (Section 4.2, Step 1)
-// through the key histogram: tau = upper edge of the first bin where the cumulative
-// count reaches k.  Also rolls the histogram reference and the running minimum.
-__global__ void k_tau(Work w, int control, const float* __restrict__ mlp) {
-    __shared__ unsigned sh[kBins];
+// Loop control, then per instance the selection threshold: the plain control selects the k
+// nearest windows (Section 4.2, Step 1) through the key histogram: tau = upper edge of the
+// first bin where the cumulative count reaches k.  Also rolls the histogram reference and
+// the running minimum.  Every block decides from the counters as the last iteration left
+// them; the block that finishes last resets them for this one.  kBins threads a block.
+__global__ void __launch_bounds__(kBins) k_ctrl(Work w, int control, const float* __restrict__ mlp,
+                                                cudaGraphConditionalHandle handle, int use_cond, long long max_iters) {
+    __shared__ unsigned prefix[kBins];
+    __shared__ unsigned wsum[kBins / 32];
     __shared__ float feat[kFeatures];
     __shared__ float hb0[kHidden], hb1[kHidden];
     __shared__ float y;
+    __shared__ int s_bin;
+    __shared__ long long s_k;
     Counters* cnt = w.cnt;
-    if (cnt->halt) return;
-    const int it = cnt->iter;
-    const unsigned* hist = w.hist[it & 1];
-    unsigned* hist_nx = w.hist[(it + 1) & 1];
-    for (int inst = blockIdx.x; inst < w.n_inst; inst += gridDim.x) {
-        InstCtl& c = w.ctl[inst];
-        const int np = c.n_next;
-        for (int b = threadIdx.x; b < kBins; b += blockDim.x) sh[b] = hist[inst * kBins + b];
-        __syncthreads();
-        const bool learned = control == PCH_CONTROL_LEARNED && mlp != nullptr && np > 0;
-        if ((learned || w.trace) && threadIdx.x == 0) controller_features(c, w.inst[inst], sh, np, it, feat);
-        __syncthreads();
-        if (learned) mlp_forward_block(mlp, feat, hb0, hb1, &y);
-        if (threadIdx.x == 0) {
-            double tau;
-            const double ref = c.ref;
-            const double lbar = w.inst[inst].lbar;
-            long long k = c.k_target;
-            if (learned) {
-                c.ctl_out = y;
-                // y = log2(windows to select) / 24, clamped to the range of k the network
-                // was trained on (2^12 to 2^24); the plain k only when it is not finite.
-                // (Falling back to the plain k for a finite output beyond that range, a
-                // small k under this control, made late iterations select few windows.)
-                if (isfinite(y)) k = (long long)exp2(24.0 * (double)fminf(fmaxf(y, 12.f / 24.f), 1.f));
+    if (cnt->halt) {
+        if (use_cond && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(handle, 0u);
+        return;
+    }
+    const int t = threadIdx.x, lane = t & 31;
+    const int it = cnt->iter + 1;
+    const int n_child = min(cnt->n_child + cnt->n_fan, w.arena_cap), n_sel = cnt->n_sel;
+    const int n_pool = cnt->n_rest + cnt->n_app, n_new = w.append ? 0 : n_child;
+    const int n_req = min(cnt->n_req_next, w.req_cap);
+    int error = cnt->error;
+    // done; an error; or the pool may not hold what this iteration leaves (the host grows it).
+    // (A face-point source's windows are in the arena before iteration 0: k_append takes
+    // them with that iteration's own.)
+    const int kept = w.append && it > 0 ? 0 : n_child;
+    const bool done = n_pool + kept == 0 && n_req == 0;
+    if (!done && (long long)it >= max_iters) error |= kErrIter;
+    const bool grow = n_pool + (w.append ? w.arena_cap : n_new) > w.pool_cap;
+    const bool halt = done || error != 0 || grow;
+    if (!halt) {
+        const unsigned* hist = w.hist[it & 1];
+        unsigned* hist_nx = w.hist[(it + 1) & 1];
+        for (int inst = blockIdx.x; inst < w.n_inst; inst += gridDim.x) {
+            InstCtl& c = w.ctl[inst];
+            const int np = c.n_next;
+            unsigned incl = hist[inst * kBins + t];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned x = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += x;
             }
-            if (np == 0) {
-                tau = -INFINITY;
-            } else if ((long long)np <= k) {
-                tau = INFINITY;
-            } else {
-                long long run = 0;
-                int b = 0;
-                for (; b < kBins; ++b) {
-                    run += sh[b];
-                    if (run >= k) break;
+            if (lane == 31) wsum[t / 32] = incl;
+            hist_nx[inst * kBins + t] = 0u;
+            __syncthreads();
+            for (int q = 0; q < t / 32; ++q) incl += wsum[q];
+            prefix[t] = incl;
+            if (t == 0) c.last_ratio = n_sel > 0 ? (float)n_child / (float)n_sel : 0.f;
+            __syncthreads();
+            const bool learned = control == PCH_CONTROL_LEARNED && mlp != nullptr && np > 0;
+            if (learned || w.trace) {
+                if (t < kFeatures) controller_features(c, w.inst[inst], prefix, np, it, feat);
+                __syncthreads();
+                if (learned) mlp_forward_block(mlp, feat, hb0, hb1, &y);
+            }
+            if (t == 0) {
+                long long k = c.k_target;
+                if (learned) {
+                    c.ctl_out = y;
+                    // y = log2(windows to select) / 24, clamped to the range of k the network
+                    // was trained on (2^12 to 2^24); the plain k only when it is not finite.
+                    // (Falling back to the plain k for a finite output beyond that range, a
+                    // small k under this control, made late iterations select few windows.)
+                    if (isfinite(y)) k = (long long)exp2(24.0 * (double)fminf(fmaxf(y, 12.f / 24.f), 1.f));
                 }
-                tau = b >= kBins - 1 ? INFINITY : bin_upper(b, ref, lbar);
+                s_k = k;
+                s_bin = kBins - 1;
             }
-            if (w.trace && np > 0) {
-                int row = atomicAdd(w.trace_rows, 1);
-                if (row < w.trace_cap) {
-                    float* f = w.trace + (size_t)row * (kFeatures + 2);
-                    for (int j = 0; j < kFeatures; ++j) f[j] = feat[j];
-                    f[kFeatures] = (float)(log2((double)k) / 24.0);
-                    f[kFeatures + 1] = (float)inst;
+            __syncthreads();
+            if ((long long)prefix[t] >= s_k && (t == 0 || (long long)prefix[t - 1] < s_k)) s_bin = t;
+            __syncthreads();
+            if (t == 0) {
+                const double ref = c.ref;
+                const unsigned fbias = w.inst[inst].fbias;
+                double tau = INFINITY;
+                if (np == 0) tau = -INFINITY;
+                else if ((long long)np > s_k && s_bin < kBins - 1) tau = bin_upper(s_bin, ref, w.inst[inst].lbar);
+                if (w.trace && np > 0) {
+                    int row = atomicAdd(w.trace_rows, 1);
+                    if (row < w.trace_cap) {
+                        float* f = w.trace + (size_t)row * (kFeatures + 2);
+                        for (int j = 0; j < kFeatures; ++j) f[j] = feat[j];
+                        f[kFeatures] = (float)(log2((double)s_k) / 24.0);
+                        f[kFeatures + 1] = (float)inst;
+                    }
                 }
+                // the strided selection decides by per-thread thresholds instead; tau = -inf
+                // also turns chaining off (the paper propagates each selected window one hop)
+                c.tau = control == PCH_CONTROL_STRIDED ? -INFINITY : tau;
+                c.tauf = f_of(c.tau, fbias);
+                c.n_pending = np;
+                c.n_next = 0;
+                if (c.kminf != ~0u) {              // min key of the pending windows
+                    c.ref = of_f_bits(c.kminf, fbias);
+                    c.reff = __uint_as_float(c.kminf);
+                }
+                c.kminf = ~0u;
             }
-            // the strided selection decides by per-thread thresholds instead; tau = -inf
-            // also turns chaining off (the paper propagates each selected window one hop)
-            c.tau = control == PCH_CONTROL_STRIDED ? -INFINITY : tau;
-            c.tauf = f_of(c.tau, w.inst[inst].fbias);
-            c.n_pending = np;
-            c.n_next = 0;
-            if (c.kmin != ~0ull) c.ref = bitsd(c.kmin);   // min key of the current pool
-            c.kmin = ~0ull;
+            __syncthreads();
         }
-        for (int b = threadIdx.x; b < kBins; b += blockDim.x) hist_nx[inst * kBins + b] = 0u;
-        __syncthreads();
+    }
+    if (t == 0) {
+        __threadfence();
+        if (atomicAdd(&cnt->ticket, 1) == (int)gridDim.x - 1) {      // every block has read the counters
+            cnt->ticket = 0;
+            cnt->error = error;
+            cnt->done = done ? 1 : 0;
+            cnt->n_pending = n_pool + n_new;
+            if (!halt || done || error) {
+                cnt->iter = it;
+                cnt->scanned += (unsigned long long)n_pool;
+                cnt->sorted += (unsigned long long)n_child;
+                if ((unsigned long long)(n_pool + n_new) > cnt->peak_pending)
+                    cnt->peak_pending = (unsigned long long)(n_pool + n_new);
+            }
+            if (!halt) {
+                cnt->n_pool = n_pool;
+                cnt->n_new = n_new;
+                cnt->n_req = n_req;
+                cnt->n_req_next = 0;
+                cnt->n_rest = 0;
+                cnt->n_sel = 0;
+                cnt->n_child = w.append ? kept : 0;
+                cnt->n_fan = 0;
+                cnt->n_app = 0;
+                cnt->work_next = 0;
+            }
+            cnt->halt = halt ? 1 : 0;
+            if (use_cond) cudaGraphSetConditional(handle, halt ? 0u : 1u);
+        }
     }
 }
 
@@ -399,7 +479,7 @@ __global__ void __launch_bounds__(256) k_strided(Work w) {
     if (cnt->halt) return;
     const int T = w.stride_T;
     const double* __restrict__ key = w.pool[cnt->iter & 1].key;
-    const int n = min(cnt->n_pending, w.pool_cap);
+    const int n = cnt->n_pool;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < T; t += gridDim.x * blockDim.x) {
         unsigned long long bk[M];
         int bi[M];
@@ -424,27 +504,50 @@ __global__ void __launch_bounds__(256) k_strided(Work w) {
     }
 }
 
-// Compaction: selected windows to the work list, the rest to the next pool.
+// A window's distance back to the source: from the point of [A, B] nearest I.
+__device__ __forceinline__ double window_key(const Win& W) {
+    const double foot = lt_s(W.px, W.A) ? W.A - W.px : (lt_s(W.B, W.px) ? W.B - W.px : 0.0);
+    return W.d + (sbits(foot) == 0 ? -W.py : sqrt_nr(fma(foot, foot, W.py * W.py)));
+}
+// A window created by the last iteration against the distances after its events (it is
+// nowhere closer than its key).
+__device__ __forceinline__ bool created_useless(const Inst& I, const Win& W) {
+    const HERec& R = I.rec[W.he];
+    const double g0 = ldg_dist(I.g, R.v0 & ~kPseudoBit), g1 = ldg_dist(I.g, R.v1 & ~kPseudoBit);
+    return dominated(W.key, g0 + W.B) || dominated(W.key, g1 + (R.L - W.A)) || stale_source(I, W.src, W.d);
+}
+
+// Compaction: selected windows to the work list, the rest to the next pool.  Reads the
+// pending windows where they are, in the pool and in the arena, so a created window is
+// written and read once on its way to the work list.
 __global__ void __launch_bounds__(256) k_compact(Work w) {
-    __shared__ unsigned sh_hist[kShHistInst * kBins];
+    __shared__ PoolStats ps;
     Counters* cnt = w.cnt;
     if (cnt->halt) return;
-    const int it = cnt->iter;
+    const int it = cnt->iter, lane = threadIdx.x & 31;
     const WinSoA cur = w.pool[it & 1], nxt = w.pool[(it + 1) & 1];
-    const int n = min(cnt->n_pending, w.pool_cap);
-    PoolStats ps{w.n_inst <= kShHistInst ? sh_hist : nullptr, w.hist[(it + 1) & 1], w.n_inst};
-    if (ps.sh_hist) {
-        for (int j = threadIdx.x; j < w.n_inst * kBins; j += blockDim.x) sh_hist[j] = 0u;
-        __syncthreads();
-    }
+    const int n_pool = cnt->n_pool, n = n_pool + cnt->n_new;
+    unsigned* g_hist = w.hist[(it + 1) & 1];
+    if (blockIdx.x * blockDim.x >= n) return;
+    stats_begin(ps, w.n_inst);
+    int created = 0;
     for (int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
-        int i = base + threadIdx.x;
+        const int i = base + threadIdx.x;
         bool valid = i < n;
         Win W{0, 0, -1, 0u, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         if (valid) {
-            W = load_win(cur, i);
-            W.key = cur.key[i];
-            if (stale_source(w.inst[W.inst], W.src, W.d)) valid = false;   // dropped from the pool
+            if (i < n_pool) {
+                W = load_win(cur, i);
+                W.key = cur.key[i];
+                if (stale_source(w.inst[W.inst], W.src, W.d)) valid = false;   // dropped from the pool
+            } else if (w.arena.he[i - n_pool] < 0) {
+                valid = false;                                                 // an empty slot
+            } else {
+                W = load_win(w.arena, i - n_pool);
+                W.key = window_key(W);
+                valid = !created_useless(w.inst[W.inst], W);
+                created += valid ? 1 : 0;
+            }
         }
         bool sel;
         if (w.stride_T > 0) {           // strided selection: the owning thread's threshold
@@ -452,24 +555,31 @@ __global__ void __launch_bounds__(256) k_compact(Work w) {
             const unsigned long long kb = dbits(W.key), tk = w.sthr_key[t];
             sel = valid && (kb < tk || (kb == tk && i <= w.sthr_idx[t]));
         } else {
-            sel = valid && W.key <= w.ctl[W.inst].tau;
+            sel = valid && le_s(W.key, w.ctl[W.inst].tau);
         }
-        int slot = warp_reserve(&cnt->n_sel, sel ? 1 : 0);
-        if (sel && slot >= w.sel_cap) sel = false;   // work list full: stays pending
-        if (sel) store_win(w.sel, slot, W);
+        // both reservations at once, from two lanes
         bool rest = valid && !sel;
-        int rslot = warp_reserve(&cnt->n_rest, rest ? 1 : 0);
+        const unsigned sm = __ballot_sync(0xffffffffu, sel), rm = __ballot_sync(0xffffffffu, rest);
+        const unsigned lt = (1u << lane) - 1u;
+        int got = 0;
+        if (lane < 2 && (lane ? rm : sm)) got = atomicAdd(lane ? &cnt->n_rest : &cnt->n_sel, __popc(lane ? rm : sm));
+        int slot = __shfl_sync(0xffffffffu, got, 0) + __popc(sm & lt);
+        int rslot = __shfl_sync(0xffffffffu, got, 1) + __popc(rm & lt);
+        const bool over = sel && slot >= w.sel_cap;         // work list full: stays pending
+        if (sel && !over) store_win(w.sel, slot, W);
+        if (__any_sync(0xffffffffu, over)) {
+            const int s2 = warp_reserve(&cnt->n_rest, over);
+            if (over) { rest = true; rslot = s2; }
+        }
         if (rest) {
             store_win(nxt, rslot, W);
             nxt.key[rslot] = W.key;
         }
-        pool_stat(w, ps, W.inst, W.key, rest);
+        stats_add(w, ps, g_hist, W.inst, f_of(W.key, w.inst[W.inst].fbias), rest);
     }
-    if (ps.sh_hist) {
-        __syncthreads();
-        for (int j = threadIdx.x; j < w.n_inst * kBins; j += blockDim.x)
-            if (sh_hist[j]) atomicAdd(&ps.g_hist[j], sh_hist[j]);
-    }
+    created = __reduce_add_sync(0xffffffffu, created);
+    if (lane == 0 && created) atomicAdd(&cnt->created, (unsigned long long)created);
+    stats_end(w, ps, g_hist);
 }
 
 // ====================================================================== Step 2: propagation
@@ -866,6 +976,7 @@ __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int
                     w.arena.B[slot] = c.B;
                     w.arena.px[slot] = c.px;
                     w.arena.py[slot] = c.py;
+                    w.arena.keyf[slot] = c.key;
                 } else {
                     atomicOr(&cnt->error, kErrPoolFull);
                 }
@@ -942,6 +1053,20 @@ template <bool PROV>
 __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
     Counters* cnt = w.cnt;
     if (cnt->halt) return;
+    // first the selection statistics of the windows that the propagation created (here, where
+    // the GPU has little else to do: from inside the propagation kernel they cost 8% of it)
+    __shared__ PoolStats ps;
+    const int n_prop = min(cnt->n_child, w.arena_cap);
+    if (!w.append && blockIdx.x * blockDim.x < n_prop) {
+        unsigned* g_hist = w.hist[(cnt->iter + 1) & 1];
+        stats_begin(ps, w.n_inst);
+        for (int base = blockIdx.x * blockDim.x; base < n_prop; base += gridDim.x * blockDim.x) {
+            const int i = base + threadIdx.x;
+            const bool on = i < n_prop;
+            stats_add(w, ps, g_hist, on ? w.arena.inst[i] & kInstMask : 0, on ? w.arena.keyf[i] : 0.f, on);
+        }
+        stats_end(w, ps, g_hist);
+    }
     const int lane = threadIdx.x & 31;
     const int sl = lane & (kFanLanes - 1);
     const int lead = lane & ~(kFanLanes - 1);
@@ -1125,7 +1250,7 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
             const unsigned bal = (__ballot_sync(gmask, win) >> lead) & ((1u << kFanLanes) - 1u);
             const int cntw = __popc(bal);
             int base = 0;
-            if (sl == 0 && cntw) base = atomicAdd(&cnt->n_child, cntw);
+            if (sl == 0 && cntw) base = w.append ? atomicAdd(&cnt->n_child, cntw) : n_prop + atomicAdd(&cnt->n_fan, cntw);
             base = __shfl_sync(gmask, base, lead);
             if (base + cntw > w.arena_cap) {
                 // no room this iteration: mark the reserved slots empty, retry next iteration
@@ -1167,6 +1292,9 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
                 continue;
             }
             store_win(w.arena, slot, {Ro.twin, rq.inst, (int)v, kPendA | kPendB, D, A, B, px, py, 0.0});
+            if (!w.append)
+                stats_created(w, w.hist[(it + 1) & 1], rq.inst,
+                              f_of(D + (px < A ? IA : (px > B ? IB : -py)), I.fbias));
             ++n_fwin;
         }
     }
@@ -1176,44 +1304,36 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
 }
 
 // ====================================================================== Step 3/4: append
+// (edge sort and strided control only) The new windows, in their sorted order if there is
+// one, to the end of the next pool, with the re-filter and the per-edge trimming.
 __global__ void __launch_bounds__(256) k_append(Work w, const unsigned* __restrict__ keys, const int* __restrict__ vals,
                                                 int trim) {
-    __shared__ unsigned sh_hist[kShHistInst * kBins];
+    __shared__ PoolStats ps;
     Counters* cnt = w.cnt;
     if (cnt->halt) return;
     const int it = cnt->iter;
     const WinSoA nxt = w.pool[(it + 1) & 1];
-    const int n = min(cnt->n_child, w.arena_cap);
+    const int n = min(cnt->n_child + cnt->n_fan, w.arena_cap);
     const int n_rest = cnt->n_rest;
-    PoolStats ps{w.n_inst <= kShHistInst ? sh_hist : nullptr, w.hist[(it + 1) & 1], w.n_inst};
-    if (ps.sh_hist) {
-        for (int j = threadIdx.x; j < w.n_inst * kBins; j += blockDim.x) sh_hist[j] = 0u;
-        __syncthreads();
-    }
+    unsigned* g_hist = w.hist[(it + 1) & 1];
+    if (blockIdx.x * blockDim.x >= n) return;
+    stats_begin(ps, w.n_inst);
     constexpr int kTrimReach = 4;
+    int trimmed = 0, created = 0;
     for (int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
         const int i = base + threadIdx.x;
         // without a sort (keys == nullptr) the arena is appended in its own order
         unsigned k = i < n ? (keys ? keys[i] : (w.arena.he[i] < 0 ? ~0u : 0u)) : ~0u;
         bool keep = k != ~0u;
         Win W{0, 0, -1, 0u, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        int trimmed = 0;
         if (keep) {
             W = load_win(w.arena, keys ? vals[i] : i);
-            const double d = W.d, A = W.A, B = W.B;
-            const Inst& I = w.inst[W.inst];
-            const HERec R = I.rec[W.he];
-            // the window's distance back to the source: from the point of [A, B] nearest I
-            const double foot = W.px < A ? A - W.px : (W.px > B ? B - W.px : 0.0);
-            const double key = d + (foot == 0.0 ? -W.py : sqrt_nr(fma(foot, foot, W.py * W.py)));
-            W.key = key;
-            // re-filter against the distances after this iteration's events (the window
-            // is nowhere closer than `key`)
-            double g0 = ldg_dist(I.g, R.v0 & ~kPseudoBit), g1 = ldg_dist(I.g, R.v1 & ~kPseudoBit);
-            if (dominated(key, g0 + B) || dominated(key, g1 + (R.L - A)) || stale_source(I, W.src, d)) keep = false;
+            W.key = window_key(W);
+            keep = !created_useless(w.inst[W.inst], W);
             // per-edge trimming: a window on the same edge that covers [A, B] and is
             // everywhere shorter than this window's nearest point makes it useless
             if (keep && trim) {
+                const double A = W.A, B = W.B;
                 for (int dir = -1; dir <= 1 && keep; dir += 2) {
                     for (int s = 1; s <= kTrimReach && keep; ++s) {
                         int j = i + dir * s;
@@ -1224,12 +1344,13 @@ __global__ void __launch_bounds__(256) k_append(Work w, const unsigned* __restri
                         double d2 = w.arena.d[jj], px2 = w.arena.px[jj], py2 = w.arena.py[jj];
                         double ea = A - px2, eb = B - px2;
                         double mx = d2 + sqrt(fmax(ea * ea, eb * eb) + py2 * py2);
-                        if (dominated(key, mx)) { keep = false; trimmed = 1; }
+                        if (dominated(W.key, mx)) { keep = false; ++trimmed; }
                     }
                 }
             }
         }
-        int slot = warp_reserve(&cnt->n_app, keep ? 1 : 0);
+        created += keep ? 1 : 0;
+        int slot = warp_reserve(&cnt->n_app, keep);
         if (keep) {
             int pos = n_rest + slot;
             if (pos < w.pool_cap) {
@@ -1239,42 +1360,15 @@ __global__ void __launch_bounds__(256) k_append(Work w, const unsigned* __restri
                 atomicOr(&cnt->error, kErrPoolFull);
             }
         }
-        pool_stat(w, ps, W.inst, W.key, keep);
-        warp_add_ull(&cnt->trimmed, trimmed);
-        warp_add_ull(&cnt->created, keep ? 1 : 0);
+        stats_add(w, ps, g_hist, W.inst, f_of(W.key, w.inst[W.inst].fbias), keep);
     }
-    if (ps.sh_hist) {
-        __syncthreads();
-        for (int j = threadIdx.x; j < w.n_inst * kBins; j += blockDim.x)
-            if (sh_hist[j]) atomicAdd(&ps.g_hist[j], sh_hist[j]);
+    trimmed = __reduce_add_sync(0xffffffffu, trimmed);
+    created = __reduce_add_sync(0xffffffffu, created);
+    if ((threadIdx.x & 31) == 0) {
+        if (trimmed) atomicAdd(&cnt->trimmed, (unsigned long long)trimmed);
+        if (created) atomicAdd(&cnt->created, (unsigned long long)created);
     }
-}
-
-// ====================================================================== loop control
-__global__ void k_finish(Work w, cudaGraphConditionalHandle handle, int use_cond, long long max_iters) {
-    Counters* c = w.cnt;
-    if (!c->halt) {
-        c->scanned += (unsigned long long)min(c->n_pending, w.pool_cap);
-        c->sorted += (unsigned long long)min(c->n_child, w.arena_cap);
-        int np = c->n_rest + c->n_app;
-        const float ratio = c->n_sel > 0 ? (float)c->n_app / (float)c->n_sel : 0.f;
-        for (int i = 0; i < w.n_inst; ++i) w.ctl[i].last_ratio = ratio;
-        c->n_pending = np;
-        if ((unsigned long long)np > c->peak_pending) c->peak_pending = (unsigned long long)np;
-        c->n_req = min(c->n_req_next, w.req_cap);
-        c->n_req_next = 0;
-        c->n_rest = 0;
-        c->n_sel = 0;
-        c->n_child = 0;
-        c->n_app = 0;
-        c->work_next = 0;
-        c->iter += 1;
-        c->done = (np == 0 && c->n_req == 0) ? 1 : 0;
-        if (!c->done && c->iter >= max_iters) c->error |= kErrIter;
-        // stop for the host: finished, an error, or the pool may not hold one more iteration
-        c->halt = (c->done || c->error != 0 || np + w.arena_cap > w.pool_cap) ? 1 : 0;
-    }
-    if (use_cond) cudaGraphSetConditional(handle, c->halt ? 0u : 1u);
+    stats_end(w, ps, g_hist);
 }
 
 __global__ void k_copy_out(const unsigned long long* __restrict__ g, double* out, int n) {
@@ -1348,14 +1442,15 @@ static void drop_graph(Workspace* ws) {
     ws->graph = nullptr;
 }
 
-// `keyed`: the pending pools; the work list and the arena hold no keys.
-static void carve_soa(Carver& c, WinSoA& s, size_t cap, bool keyed) {
+// `keyed`: the pending pools; `imaged`: the arena, which holds the keys' FP32 images.
+static void carve_soa(Carver& c, WinSoA& s, size_t cap, bool keyed, bool imaged = false) {
     c.take(&s.d, cap);
     c.take(&s.A, cap);
     c.take(&s.B, cap);
     c.take(&s.px, cap);
     c.take(&s.py, cap);
     if (keyed) c.take(&s.key, cap);
+    if (imaged) c.take(&s.keyf, cap);
     c.take(&s.he, cap);
     c.take(&s.inst, cap);
     c.take(&s.src, cap);
@@ -1364,7 +1459,7 @@ static void carve_pools(Carver& c, Work& w, int pool_cap, int sel_cap, int arena
     carve_soa(c, w.pool[0], pool_cap, true);
     carve_soa(c, w.pool[1], pool_cap, true);
     carve_soa(c, w.sel, sel_cap, false);
-    carve_soa(c, w.arena, arena_cap, false);
+    carve_soa(c, w.arena, arena_cap, false, true);
     for (int j = 0; j < 2; ++j) {
         c.take(&w.req[j], req_cap);
         c.take(&w.sort_key[j], arena_cap);
@@ -1404,7 +1499,7 @@ static pch_status ensure_pools(Workspace* ws, int sel_cap, int pool_cap, int req
     c = Carver{static_cast<char*>(fresh.p), 0};
     carve_pools(c, nw, pool_cap, sel_cap, arena_cap, req_cap, sort_blocks);
     if (ws->pool_cap > 0) {
-        // growth between iterations: keep the pending pools and the fan requests
+        // growth between iterations: keep the pending windows and the fan requests
         const size_t n = (size_t)ws->pool_cap;
         for (int p = 0; p < 2; ++p) {
             cudaMemcpy(nw.pool[p].he, w.pool[p].he, n * 4, cudaMemcpyDeviceToDevice);
@@ -1418,6 +1513,15 @@ static pch_status ensure_pools(Workspace* ws, int sel_cap, int pool_cap, int req
             cudaMemcpy(nw.pool[p].src, w.pool[p].src, n * 4, cudaMemcpyDeviceToDevice);
             cudaMemcpy(nw.req[p], w.req[p], sizeof(FanReq) * (size_t)ws->req_cap, cudaMemcpyDeviceToDevice);
         }
+        const size_t na = (size_t)ws->arena_cap;
+        cudaMemcpy(nw.arena.he, w.arena.he, na * 4, cudaMemcpyDeviceToDevice);
+        cudaMemcpy(nw.arena.inst, w.arena.inst, na * 4, cudaMemcpyDeviceToDevice);
+        cudaMemcpy(nw.arena.src, w.arena.src, na * 4, cudaMemcpyDeviceToDevice);
+        cudaMemcpy(nw.arena.d, w.arena.d, na * 8, cudaMemcpyDeviceToDevice);
+        cudaMemcpy(nw.arena.A, w.arena.A, na * 8, cudaMemcpyDeviceToDevice);
+        cudaMemcpy(nw.arena.B, w.arena.B, na * 8, cudaMemcpyDeviceToDevice);
+        cudaMemcpy(nw.arena.px, w.arena.px, na * 8, cudaMemcpyDeviceToDevice);
+        cudaMemcpy(nw.arena.py, w.arena.py, na * 8, cudaMemcpyDeviceToDevice);
         e = cudaDeviceSynchronize();
         if (e) { dev_free(fresh); return set_error(PCH_ERR_CUDA, "pool growth copy: %s", cudaGetErrorString(e)); }
     }
@@ -1506,7 +1610,7 @@ static int grid_for(int blocks_per_sm) { return sm_count() * blocks_per_sm; }
 // Kernels one iteration launches (for pch_stats.kernel_launches).
 static int kernels_per_iteration(const SolveCfg& cfg) {
     int passes = (cfg.key_bits + kRsDigitBits - 1) / kRsDigitBits;
-    return 6 + (cfg.stride_T > 0 ? 1 : 0) + sort_kernels_per_pass() * passes;
+    return 4 + (cfg.append ? 1 : 0) + (cfg.stride_T > 0 ? 1 : 0) + sort_kernels_per_pass() * passes;
 }
 
 // Launch one iteration (all phases).  With `ev` (7 events) the phase boundaries are
@@ -1516,7 +1620,8 @@ static cudaError_t launch_iteration(Workspace* ws, cudaStream_t s, const SolveCf
     Work& w = ws->w;
     const int tpb = 256;
     if (ev) cudaEventRecord(ev[0], s);
-    k_tau<<<std::min(w.n_inst, 1024), 256, 0, s>>>(w, cfg.control, cfg.mlp);
+    k_ctrl<<<std::min(w.n_inst, 1024), kBins, 0, s>>>(w, cfg.control, cfg.mlp, h, use_cond, cfg.max_iters);
+    if (ev) cudaEventRecord(ev[1], s);
     if (cfg.stride_T > 0) {
         const int g = std::min((cfg.stride_T + 255) / 256, grid_for(8));
         switch (cfg.stride_m) {
@@ -1528,25 +1633,27 @@ static cudaError_t launch_iteration(Workspace* ws, cudaStream_t s, const SolveCf
         }
     }
     k_compact<<<grid_for(4), tpb, 0, s>>>(w);
-    if (ev) cudaEventRecord(ev[1], s);
+    if (ev) cudaEventRecord(ev[2], s);
     const dim3 pg(grid_for(cfg.prop_blocks_per_sm));
     const size_t psh = (size_t)cfg.prop_threads * kPropQueueBytesPerThread;
     if (cfg.prov) k_propagate<true><<<pg, cfg.prop_threads, psh, s>>>(w, cfg.hops, cfg.tail_cut, cfg.take_min);
     else k_propagate<false><<<pg, cfg.prop_threads, psh, s>>>(w, cfg.hops, cfg.tail_cut, cfg.take_min);
-    if (ev) cudaEventRecord(ev[2], s);
+    if (ev) cudaEventRecord(ev[3], s);
     if (cfg.prov) k_fan<true><<<grid_for(2), 256, 0, s>>>(w, cfg.full_fan);
     else k_fan<false><<<grid_for(2), 256, 0, s>>>(w, cfg.full_fan);
-    if (ev) cudaEventRecord(ev[3], s);
-    unsigned* kb[2] = {w.sort_key[0], w.sort_key[1]};
-    int* vb[2] = {w.sort_val[0], w.sort_val[1]};
-    const int par = cfg.key_bits == 0 ? -1 :
-        launch_sort_children(w.arena, w.inst, &w.cnt->n_child, w.arena_cap, cfg.key_bits, cfg.edge_sort, kb, vb, w.sort_hist,
-                                   w.sort_blocks, s);
     if (ev) cudaEventRecord(ev[4], s);
-    k_append<<<grid_for(4), tpb, 0, s>>>(w, par >= 0 ? kb[par] : nullptr, par >= 0 ? vb[par] : nullptr,
-                                          cfg.trim && cfg.edge_sort);
-    if (ev) cudaEventRecord(ev[5], s);
-    k_finish<<<1, 1, 0, s>>>(w, h, use_cond, cfg.max_iters);
+    if (cfg.append) {
+        unsigned* kb[2] = {w.sort_key[0], w.sort_key[1]};
+        int* vb[2] = {w.sort_val[0], w.sort_val[1]};
+        const int par = cfg.key_bits == 0 ? -1 :
+            launch_sort_children(w.arena, w.inst, &w.cnt->n_child, w.arena_cap, cfg.key_bits, kb, vb,
+                                 w.sort_hist, w.sort_blocks, s);
+        if (ev) cudaEventRecord(ev[5], s);
+        k_append<<<grid_for(4), tpb, 0, s>>>(w, par >= 0 ? kb[par] : nullptr, par >= 0 ? vb[par] : nullptr,
+                                             cfg.trim && cfg.edge_sort);
+    } else if (ev) {
+        cudaEventRecord(ev[5], s);
+    }
     if (ev) cudaEventRecord(ev[6], s);
     return cudaGetLastError();
 }
@@ -1615,15 +1722,17 @@ static pch_status run_solve(Workspace* ws, cudaStream_t s, const SolveCfg& cfg_i
             PCH_CUDA(cudaMemcpyAsync(ws->cnt_host, w.cnt, sizeof(Counters), cudaMemcpyDeviceToHost, s));
             PCH_CUDA(cudaStreamSynchronize(s));
             if (cfg.profile) {
+                // events in launch order: control, selection, propagation, fans, sort, append
+                constexpr int phase[6] = {5, 0, 1, 2, 3, 4};
                 for (int p = 0; p < 6; ++p) {
                     float ms = 0.f;
                     cudaEventElapsedTime(&ms, pev[p], pev[p + 1]);
-                    phase_ms[p] += ms;
+                    phase_ms[phase[p]] += ms;
                 }
             }
             const Counters& c = *ws->cnt_host;
             if (c.error || c.done) break;
-            if (c.n_pending + w.arena_cap > w.pool_cap) {
+            if (c.halt) {   // the pool has to grow
                 pch_status st = ensure_pools(ws, ws->sel_cap, 2 * ws->pool_cap);
                 if (st != PCH_OK) return st;
                 PCH_CUDA(cudaMemsetAsync(&w.cnt->halt, 0, sizeof(int), s));
@@ -1645,16 +1754,16 @@ static pch_status run_solve(Workspace* ws, cudaStream_t s, const SolveCfg& cfg_i
             PCH_CUDA(cudaMemcpyAsync(ws->cnt_host, w.cnt, sizeof(Counters), cudaMemcpyDeviceToHost, s));
             PCH_CUDA(cudaStreamSynchronize(s));
             const Counters& c = *ws->cnt_host;
-            // the WHILE body ran ceil(iterations / unroll) times
             if (c.error || c.done) break;
-            if (c.n_pending + w.arena_cap > w.pool_cap) {
+            if (c.halt) {   // the pool has to grow
                 pch_status st = ensure_pools(ws, ws->sel_cap, 2 * ws->pool_cap);
                 if (st != PCH_OK) return st;
                 PCH_CUDA(cudaMemsetAsync(&w.cnt->halt, 0, sizeof(int), s));
                 continue;
             }
         }
-        const long long it = ws->cnt_host->iter;
+        // (the control kernel that ends the loop is the first of one more iteration)
+        const long long it = ws->cnt_host->iter + 1;
         launches += ((it + cfg.unroll - 1) / cfg.unroll) * cfg.unroll * kernels_per_iteration(cfg);
     }
     if (cfg.loop == PCH_LOOP_HOST || cfg.profile) {
@@ -1712,18 +1821,17 @@ static SolveCfg make_cfg(const pch_options* opt, int n_inst, long long total_key
     cfg.tail_cut = default_tail_cut();
     cfg.take_min = default_take_min();
     cfg.unroll = 2;
-    // Step 3 organises the new windows into a gap-free pool; they are grouped by instance
-    // (one 8-bit radix pass for up to 256 instances, none for one), or with
-    // PCH_FLAG_EDGE_SORT ordered by (instance, half-edge) for the per-edge trimming
+    // Step 3 organises the new windows into a gap-free pool: the next iteration's compaction
+    // reads them from the arena, or with PCH_FLAG_EDGE_SORT they are ordered by (instance,
+    // half-edge) for the per-edge trimming and appended
     cfg.edge_sort = (opt && (opt->flags & PCH_FLAG_EDGE_SORT)) ? 1 : 0;
     int bits = 0;
     if (cfg.edge_sort) {
         bits = 1;
         while ((1LL << bits) <= total_keys) ++bits;   // invalid key ~0u must exceed all valid keys
-    } else {
-        while ((1LL << bits) < n_inst) ++bits;
     }
     cfg.key_bits = bits;
+    cfg.append = cfg.edge_sort || cfg.control == PCH_CONTROL_STRIDED;
     cfg.mlp = nullptr;
     cfg.stride_T = cfg.stride_m = 0;
     cfg.prov = 0;
@@ -1826,9 +1934,10 @@ pch_status solve_instances(pch_mesh* const* meshes, int n_inst, const SrcDev* sr
         kbase += dm.nh;
         I.lbar = dm.lbar; I.ilbar = 1.0 / dm.lbar;
         I.fbias = (unsigned)(1023 - 127 + std::ilogb(dm.lbar)) << 20;
+        I.ilbarf = (float)(1.0 / std::scalbn(dm.lbar, -std::ilogb(dm.lbar)));
         InstCtl& c = hctl[i];
         std::memset(&c, 0, sizeof c);
-        c.kmin = ~0ull;
+        c.kminf = ~0u;
         c.ref = 0.0;
         c.k_target = cfg.k;
         c.active = 1;
@@ -1846,6 +1955,7 @@ pch_status solve_instances(pch_mesh* const* meshes, int n_inst, const SrcDev* sr
     if (st != PCH_OK) return st;
     Work& w = ws->w;
     w.n_inst = n_inst;
+    w.append = cfg.append;
     if (cfg.stride_T > ws->sthr_cap) {
         drop_graph(ws);
         PCH_CUDA(cudaDeviceSynchronize());

@@ -20,7 +20,8 @@ struct SolveCfg {
     int prop_blocks_per_sm;
     int key_bits;
     int trim;
-    int edge_sort;          // sort new windows by (instance, half-edge) instead of by instance
+    int edge_sort;          // sort new windows by (instance, half-edge)
+    int append;             // new windows are appended to the pool at the end of the iteration (k_append)
     int unroll;
     int full_fan;
     int profile;

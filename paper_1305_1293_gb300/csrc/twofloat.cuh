@@ -31,6 +31,10 @@ __device__ __forceinline__ unsigned f_mag_bits(double x, unsigned bias) {
 __device__ __forceinline__ float f_of(double x, unsigned bias) {
     return __uint_as_float(f_mag_bits(x, bias) | ((unsigned)__double2hiint(x) & 0x80000000u));
 }
+// The double whose image these float bits are (exact; for images of nonnegative values).
+__device__ __forceinline__ double of_f_bits(unsigned f, unsigned bias) {
+    return f == 0u ? 0.0 : __hiloint2double((int)((f >> 3) + bias), (int)(f << 29));
+}
 // |x| scaled, as a two-float.
 __device__ __forceinline__ F2 f2_mag(double x, unsigned bias) {
     const unsigned f = f_mag_bits(x, bias);
