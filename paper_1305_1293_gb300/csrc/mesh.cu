@@ -3,6 +3,7 @@
 // boundary classification of Section 3.  Entry points pch_create_mesh, pch_mesh_info,
 // pch_destroy, pch_last_error.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -484,7 +485,6 @@ struct MeshTmp {
     int *twin, *vcount, *vout, *hvals, *counts, *scan_tmp, *tri_sorted, *fval[2], *fhist;
     unsigned* fkey[2];
     int* err;               // kMeshErr* flags
-    unsigned long long* bad; // first non-finite coordinate, first vertex id out of range
 };
 static void carve_tmp(Carver& c, MeshTmp& t, int nv, int nf, unsigned long long cap, bool reorder, int sort_blocks) {
     const int nh = 3 * nf;
@@ -499,7 +499,6 @@ static void carve_tmp(Carver& c, MeshTmp& t, int nv, int nf, unsigned long long 
     c.take(&t.counts, 2 + 2 * kStatBlocks);
     c.take(&t.scan_tmp, scan_tmp_ints(nv + 1));
     c.take(&t.err, 1);
-    c.take(&t.bad, 2);
     if (reorder) {
         c.take(&t.tri_sorted, nh);
         for (int j = 0; j < 2; ++j) {
@@ -511,14 +510,21 @@ static void carve_tmp(Carver& c, MeshTmp& t, int nv, int nf, unsigned long long 
     }
 }
 
-// First coordinate that is not finite and first vertex id out of range (~0: none).
-__global__ void k_check(int nv, int nf, const double* __restrict__ xyz, const int* __restrict__ tri,
-                        unsigned long long* bad) {
-    const long long n = max(3ll * nv, 3ll * nf);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        if (i < 3ll * nv && !(fabs(xyz[i]) <= 1.7976931348623157e308)) atomicMin(bad, (unsigned long long)i);
-        if (i < 3ll * nf && (unsigned)tri[i] >= (unsigned)nv) atomicMin(bad + 1, (unsigned long long)i);
+// Input checks (before any device work): one branch-free pass over each array, the index of
+// the first offender only when there is one.
+static bool all_finite(const double* x, long long n) {
+    unsigned long long bad = 0;
+    for (long long i = 0; i < n; ++i) {
+        unsigned long long b;
+        std::memcpy(&b, x + i, sizeof b);
+        bad |= ((b & 0x7fffffffffffffffull) + 0x0010000000000000ull) & 0x8000000000000000ull;   // exponent all ones
     }
+    return bad == 0;
+}
+static bool all_below(const int32_t* x, long long n, int32_t limit) {
+    unsigned most = 0;
+    for (long long i = 0; i < n; ++i) most = std::max(most, (unsigned)x[i]);
+    return most < (unsigned)limit;
 }
 
 void destroy_workspace(Workspace* w);   // solver.cu
@@ -535,6 +541,13 @@ extern "C" pch_status pch_create_mesh(const double* vertices, int32_t n_vertices
     if (!vertices || !faces || !out) return set_error(PCH_ERR_INVALID_ARG, "null pointer argument");
     if (n_vertices < 3 || n_faces < 1) return set_error(PCH_ERR_INVALID_ARG, "need >= 3 vertices and >= 1 face");
     if ((long long)n_faces * 3 >= (1LL << 31) - 1) return set_error(PCH_ERR_CAPACITY, "too many faces");
+    if (!all_finite(vertices, 3LL * n_vertices))
+        for (long long i = 0; i < 3LL * n_vertices; ++i)
+            if (!std::isfinite(vertices[i])) return set_error(PCH_ERR_INVALID_ARG, "non-finite coordinate at vertex %lld", i / 3);
+    if (!all_below(faces, 3LL * n_faces, n_vertices))
+        for (long long i = 0; i < 3LL * n_faces; ++i)
+            if (faces[i] < 0 || faces[i] >= n_vertices)
+                return set_error(PCH_ERR_INVALID_ARG, "face %lld references vertex %d out of range", i / 3, faces[i]);
 
     const int nv = n_vertices, nf = n_faces, nh = 3 * n_faces;
     const bool reorder = nf >= kReorderFaces;
@@ -549,7 +562,6 @@ extern "C" pch_status pch_create_mesh(const double* vertices, int32_t n_vertices
     void* tmp = nullptr;
     pch_status st = PCH_OK;
     int herr = 0;
-    unsigned long long hbad[2] = {~0ull, ~0ull};
     double hl = 0.0;
     int hc[2] = {0, 0};
     auto fail = [&](pch_status s) { st = s; };
@@ -574,7 +586,6 @@ extern "C" pch_status pch_create_mesh(const double* vertices, int32_t n_vertices
         carve_tmp(ct, t, nv, nf, cap, reorder, sort_blocks);
         MCHK(cudaMemcpyAsync(t.xyz, vertices, sizeof(double) * 3 * nv, cudaMemcpyHostToDevice, s));
         MCHK(cudaMemcpyAsync(d.tri, faces, sizeof(int) * nh, cudaMemcpyHostToDevice, s));
-        MCHK(cudaMemsetAsync(t.bad, 0xff, sizeof(unsigned long long) * 2, s));
         MCHK(cudaMemsetAsync(t.err, 0, sizeof(int), s));
         MCHK(cudaMemsetAsync(t.vcount, 0, sizeof(int) * (nv + 1), s));
         MCHK(cudaMemsetAsync(t.vout, 0x7f, sizeof(int) * nv, s));
@@ -582,18 +593,6 @@ extern "C" pch_status pch_create_mesh(const double* vertices, int32_t n_vertices
         const int tb = 256;
         const int gb = std::max(1, std::min((nh + tb - 1) / tb, sm_count() * 8));
         const int gv = std::max(1, std::min((nv + tb - 1) / tb, sm_count() * 8));
-        k_check<<<std::max(gb, gv), tb, 0, s>>>(nv, nf, t.xyz, d.tri, t.bad);
-        MCHK(cudaMemcpyAsync(hbad, t.bad, sizeof hbad, cudaMemcpyDeviceToHost, s));
-        MCHK(cudaStreamSynchronize(s));
-        if (hbad[0] != ~0ull) {
-            fail(set_error(PCH_ERR_INVALID_ARG, "non-finite coordinate at vertex %lld", (long long)hbad[0] / 3));
-            goto cleanup;
-        }
-        if (hbad[1] != ~0ull) {
-            fail(set_error(PCH_ERR_INVALID_ARG, "face %lld references vertex %d out of range", (long long)hbad[1] / 3,
-                           faces[hbad[1]]));
-            goto cleanup;
-        }
         const int* tri = d.tri;
         if (reorder) {
             MCHK(cudaMemsetAsync(t.box, 0x7f, sizeof(long long) * 6, s));
