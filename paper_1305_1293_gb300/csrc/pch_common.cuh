@@ -109,7 +109,7 @@ struct Inst {
     unsigned long long* ang;    // angle_split[]: packed (rounded-up distance, crossing position)
     unsigned* stamp;            // per-vertex iteration stamp (one fan request per iteration)
     float* fan_phi;             // per-vertex angular position of the incoming ray of its last fan
-    double2* fan_dir;           // per-vertex unit incoming direction of its last fan (angular frame)
+    double2* fan_dir;           // per-vertex incoming direction of its last fan (angular frame, any length)
     int nv, nh;
     long long keybase;          // sort key = keybase + half-edge
     double lbar;

@@ -225,20 +225,13 @@ __device__ __forceinline__ void stats_add(const Work& w, PoolStats& ps, unsigned
         }
     }
 }
-// A window just written to the arena (the lanes that wrote one).
-__device__ __forceinline__ void stats_created(const Work& w, unsigned* g_hist, int inst, float key) {
-    atomicAdd(&g_hist[inst * kBins + hist_bin((key - w.ctl[inst].reff) * w.inst[inst].ilbarf)], 1u);
-    const unsigned m = __activemask();
-    if (w.n_inst == 1) {
-        const unsigned mn = __reduce_min_sync(m, __float_as_uint(key));
-        if ((threadIdx.x & 31) == __ffs(m) - 1) {
-            atomicMin(&w.ctl[0].kminf, mn);
-            atomicAdd(&w.ctl[0].n_next, __popc(m));
-        }
-    } else {
-        atomicMin(&w.ctl[inst].kminf, __float_as_uint(key));
-        atomicAdd(&w.ctl[inst].n_next, 1);
-    }
+// One window of a single lane.
+__device__ __forceinline__ void stats_lane(const Work& w, PoolStats& ps, unsigned* g_hist, int inst, float key) {
+    const bool shared = w.n_inst <= kShHistInst;
+    const int slot = inst * kBins + hist_bin((key - w.ctl[inst].reff) * w.inst[inst].ilbarf);
+    atomicAdd(shared ? &ps.hist[slot] : &g_hist[slot], 1u);
+    atomicMin(shared ? &ps.kminf[inst] : &w.ctl[inst].kminf, __float_as_uint(key));
+    atomicAdd(shared ? &ps.n[inst] : &w.ctl[inst].n_next, 1);
 }
 
 // A pool window.  `inst` is the instance without the pending-event bits, `pend` those bits.
@@ -322,7 +315,11 @@ __global__ void k_init_sources(Work w, const SrcDev* __restrict__ srcs, int n_sr
                 store_win(w.arena, slot, {R.twin, s.inst, -1 - s.label, kPendA | kPendB, 0.0, 0.0, R.L, px, py, 0.0});
                 if (!w.append) {
                     const float fx = f_of(px < 0.0 ? px : (px > R.L ? px - R.L : 0.0), I.fbias), fy = f_of(py, I.fbias);
-                    stats_created(w, w.hist[0], s.inst, sqrtf(fmaf(fx, fx, fy * fy)));
+                    const float key = sqrtf(fmaf(fx, fx, fy * fy));
+                    InstCtl& c = w.ctl[s.inst];
+                    atomicAdd(&w.hist[0][s.inst * kBins + hist_bin(key * I.ilbarf)], 1u);
+                    atomicMin(&c.kminf, __float_as_uint(key));
+                    atomicAdd(&c.n_next, 1);
                 }
             }
         }
@@ -1037,35 +1034,45 @@ __device__ __forceinline__ double2 cmul_conj(double2 a, double2 b) {   // a * co
     return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.y, b.x, -a.x * b.y));
 }
 
+// x clamped to [0, L] on the integer images (a NaN: `nan`).
+__device__ __forceinline__ double clamp_s(double x, double L, double nan) {
+    return sbits(x) < 0 ? 0.0 : (lt_s(L, x) ? (sbits(x) > 0x7ff0000000000000ll ? nan : L) : x);
+}
+
 // Where the ray from the apex v of o's face along z (relative to the direction
 // v -> start(o), any length) meets o: distance from start(o), clamped to [0, L].
 __device__ __forceinline__ double fan_hit(const HERec& Ro, double2 z) {
     const double ux = -Ro.u2x, uy = -Ro.u2y;                   // v -> start(o), unit
     const double dx = fma(ux, z.x, -uy * z.y), dy = fma(ux, z.y, uy * z.x);
-    if (!(dy < 0.0)) return dx > 0.0 ? Ro.L : 0.0;             // parallel to o or turned away
-    const double s = fma(-Ro.yc * dx, rcp_nr(dy), Ro.xc);
-    return s < 0.0 ? 0.0 : (s > Ro.L ? Ro.L : s);
+    if (!(sbits(dy) < 0 && sbits(dy) != (long long)0x8000000000000000ull)) return gt0_s(dx) ? Ro.L : 0.0;   // parallel to o or turned away
+    return clamp_s(fma(-Ro.yc * dx, rcp_nr(dy), Ro.xc), Ro.L, __longlong_as_double(0x7ff8000000000000ll));
 }
 
+// Bound by latency (a few thousand candidates an iteration, dependent loads and FP64
+// instructions of 64 cycles): the new windows are filtered in FP32 before their slots are
+// reserved, directions keep their length, and the statistics are collected in shared memory
+// (per window, global atomics on an instance's few words took a third of the kernel). 24 uneven
+// meshes, 4.3M fan windows: 32.9 -> 29.9 ms a call.
 // kFanLanes lanes per fan candidate; lane j of the group handles corners j, j + 8, ...
 // of the vertex's one-ring.  PROV: also record the distance events (geodesic paths).
 template <bool PROV>
 __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
     Counters* cnt = w.cnt;
     if (cnt->halt) return;
+    const int nreq = min(cnt->n_req, w.req_cap), n_prop = min(cnt->n_child, w.arena_cap);
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&cnt->fan_cand, (unsigned long long)nreq);
+    if (blockIdx.x * blockDim.x >= max(n_prop, nreq * kFanLanes)) return;
     // first the selection statistics of the windows that the propagation created (here, where
     // the GPU has little else to do: from inside the propagation kernel they cost 8% of it)
     __shared__ PoolStats ps;
-    const int n_prop = min(cnt->n_child, w.arena_cap);
-    if (!w.append && blockIdx.x * blockDim.x < n_prop) {
-        unsigned* g_hist = w.hist[(cnt->iter + 1) & 1];
+    unsigned* g_hist = w.hist[(cnt->iter + 1) & 1];
+    if (!w.append) {
         stats_begin(ps, w.n_inst);
         for (int base = blockIdx.x * blockDim.x; base < n_prop; base += gridDim.x * blockDim.x) {
             const int i = base + threadIdx.x;
             const bool on = i < n_prop;
             stats_add(w, ps, g_hist, on ? w.arena.inst[i] & kInstMask : 0, on ? w.arena.keyf[i] : 0.f, on);
         }
-        stats_end(w, ps, g_hist);
     }
     const int lane = threadIdx.x & 31;
     const int sl = lane & (kFanLanes - 1);
@@ -1073,8 +1080,6 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
     const unsigned gmask = ((1u << kFanLanes) - 1u) << lead;
     const unsigned below = (1u << sl) - 1u;
     const int it = cnt->iter;
-    const int nreq = min(cnt->n_req, w.req_cap);
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&cnt->fan_cand, (unsigned long long)nreq);
     const FanReq* req = w.req[it & 1];
     FanReq* req_nx = w.req[(it + 1) & 1];
     const unsigned stamp_fan = (unsigned)it + 1u;
@@ -1086,6 +1091,12 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
         const unsigned v = rq.v;
         const double D = rq.D;
         const Inst& I = w.inst[rq.inst];
+        // (the vertex's data is loaded before the answer of the candidate's test below arrives)
+        const int hr = max(rq.href, 0);
+        const int s = I.vstart[v], e = I.vstart[v + 1];
+        const unsigned char vflag = I.vflag[v];
+        const float T = I.vtheta[v], phi_ref = I.vphi[hr];
+        const double2 rot_ref = I.vrot[hr], rot_v = I.vtrot[v];
         // 1: the iteration's fan of the vertex (a candidate from an event that lowered its
         // distance, carrying its final distance, the first this iteration); 2: a tie
         // deferred an iteration, fanned if its direction is new; 0: superseded, or
@@ -1105,14 +1116,12 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
         }
         kind = __shfl_sync(gmask, kind, lead);
         if (!kind) continue;
-        const int s = I.vstart[v], e = I.vstart[v + 1];
-        const bool boundary = (I.vflag[v] & 1) != 0;
+        const bool boundary = (vflag & 1) != 0;
         const bool all = full_fan != 0 || rq.href < 0;
         if (all && kind == 2) continue;            // a fan of every direction was made already
         // wedges in FP32 angular coordinates, unwrapped (interior ones are tested at
         // shifts of the total angle T): interior [phi + pi, phi + T - pi]; boundary
         // [-inf, phi - pi] and [phi + pi, +inf]
-        const float T = I.vtheta[v];
         double2 za = make_double2(0.0, 0.0), zb = za, tr = make_double2(1.0, 0.0), zlo = za, zhi = za, tie_z = za;
         bool tie_lo = false, tie_hi = false;       // a tie's wedge cut to the part outside the last fan's
         float tie_w = 0.f;
@@ -1120,19 +1129,18 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
         float wlo[2] = {0.f, 0.f}, whi[2] = {0.f, 0.f};
         bool lo_open[2] = {false, false}, hi_open[2] = {false, false};
         if (!all) {
-            float phi = I.vphi[rq.href] + atan2f((float)rq.dy, (float)rq.dx);
+            float phi = phi_ref + atan2f((float)rq.dy, (float)rq.dx);
             // the incoming ray in the vertex's angular frame, turned by pi: the direction of
             // phi + pi (and of phi - pi); zb is that of phi + T - pi
-            const double2 E = cmul(I.vrot[rq.href], make_double2(rq.dx, rq.dy));
+            const double2 E = cmul(rot_ref, make_double2(rq.dx, rq.dy));
             za = make_double2(-E.x, -E.y);
-            tr = I.vtrot[v];
+            tr = rot_v;
             zb = cmul(za, tr);
             if (boundary) phi = fminf(fmaxf(phi, 0.f), T);
-            // the unit incoming direction and its angular position on the sheet [0, T) of an
-            // interior vertex (positions phi and phi + T are one direction; their unit numbers
-            // differ by the turn e^(i T), which is not 1 at a saddle)
-            const double en_s = rsqrt(fma(E.x, E.x, E.y * E.y));
-            double2 en = make_double2(E.x * en_s, E.y * en_s);
+            // the incoming direction (of any length) and its angular position on the sheet
+            // [0, T) of an interior vertex (positions phi and phi + T are one direction; their
+            // numbers differ by the turn e^(i T), which is not 1 at a saddle)
+            double2 en = E;
             float phic = phi;
             int kc = 0;
             if (!boundary) {
@@ -1156,7 +1164,8 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
                     const int sh = boundary ? 0 : (int)rintf((phic - fp) / T);
                     double2 ea = en;
                     for (int q = 0; q < abs(sh) && q < 3; ++q) ea = sh > 0 ? cmul_conj(ea, tr) : cmul(ea, tr);
-                    if (fma(ea.x, fd.x, ea.y * fd.y) > 0.0 && fabs(fma(ea.x, fd.y, -ea.y * fd.x)) <= kTieDir) continue;
+                    const double along = fma(ea.x, fd.x, ea.y * fd.y);
+                    if (along > 0.0 && fabs(fma(ea.x, fd.y, -ea.y * fd.x)) <= kTieDir * along) continue;
                 }
                 if (sl == 0) atomicAdd(&cnt->fan_ties, 1ull);
                 // at an interior saddle whose two fanned areas overlap, only the part of this
@@ -1241,12 +1250,32 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
                         else if (shift == -1) t = make_double2(tr.x, -tr.y);
                         else if (shift == -2) t = cmul_conj(make_double2(tr.x, -tr.y), tr);
                         const double2 cr = I.vrot[hv];
-                        if (ex0) s0 = fmax(fan_hit(Ro, cmul_conj(cmul(zlo, t), cr)) - kFanWiden * Ro.L, 0.0);
-                        if (ex1) s1 = fmin(fan_hit(Ro, cmul_conj(cmul(zhi, t), cr)) + kFanWiden * Ro.L, Ro.L);
+                        if (ex0) s0 = clamp_s(fan_hit(Ro, cmul_conj(cmul(zlo, t), cr)) - kFanWiden * Ro.L, Ro.L, 0.0);
+                        if (ex1) s1 = clamp_s(fan_hit(Ro, cmul_conj(cmul(zhi, t), cr)) + kFanWiden * Ro.L, Ro.L, Ro.L);
                     }
                 }
             }
-            const bool win = has && Ro.twin >= 0;
+            // window on twin(o) = (b -> a): I = v at (L - xc, -yc), interval [L - s1, L - s0],
+            // if it is not narrower than 2^-40 of the edge and the paths via a and b do not beat
+            // it (FP32 with margins, as the propagation's filters)
+            bool win = has && Ro.twin >= 0;
+            Win W{};
+            float keyf = 0.f;
+            if (win) {
+                const unsigned fb = I.fbias;
+                const double ga = ldg_dist(I.g, Ro.v0 & ~kPseudoBit), gb = ldg_dist(I.g, Ro.v1 & ~kPseudoBit);
+                const double px = Ro.L - Ro.xc, py = -Ro.yc;
+                W = {Ro.twin, rq.inst, (int)v, kPendA | kPendB, D, Ro.L - s1, Ro.L - s0, px, py, 0.0};
+                const double ax = W.A - px, bx = W.B - px;
+                const F2 df = f2_mag(D, fb), yf = f2_mag(py, fb), yy = f2_sq(yf);
+                const F2 lenA = f2_hyp(f2_mag(ax, fb), yy), lenB = f2_hyp(f2_mag(bx, fb), yy);
+                const float Lf = f_of(Ro.L, fb);
+                const float mrg = fmaf(df.h + fmaxf(lenA.h, lenB.h), kDomF, Lf * kLocalF);
+                win = lt_s(times_eps(Ro.L), W.B - W.A) &&
+                      !(f2_add_f(f2_sub(df, f2_mag(gb, fb)), lenB) > f_of(W.B, fb) + mrg ||
+                        f2_add_f(f2_sub(df, f2_mag(ga, fb)), lenA) > (Lf - f_of(W.A, fb)) + mrg);
+                keyf = df.h + (gt0_s(ax) ? lenA.h : (sbits(bx) < 0 ? lenB.h : yf.h));
+            }
             const unsigned bal = (__ballot_sync(gmask, win) >> lead) & ((1u << kFanLanes) - 1u);
             const int cntw = __popc(bal);
             int base = 0;
@@ -1264,9 +1293,11 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
                 deferred = true;
                 continue;
             }
-            if (!has) continue;
-            const double Lo = Ro.L;
-            if (!win) {
+            if (win) {
+                store_win(w.arena, base + __popc(bal & below), W);
+                if (!w.append) stats_lane(w, ps, g_hist, rq.inst, keyf);
+                ++n_fwin;
+            } else if (has && Ro.twin < 0) {
                 // boundary edge: endpoint events for the covered endpoints
                 const unsigned a = Ro.v0 & ~kPseudoBit, b = Ro.v1 & ~kPseudoBit;
                 double ga = ldg_dist(I.g, a), gb = ldg_dist(I.g, b);
@@ -1275,32 +1306,17 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
                 if (s0 <= 0.0)
                     if (const int ev = vertex_event<PROV>(I, Ro.v0, D + Ro.L2, ga, &w, &es))
                         push_fan(req_nx, &cnt->n_req_next, w.req_cap, &cnt->error, rq.inst, a, D + Ro.L2, o, Ro.xc, Ro.yc, ev);
-                if (s1 >= Lo)
+                if (s1 >= Ro.L)
                     if (const int ev = vertex_event<PROV>(I, Ro.v1, D + Ro.L1, gb, &w, &es))
                         push_fan(req_nx, &cnt->n_req_next, w.req_cap, &cnt->error, rq.inst, b, D + Ro.L1, he_next(o), 1.0,
                                  0.0, ev);
-                continue;
             }
-            // window on twin(o) = (b -> a): I = v at (Lo - xc, -yc), interval [Lo - s1, Lo - s0]
-            const int slot = base + __popc(bal & below);
-            const double A = Lo - s1, B = Lo - s0;
-            const double px = Lo - Ro.xc, py = -Ro.yc;
-            const double IA = sqrt_nr(fma(A - px, A - px, py * py)), IB = sqrt_nr(fma(B - px, B - px, py * py));
-            const double ga = ldg_dist(I.g, Ro.v0 & ~kPseudoBit), gb = ldg_dist(I.g, Ro.v1 & ~kPseudoBit);
-            if (!(B - A > times_eps(Lo)) || dominated(D + IB, gb + B) || dominated(D + IA, ga + (Lo - A))) {
-                w.arena.he[slot] = -1;
-                continue;
-            }
-            store_win(w.arena, slot, {Ro.twin, rq.inst, (int)v, kPendA | kPendB, D, A, B, px, py, 0.0});
-            if (!w.append)
-                stats_created(w, w.hist[(it + 1) & 1], rq.inst,
-                              f_of(D + (px < A ? IA : (px > B ? IB : -py)), I.fbias));
-            ++n_fwin;
         }
     }
     const unsigned f1 = __reduce_add_sync(0xffffffffu, n_fans), f2 = __reduce_add_sync(0xffffffffu, n_fwin);
     if (lane == 0 && f1) atomicAdd(&cnt->fans, (unsigned long long)f1);
     if (lane == 0 && f2) atomicAdd(&cnt->fan_windows, (unsigned long long)f2);
+    if (!w.append) stats_end(w, ps, g_hist);
 }
 
 // ====================================================================== Step 3/4: append
