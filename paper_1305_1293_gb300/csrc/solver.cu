@@ -132,16 +132,24 @@ __device__ __forceinline__ int vertex_event(const Inst& I, unsigned vf, double D
                                             const Work* w = nullptr, const EvSrc* es = nullptr) {
     const bool pseudo = (vf & kPseudoBit) != 0;
     if (!lt_s(D, gcache)) return pseudo && dbits(D) <= dbits(gcache) + kDomUlps ? kReqTie : kEvNone;
-    unsigned v = vf & ~kPseudoBit;
-    unsigned long long nb = dbits(D);
-    unsigned long long old = atomicMin(I.g + v, nb);
-    if (nb < old) {
-        if constexpr (PROV) log_event(*w, *es, v, nb);
+    const unsigned v = vf & ~kPseudoBit;
+    const unsigned long long nb = dbits(D);
+    if constexpr (PROV) {
+        const unsigned long long old = atomicMin(I.g + v, nb);
+        if (nb < old) {
+            log_event(*w, *es, v, nb);
+            gcache = D;
+            return pseudo ? kReqLowered : kEvNone;
+        }
+        gcache = bitsd(old);
+        return pseudo && nb <= old + kDomUlps ? kReqTie : kEvNone;
+    } else {
+        // without waiting for the atomic's answer: an event that another one has beaten since
+        // g was read makes a candidate that k_fan compares with the final distance
+        atomicMin(I.g + v, nb);
         gcache = D;
         return pseudo ? kReqLowered : kEvNone;
     }
-    gcache = bitsd(old);
-    return pseudo && nb <= old + kDomUlps ? kReqTie : kEvNone;
 }
 
 // A fan candidate carries the incoming ray as a direction (dx, dy), of any length, in
@@ -624,6 +632,59 @@ __device__ __forceinline__ double ray_hit(double m, double dx, double ux, double
 constexpr float kDomF = 1.3e-12f;
 constexpr float kLocalF = 0x1p-20f;
 
+// A warp's shared memory in the propagation kernel: the queue of the windows of its next
+// round (one a lane; a round reads its entries before it writes the next round's), and fan
+// candidates on their way to the request list, so that no round waits for the slot of one.
+constexpr int kFanBuf = 16;
+constexpr int kChildBuf = 8;
+struct WarpMem {
+    double d[32], A[32], px[32], py[32], ax[32];
+    union {
+        struct {
+            double B[32], bx[32];
+        };
+        struct {                            // pairs of lanes (propagate_pairs) keep one end a lane:
+            double d[kChildBuf], A[kChildBuf], B[kChildBuf], px[kChildBuf], py[kChildBuf];
+            int he[kChildBuf], inst[kChildBuf], src[kChildBuf];
+            float key[kChildBuf];
+        } child;                            // here children on their way to the arena
+    };
+    int he[32], inst[32], src[32], hop[32];
+    FanReq fan[kFanBuf];
+    int n_fan, pad[7];
+};
+static_assert(sizeof(WarpMem) == 72 * 32 + kFanBuf * sizeof(FanReq) + 32 && sizeof(WarpMem) % 16 == 0, "layout");
+constexpr int kPropSmemBytesPerThread = (int)sizeof(WarpMem) / 32;
+static_assert(sizeof(WarpMem) % 32 == 0, "bytes a thread");
+
+__device__ __forceinline__ void queue_fan(const Work& w, Counters* cnt, FanReq* req, WarpMem& m, int inst, unsigned v, double D,
+                                          int href, double dx, double dy, int tie) {
+    const int slot = atomicAdd(&m.n_fan, 1);
+    if (slot < kFanBuf) {
+        FanReq r;
+        r.inst = inst; r.v = v; r.href = href; r.tie = tie; r.D = D; r.dx = dx; r.dy = dy;
+        m.fan[slot] = r;
+    } else {
+        push_fan(req, &cnt->n_req, w.req_cap, &cnt->error, inst, v, D, href, dx, dy, tie);
+    }
+}
+// (whole warp) The buffered candidates to the request list.
+__device__ __forceinline__ void flush_fans(const Work& w, Counters* cnt, FanReq* req, WarpMem& m) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    const int n = min(m.n_fan, kFanBuf);
+    int base = 0;
+    if (lane == 0 && n) base = atomicAdd(&cnt->n_req, n);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (lane < n) {
+        if (base + lane < w.req_cap) req[base + lane] = m.fan[lane];
+        else atomicOr(&cnt->error, kErrReqFull);
+    }
+    __syncwarp();
+    if (lane == 0) m.n_fan = 0;
+    __syncwarp();
+}
+
 // Algorithm 2 for one window: events, one angle one split, the child with the Xin-Wang
 // filter.  A window with two children computes the right one and asks for the left one
 // to be deferred (`defer`): each lane computes one child a round.  Returns whether the
@@ -640,7 +701,7 @@ constexpr float kLocalF = 0x1p-20f;
 // it in FP64, 62 instructions a window, eight fields on the 327,680-face sphere took
 // 86.1 ms and take 39.2, the 1M-face torus 49.3 and 22.5.
 template <bool PROV>
-__device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, FanReq* req, const LaneWin& W,
+__device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, FanReq* req, WarpMem& m, const LaneWin& W,
                                                  ChildOut& c, bool& has_child, bool& defer, bool& occ, bool& comp) {
     has_child = defer = occ = comp = false;
     const Inst& I = w.inst[W.inst];
@@ -682,13 +743,13 @@ __device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, F
             if ((W.pend & kPendA) && le_s(A, tol)) {
                 const double D0 = d + sqrt_nr(fma(px, px, py2));
                 if (const int ev = vertex_event<PROV>(I, R.v0, D0, g0, &w, &es))   // the ray arrives at v0 from I (h's frame)
-                    push_fan(req, &cnt->n_req, w.req_cap, &cnt->error, W.inst, R.v0 & ~kPseudoBit, D0, W.h, px, py, ev);
+                    queue_fan(w, cnt, req, m, W.inst, R.v0 & ~kPseudoBit, D0, W.h, px, py, ev);
             }
             if ((W.pend & kPendB) && sbits(L) - sbits(B) <= kSnapUlps) {
                 const double q = L - px;
                 const double D1 = d + sqrt_nr(fma(q, q, py2));
                 if (const int ev = vertex_event<PROV>(I, R.v1, D1, g1, &w, &es))   // at v1, in the frame of twin(h) = (v1 -> v0)
-                    push_fan(req, &cnt->n_req, w.req_cap, &cnt->error, W.inst, R.v1 & ~kPseudoBit, D1, R.twin, q, -py, ev);
+                    queue_fan(w, cnt, req, m, W.inst, R.v1 & ~kPseudoBit, D1, R.twin, q, -py, ev);
             }
         }
         // occupancy of v2: the ray I -> v2 crosses e at xs; xs < A exactly when
@@ -741,7 +802,7 @@ __device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, F
                 // prev(h) = (v2 -> v0), whose axis is (-xc, -yc) / L2
                 const int hp = 3 * (W.h / 3) + (W.h % 3 + 2) % 3;
                 const double ux = -R.u2x, uy = -R.u2y, ex = px - R.xc, ey = py - R.yc;
-                push_fan(req, &cnt->n_req, w.req_cap, &cnt->error, W.inst, R.v2 & ~kPseudoBit, D2, hp,
+                queue_fan(w, cnt, req, m, W.inst, R.v2 & ~kPseudoBit, D2, hp,
                          ex * ux + ey * uy, ux * ey - uy * ex, ev);
             }
             if (near_end) {
@@ -824,10 +885,335 @@ __device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, F
     return prop;
 }
 
-// Windows in flight per warp: the shared-memory queue of chained children holds at most
-// one window per lane, 7 doubles and 4 ints an entry.  A round reads its entries before
-// it writes the next round's, so one buffer serves both.
-constexpr int kPropQueueBytesPerThread = 7 * 8 + 4 * 4;
+// ---------------------------------------------------------------- sparse lists: pairs of lanes
+// The same rounds with two lanes a window, for iterations whose selected list leaves most
+// lanes empty (a small mesh, a ring-shaped frontier).  A round is then bound by one warp's
+// latency: an FP64 instruction takes 64 cycles there however many lanes are active, so
+// the even lane computes what belongs to the window's end A and the odd lane what belongs to
+// B (the ray, the length, the tests at that end; of the frame change one component each): 11
+// FP64 instructions instead of 21, and half the FP32 ones.  A left child is handed to a free
+// pair within the round; no atomic's answer is waited for (fan candidates and children pass
+// through shared memory).  Chosen when at most kPairQuota windows a resident warp are
+// selected, half a warp: lists of 16 a warp still run faster in pairs (terrain 512 x 512 7.89
+// -> 7.54 ms; with lines at 4 and 8 a warp 7.69 and 7.62), longer ones fill whole warps.
+// 187 x 331 grid 4.50 -> 3.77 ms, 64 sources on 100,820 faces 2.66 -> 2.31, Voronoi labels
+// on 327,680 faces 10.5 -> 9.1, 5,120 faces 1.31 -> 1.21.
+constexpr int kPairQuota = 16;
+constexpr unsigned kPairLanes = 0x55555555u;        // the even lane of every pair
+
+// One lane's share of a window: its end e (A or B) and ex = e - px.
+struct PairWin {
+    int h, inst, src, hop;
+    bool task, pend;
+    double d, e, px, py, ex;
+};
+
+__device__ __forceinline__ double shfl_other(double x) { return __shfl_xor_sync(0xffffffffu, x, 1); }
+
+__device__ __forceinline__ void pair_put(WarpMem& m, int at, const PairWin& W, int hop) {
+    m.he[at] = W.h; m.inst[at] = W.inst; m.src[at] = W.src; m.hop[at] = hop;
+    m.d[at] = W.d; m.A[at] = W.e; m.px[at] = W.px; m.py[at] = W.py; m.ax[at] = W.ex;
+}
+__device__ __forceinline__ void pair_get(const WarpMem& m, int at, PairWin& W) {
+    const int hop = m.hop[at];
+    W.h = m.he[at]; W.inst = m.inst[at]; W.src = m.src[at];
+    W.task = (hop & kHopTask) != 0;
+    W.pend = (hop >> kHopPend & 1) != 0;
+    W.hop = hop & kHopMask;
+    W.d = m.d[at]; W.e = m.A[at]; W.px = m.px[at]; W.py = m.py[at]; W.ex = m.ax[at];
+}
+
+// (whole warp) The buffered children to the arena; returns its fill after them.
+__device__ __forceinline__ int flush_children(const Work& w, Counters* cnt, const WarpMem& m, int n) {
+    const int lane = threadIdx.x & 31;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(&cnt->n_child, n);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    const int slot = base + lane;
+    if (lane < n && slot < w.arena_cap) {
+        w.arena.he[slot] = m.child.he[lane]; w.arena.inst[slot] = m.child.inst[lane]; w.arena.src[slot] = m.child.src[lane];
+        w.arena.d[slot] = m.child.d[lane]; w.arena.A[slot] = m.child.A[lane]; w.arena.B[slot] = m.child.B[lane];
+        w.arena.px[slot] = m.child.px[lane]; w.arena.py[slot] = m.child.py[lane]; w.arena.keyf[slot] = m.child.key[lane];
+    } else if (lane < n) {
+        atomicOr(&cnt->error, kErrPoolFull);
+    }
+    __syncwarp();
+    return base + n;
+}
+
+template <bool PROV>
+__device__ __forceinline__ void propagate_pairs(const Work& w, Counters* cnt, FanReq* req, WarpMem& m, int n,
+                                                int quota, int room, int hops, int tail_cut) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, slot = lane >> 1, even = lane & ~1;
+    const bool end_b = (lane & 1) != 0;
+    const unsigned before = ((1u << even) - 1u) & kPairLanes;
+    int seen_child = *(volatile int*)&cnt->n_child;
+    unsigned n_prop = 0, n_chain = 0, n_exam = 0, n_occ = 0, n_comp = 0, n_ray = 0;
+    bool dry = false;
+    int nq = 0, nout = 0;                               // queued windows, children held back
+    for (;;) {
+        PairWin W;
+        bool have = slot < nq;
+        W.h = W.inst = W.hop = 0;
+        W.src = -1;
+        W.task = W.pend = false;
+        W.d = W.e = W.px = W.py = W.ex = 0.0;
+        if (have) pair_get(m, lane, W);
+        if (nq < quota && !dry) {
+            int base = 0;
+            if (lane == 0) base = atomicAdd(&cnt->work_next, quota - nq);
+            base = __shfl_sync(full, base, 0);
+            if (base + quota - nq >= n) dry = true;
+            const int idx = base + slot - nq;
+            if (slot >= nq && slot < quota && idx < n) {
+                const int fi = w.sel.inst[idx];
+                W.h = w.sel.he[idx]; W.src = w.sel.src[idx]; W.d = w.sel.d[idx];
+                W.e = end_b ? w.sel.B[idx] : w.sel.A[idx];
+                W.px = w.sel.px[idx]; W.py = w.sel.py[idx];
+                W.inst = fi & kInstMask;
+                W.pend = ((unsigned)fi & (end_b ? kPendB : kPendA)) != 0;
+                W.ex = W.e - W.px;
+                have = true;
+            }
+        }
+        const unsigned live = __ballot_sync(full, have) & kPairLanes;
+        if (!live) {
+            if (nout) flush_children(w, cnt, m, nout);
+            flush_fans(w, cnt, req, m);
+            const unsigned long long sums[6] = {n_prop, n_chain, n_exam, n_occ, n_comp, n_ray};
+            unsigned long long* dst[6] = {&cnt->propagated, &cnt->chained, &cnt->examined, &cnt->occupied,
+                                          &cnt->children, &cnt->rays};
+            if (lane == 0)
+                for (int j = 0; j < 6; ++j)
+                    if (sums[j]) atomicAdd(dst[j], sums[j]);
+            break;
+        }
+        __syncwarp();                                   // every lane has read its entry
+        // ---- the window's own part (as propagate_window's; a pair decides as one)
+        const unsigned own = __ballot_sync(full, have && !W.task);
+        const bool mine = have && !W.task;
+        const Inst* Ip = w.inst + W.inst;
+        HERec R = Ip->rec[W.h];
+        double g0 = ldg_dist(Ip->g, R.v0 & ~kPseudoBit);
+        double g1 = ldg_dist(Ip->g, R.v1 & ~kPseudoBit);
+        double g2 = ldg_dist(Ip->g, R.v2 & ~kPseudoBit);
+        bool stale = mine && stale_source(*Ip, W.src, W.d);
+        unsigned long long aw = kEmptyAngle;
+        if (mine) aw = __ldcg(Ip->ang + W.h);
+        bool left = false, right = false, occ = false, prop = mine;
+        {
+            const unsigned fb = Ip->fbias;
+            const float Lf = f_of(R.L, fb), xcf = f_of(R.xc, fb), ycf = f_of(R.yc, fb), ef = f_of(W.e, fb);
+            if (__any_sync(full, mine && W.hop == 0)) {
+                const F2 df = f2_mag(W.d, fb);
+                const F2 len = f2_hyp(f2_mag(W.ex, fb), f2_sq(f2_mag(W.py, fb)));
+                const float mrg = fmaf(df.h + len.h, kDomF, Lf * kLocalF);
+                const float t = f2_add_f(f2_sub(df, f2_mag(end_b ? g0 : g1, fb)), len);
+                const unsigned bad = __ballot_sync(full, mine && W.hop == 0 && t > (end_b ? ef : Lf - ef) + mrg);
+                if (bad >> even & 3u) prop = false;
+            }
+            const double tol = times_eps(R.L);
+            const EvSrc es{W.inst, W.h, W.src, 0, W.px, W.py};
+            if (prop && W.pend && !stale && (end_b ? sbits(R.L) - sbits(W.e) <= kSnapUlps : le_s(W.e, tol))) {
+                // endpoint event at v0 (A = v0) or v1 (B = v1)
+                const double z = end_b ? R.L - W.px : W.px;
+                const double D = W.d + sqrt_nr(fma(z, z, W.py * W.py));
+                const unsigned v = end_b ? R.v1 : R.v0;
+                double g = end_b ? g1 : g0;
+                if (const int ev = vertex_event<PROV>(*Ip, v, D, g, &w, &es))
+                    queue_fan(w, cnt, req, m, W.inst, v & ~kPseudoBit, D, end_b ? R.twin : W.h, z,
+                             end_b ? -W.py : W.py, ev);
+            }
+            // occupancy: the sign of cross(e - I, v2 - e) at either end
+            const float exf = f_of(W.ex, fb), pyf = f_of(W.py, fb);
+            const float v = fmaf(exf, ycf, pyf * (xcf - ef));
+            const float err = fmaf(fabsf(exf), ycf, fmaf(fabsf(pyf), fabsf(xcf) + Lf, Lf * ycf * 0x1p-10f)) * 0x1p-20f;
+            const int sg = v > err ? 1 : (v < -err ? -1 : 0);
+            const int so = __shfl_xor_sync(full, sg, 1);
+            const int sA = end_b ? so : sg, sB = end_b ? sg : so;
+            const bool sure = sA > 0 || sB < 0 || (sA < 0 && sB > 0);
+            bool flag = false;
+            if (prop && !sure) {
+                const double den = R.yc - W.py, num = (R.xc - W.px) * (-W.py);
+                const double r = fma(end_b ? W.ex + tol : W.ex - tol, den, -num);
+                flag = end_b ? ge0_s(r) : gt0_s(r);
+            }
+            const unsigned flags = __ballot_sync(full, flag);
+            const bool before_A = sure ? sA > 0 : (flags >> even & 1u) != 0;
+            occ = prop && (sure ? sA < 0 && sB > 0 : !before_A && (flags >> even & 2u) != 0);
+            if (prop) {
+                right = before_A;
+                left = !before_A;
+            }
+            bool narrow = false;                        // v2's ray within the tolerance of this end
+            if (occ) {
+                if (stale) {
+                    left = right = false;
+                } else {
+                    const double dx = R.xc - W.px, dy = R.yc - W.py;
+                    const double xs = fma(dx * (-W.py), rcp_nr(dy), W.px);
+                    const long long pos = edge_pos(xs, R.L);
+                    const double D2 = W.d + sqrt_nr(fma(dx, dx, dy * dy));
+                    // (the even lane's reading decides for the pair)
+                    const unsigned pm = 3u << even;
+                    const unsigned long long a0 = __shfl_sync(pm, aw, even);
+                    if (a0 == kEmptyAngle || dbits(D2) < (a0 & ~kAngleXMask)) {
+                        left = right = true;
+                        if (!end_b) atomicMin(Ip->ang + W.h, pack_angle(D2, pos));
+                    } else {
+                        const long long qx = (long long)(a0 & kAngleXMask);
+                        left = min(pos + kSplitTol, kPosMax) >> kPosLow < qx;
+                        right = max(pos - kSplitTol, 0ll) >> kPosLow > qx;
+                        if (!left && !right) left = right = true;
+                    }
+                    if (!end_b)
+                        if (const int ev = vertex_event<PROV>(*Ip, R.v2, D2, g2, &w, &es)) {
+                            const int hp = 3 * (W.h / 3) + (W.h % 3 + 2) % 3;
+                            const double ux = -R.u2x, uy = -R.u2y, fx = W.px - R.xc, fy = W.py - R.yc;
+                            queue_fan(w, cnt, req, m, W.inst, R.v2 & ~kPseudoBit, D2, hp,
+                                     fx * ux + fy * uy, ux * fy - uy * fx, ev);
+                        }
+                    if (!sure) narrow = le_s(end_b ? W.e - xs : xs - W.e, tol);
+                }
+            }
+            const unsigned nm = __ballot_sync(full, narrow);
+            if (nm >> even & 1u) left = false;
+            if (nm >> even & 2u) right = false;
+            right = right && R.tw1 >= 0;
+            left = left && R.tw2 >= 0;
+            prop = prop && !stale;
+            if (have && W.task) {
+                occ = true;
+                left = R.tw2 >= 0;
+            }
+        }
+        n_exam += __popc(own & kPairLanes);
+        n_prop += __popc(__ballot_sync(full, prop) & kPairLanes);
+        n_occ += __popc(__ballot_sync(full, occ && mine) & kPairLanes);
+        // ---- left children of windows with two: to pairs without a child, else the next round
+        bool defer = right && left;
+        const unsigned tm = __ballot_sync(full, defer) & kPairLanes;
+        if (tm) {
+            const unsigned fm = __ballot_sync(full, !right && !left) & kPairLanes;
+            const int nfree = min(__popc(fm), __popc(tm)), rank = __popc(tm & before), j = __popc(fm & before);
+            if (defer && rank < nfree) {
+                pair_put(m, 2 * rank + (lane & 1), W, W.hop | kHopTask);
+                defer = false;
+            }
+            __syncwarp();
+            if ((fm >> even & 1u) && j < nfree) {
+                pair_get(m, 2 * j + (lane & 1), W);
+                Ip = w.inst + W.inst;
+                R = Ip->rec[W.h];
+                g0 = ldg_dist(Ip->g, R.v0 & ~kPseudoBit);
+                g1 = ldg_dist(Ip->g, R.v1 & ~kPseudoBit);
+                g2 = ldg_dist(Ip->g, R.v2 & ~kPseudoBit);
+                occ = left = true;
+                stale = false;
+            }
+            __syncwarp();
+        }
+        // ---- the child (as propagate_window's)
+        const bool rt = right, comp = right || left;
+        const unsigned fb = Ip->fbias;
+        const int che = rt ? R.tw1 : R.tw2;
+        if (comp) {
+            const char* cr = reinterpret_cast<const char*>(Ip->rec + che);
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(cr));
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(cr + sizeof(HERec) - 8));
+        }
+        const float tau = w.ctl[W.inst].tauf;
+        const double Lc = rt ? R.L1 : R.L2, ux = rt ? R.u1x : R.u2x, uy = rt ? R.u1y : R.u2y;
+        const double shared = rt ? R.L : 0.0, base = rt ? Lc : 0.0;
+        const double rx = W.px - shared;
+        // the even lane Ipx, the odd lane Ipy
+        const double part = fma(W.py, end_b ? ux : uy, end_b ? 0.0 : base);
+        const double Ic = fma(rx, end_b ? -uy : ux, part);
+        const double Io = shfl_other(Ic), po = shfl_other(part);
+        const double Ipx = end_b ? Io : Ic, Ipy = end_b ? Ic : Io, upy = end_b ? part : po;
+        double p = end_b ? Lc : 0.0;                    // at v2 of an occupied window
+        if (comp && !(occ && end_b != rt)) p = ray_hit(W.e - shared, W.ex, ux, uy, upy, W.py, base, Lc);
+        const double pother = shfl_other(p);
+        const float Lcf = f_of(Lc, fb), pf = f_of(p, fb), pof = __shfl_xor_sync(full, pf, 1);
+        const float width = end_b ? pf - pof : pof - pf;
+        bool child = comp && !stale;
+        if (child && !(width > Lcf * kLocalF)) child = lt_s(times_eps(Lc), end_b ? p - pother : pother - p);
+        const double exc = p - Ipx;
+        const F2 df = f2_mag(W.d, fb), yf = f2_mag(Ipy, fb);
+        const F2 len = f2_hyp(f2_mag(exc, fb), f2_sq(yf));
+        float key;
+        {
+            const float Lf = f_of(R.L, fb), xcf = f_of(R.xc, fb), ycf = f_of(R.yc, fb);
+            const float mrg = fmaf(df.h + len.h, kDomF, (Lf + Lcf + fabsf(xcf) + ycf) * kLocalF);
+            // B against the start vertex, A against the end vertex, both against T
+            const F2 e1 = f2_sub(df, f2_mag(end_b ? (rt ? g2 : g0) : (rt ? g1 : g2), fb));
+            const F2 eT = f2_sub(df, f2_mag(rt ? g0 : g1, fb));
+            const float uxf = f_of(ux, 896u << 20), uyf = f_of(uy, 896u << 20);
+            const float X = fmaf(pf, uxf, rt ? xcf : -Lf), Y = fmaf(pf, uyf, rt ? ycf : 0.f);
+            const float tT = f2_add_f(eT, len) - mrg;
+            const unsigned b1 = __ballot_sync(full, f2_add_f(e1, len) > (end_b ? pf : Lcf - pf) + mrg);
+            const unsigned b3 = __ballot_sync(full, tT > 0.f && tT * tT > fmaf(X, X, Y * Y) * (1.f + 0x1p-18f));
+            if ((b1 >> even & 3u) != 0u || (b3 >> even & 3u) == 3u) child = false;
+            const float side = (end_b ? sbits(exc) < 0 : gt0_s(exc)) ? len.h : -1.f;
+            const float other = __shfl_xor_sync(full, side, 1);
+            const float kA = end_b ? other : side, kB = end_b ? side : other;
+            key = df.h + (kA >= 0.f ? kA : (kB >= 0.f ? kB : yf.h));
+        }
+        const bool pend = end_b ? sbits(Lc) - sbits(p) <= kSnapUlps && !(occ && !rt) && (!rt || sbits(R.L) - sbits(W.e) > kSnapUlps)
+                                : le_s(p, times_eps(Lc)) && !(occ && rt) && (rt || !le_s(W.e, times_eps(R.L)));
+        bool cont = child && W.hop + 1 < hops && key <= tau && (!dry || __popc(live) >= tail_cut) && seen_child < room;
+        const unsigned dm = __ballot_sync(full, defer) & kPairLanes, cm = __ballot_sync(full, cont) & kPairLanes;
+        const unsigned endm = __ballot_sync(full, pend);
+        const int ntask = __popc(dm);
+        if (defer) pair_put(m, 2 * __popc(dm & before) + (lane & 1), W, W.hop | kHopTask);
+        const int cs = ntask + __popc(cm & before);
+        if (cont && cs >= 16) cont = false;
+        if (cont) {
+            const PairWin C{che, W.inst, W.src, 0, false, false, W.d, p, Ipx, Ipy, exc};
+            pair_put(m, 2 * cs + (lane & 1), C, (W.hop + 1) | (pend ? 1 << kHopPend : 0));
+        }
+        const bool emit = child && !cont;
+        const unsigned wm = __ballot_sync(full, emit) & kPairLanes;
+        if (wm) {
+            int k = __popc(wm & before);                // through the buffer, kChildBuf at a time
+            for (unsigned left_m = wm; left_m;) {
+                const int room_b = kChildBuf - nout, now = min(room_b, __popc(left_m));
+                if (emit && (left_m >> even & 1u) && k < now) {
+                    const int o = nout + k;
+                    if (!end_b) {
+                        m.child.he[o] = che;
+                        m.child.inst[o] = W.inst | (int)((endm >> even & 1u ? kPendA : 0u) | (endm >> even & 2u ? kPendB : 0u));
+                        m.child.src[o] = W.src;
+                        m.child.A[o] = p;
+                        m.child.px[o] = Ipx;
+                    } else {
+                        m.child.d[o] = W.d;
+                        m.child.B[o] = p;
+                        m.child.py[o] = Ipy;
+                        m.child.key[o] = key;
+                    }
+                }
+                nout += now;
+                k -= now;
+                for (int j = 0; j < now; ++j) left_m &= left_m - 1u;
+                __syncwarp();
+                if (nout == kChildBuf) {
+                    seen_child = flush_children(w, cnt, m, nout);
+                    nout = 0;
+                }
+            }
+        }
+        __syncwarp();
+        if (m.n_fan >= kFanBuf / 2) flush_fans(w, cnt, req, m);
+        const unsigned pm = __ballot_sync(full, comp) & kPairLanes;
+        n_comp += __popc(pm);
+        n_ray += 2 * __popc(pm) - __popc(__ballot_sync(full, comp && occ) & kPairLanes);
+        nq = min(16, ntask + __popc(cm));
+        n_chain += nq - ntask;
+        __syncwarp();          // the queue is written
+    }
+}
 
 // Step 3 of the iteration (Algorithm 2 over the selected windows), persistent.  Every
 // warp advances on its own in rounds: in each round lane t takes entry t of the warp's
@@ -843,19 +1229,8 @@ constexpr int kPropQueueBytesPerThread = 7 * 8 + 4 * 4;
 // PROV: also record the distance events (geodesic paths).
 template <bool PROV>
 __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int take_min) {
-    extern __shared__ double q_mem[];   // blockDim.x * kPropQueueBytesPerThread bytes
-    const int QB = blockDim.x;
-    double* q_d = q_mem;
-    double* q_A = q_d + QB;
-    double* q_B = q_A + QB;
-    double* q_px = q_B + QB;
-    double* q_py = q_px + QB;
-    double* q_ax = q_py + QB;
-    double* q_bx = q_ax + QB;
-    int* q_he = reinterpret_cast<int*>(q_bx + QB);
-    int* q_inst = q_he + QB;
-    int* q_src = q_inst + QB;
-    int* q_hop = q_src + QB;
+    extern __shared__ double prop_smem[];   // blockDim.x * kPropSmemBytesPerThread bytes
+    WarpMem& m = reinterpret_cast<WarpMem*>(prop_smem)[threadIdx.x >> 5];
     Counters* cnt = w.cnt;
     if (cnt->halt) return;
     const unsigned full = 0xffffffffu;
@@ -875,6 +1250,12 @@ __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int
     // resident warp or more fills whole warps.
     const int nwarps = threads >> 5;
     const int quota = max(take_min, min(32, (n + nwarps - 1) / max(nwarps, 1)));
+    if (lane == 0) m.n_fan = 0;
+    __syncwarp();
+    if (quota <= kPairQuota) {
+        propagate_pairs<PROV>(w, cnt, req, m, n, quota, room, hops, tail_cut);
+        return;
+    }
     const unsigned take_mask = quota >= 32 ? 0xffffffffu : (1u << quota) - 1u;
     // the arena fill this warp last saw (updated whenever it reserves arena slots)
     int seen_child = *(volatile int*)&cnt->n_child;
@@ -890,15 +1271,14 @@ __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int
         W.src = -1;
         W.pend = 0u;
         W.d = W.A = W.B = W.px = W.py = W.ax = W.bx = 0.0;
-        const int q0 = threadIdx.x & ~31;                   // the warp's region of the queue
         if (have) {
-            const int q = q0 + lane;
-            W.h = q_he[q]; W.inst = q_inst[q]; W.src = q_src[q];
-            const int hop = q_hop[q];
+            const int q = lane;
+            W.h = m.he[q]; W.inst = m.inst[q]; W.src = m.src[q];
+            const int hop = m.hop[q];
             W.task = (hop & kHopTask) != 0;
             W.pend = (unsigned)hop << (30 - kHopPend) & (kPendA | kPendB);
             W.hop = hop & kHopMask;
-            W.d = q_d[q]; W.A = q_A[q]; W.B = q_B[q]; W.px = q_px[q]; W.py = q_py[q]; W.ax = q_ax[q]; W.bx = q_bx[q];
+            W.d = m.d[q]; W.A = m.A[q]; W.B = m.B[q]; W.px = m.px[q]; W.py = m.py[q]; W.ax = m.ax[q]; W.bx = m.bx[q];
         }
         const unsigned need = __ballot_sync(full, !have) & take_mask;   // lanes nq.. below the quota
         if (need && !dry) {
@@ -922,6 +1302,7 @@ __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int
         }
         const unsigned live = __ballot_sync(full, have);    // (also: every lane has read its entry)
         if (!live) {                                        // nothing queued and nothing left to take
+            flush_fans(w, cnt, req, m);
             const unsigned long long sums[6] = {n_prop, n_chain, n_exam, n_occ, n_comp, n_ray};
             unsigned long long* dst[6] = {&cnt->propagated, &cnt->chained, &cnt->examined, &cnt->occupied,
                                           &cnt->children, &cnt->rays};
@@ -932,7 +1313,7 @@ __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int
         }
         ChildOut c;
         bool child = false, defer = false, occ = false, comp = false, prop = false;
-        if (have) prop = propagate_window<PROV>(w, cnt, req, W, c, child, defer, occ, comp);
+        if (have) prop = propagate_window<PROV>(w, cnt, req, m, W, c, child, defer, occ, comp);
         __syncwarp();
         bool cont = child && W.hop + 1 < hops && c.key <= w.ctl[W.inst].tauf &&
                     (!dry || nq >= tail_cut) && seen_child < room;
@@ -941,17 +1322,17 @@ __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int
         const unsigned tm = __ballot_sync(full, defer), cm = __ballot_sync(full, cont);
         const int ntask = __popc(tm);
         if (defer) {
-            const int q = q0 + __popc(tm & lt);
-            q_he[q] = W.h; q_inst[q] = W.inst; q_src[q] = W.src; q_hop[q] = W.hop | kHopTask;
-            q_d[q] = W.d; q_A[q] = W.A; q_B[q] = W.B; q_px[q] = W.px; q_py[q] = W.py; q_ax[q] = W.ax; q_bx[q] = W.bx;
+            const int q = __popc(tm & lt);
+            m.he[q] = W.h; m.inst[q] = W.inst; m.src[q] = W.src; m.hop[q] = W.hop | kHopTask;
+            m.d[q] = W.d; m.A[q] = W.A; m.B[q] = W.B; m.px[q] = W.px; m.py[q] = W.py; m.ax[q] = W.ax; m.bx[q] = W.bx;
         }
         if (cont) {
             const int slot = ntask + __popc(cm & lt);
             if (slot < 32) {
-                const int q = q0 + slot;
-                q_he[q] = c.he; q_inst[q] = W.inst; q_src[q] = W.src;
-                q_hop[q] = (W.hop + 1) | (int)(c.pend >> (30 - kHopPend));
-                q_d[q] = W.d; q_A[q] = c.A; q_B[q] = c.B; q_px[q] = c.px; q_py[q] = c.py; q_ax[q] = c.ax; q_bx[q] = c.bx;
+                const int q = slot;
+                m.he[q] = c.he; m.inst[q] = W.inst; m.src[q] = W.src;
+                m.hop[q] = (W.hop + 1) | (int)(c.pend >> (30 - kHopPend));
+                m.d[q] = W.d; m.A[q] = c.A; m.B[q] = c.B; m.px[q] = c.px; m.py[q] = c.py; m.ax[q] = c.ax; m.bx[q] = c.bx;
             } else {
                 cont = false;
             }
@@ -989,6 +1370,7 @@ __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int
         nq = min(32, ntask + __popc(cm));
         n_chain += nq - ntask;
         __syncwarp();          // the queue is written
+        if (m.n_fan >= kFanBuf / 2) flush_fans(w, cnt, req, m);
     }
 }
 
@@ -1061,7 +1443,10 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
     if (cnt->halt) return;
     const int nreq = min(cnt->n_req, w.req_cap), n_prop = min(cnt->n_child, w.arena_cap);
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&cnt->fan_cand, (unsigned long long)nreq);
-    if (blockIdx.x * blockDim.x >= max(n_prop, nreq * kFanLanes)) return;
+    // (the fans' candidates go to the last blocks, the statistics to the first, so that a
+    // short list of each runs side by side)
+    const int fan_block = gridDim.x - 1 - blockIdx.x;
+    if (blockIdx.x * blockDim.x >= n_prop && fan_block * blockDim.x >= nreq * kFanLanes) return;
     // first the selection statistics of the windows that the propagation created (here, where
     // the GPU has little else to do: from inside the propagation kernel they cost 8% of it)
     __shared__ PoolStats ps;
@@ -1083,7 +1468,7 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
     const FanReq* req = w.req[it & 1];
     FanReq* req_nx = w.req[(it + 1) & 1];
     const unsigned stamp_fan = (unsigned)it + 1u;
-    const int group0 = (blockIdx.x * blockDim.x + threadIdx.x) / kFanLanes;
+    const int group0 = (fan_block * blockDim.x + threadIdx.x) / kFanLanes;
     const int ngroups = (gridDim.x * blockDim.x) / kFanLanes;
     unsigned n_fans = 0, n_fwin = 0;
     for (int r = group0; r < nreq; r += ngroups) {     // uniform over the group
@@ -1651,7 +2036,7 @@ static cudaError_t launch_iteration(Workspace* ws, cudaStream_t s, const SolveCf
     k_compact<<<grid_for(4), tpb, 0, s>>>(w);
     if (ev) cudaEventRecord(ev[2], s);
     const dim3 pg(grid_for(cfg.prop_blocks_per_sm));
-    const size_t psh = (size_t)cfg.prop_threads * kPropQueueBytesPerThread;
+    const size_t psh = (size_t)cfg.prop_threads * kPropSmemBytesPerThread;
     if (cfg.prov) k_propagate<true><<<pg, cfg.prop_threads, psh, s>>>(w, cfg.hops, cfg.tail_cut, cfg.take_min);
     else k_propagate<false><<<pg, cfg.prop_threads, psh, s>>>(w, cfg.hops, cfg.tail_cut, cfg.take_min);
     if (ev) cudaEventRecord(ev[3], s);
