@@ -529,7 +529,8 @@ __global__ void __launch_bounds__(256) k_compact(Work w) {
     __shared__ PoolStats ps;
     Counters* cnt = w.cnt;
     if (cnt->halt) return;
-    const int it = cnt->iter, lane = threadIdx.x & 31;
+    __shared__ int wcount[2][8], wbase[2][8];
+    const int it = cnt->iter, lane = threadIdx.x & 31, warp = threadIdx.x / 32;
     const WinSoA cur = w.pool[it & 1], nxt = w.pool[(it + 1) & 1];
     const int n_pool = cnt->n_pool, n = n_pool + cnt->n_new;
     unsigned* g_hist = w.hist[(it + 1) & 1];
@@ -562,14 +563,29 @@ __global__ void __launch_bounds__(256) k_compact(Work w) {
         } else {
             sel = valid && le_s(W.key, w.ctl[W.inst].tau);
         }
-        // both reservations at once, from two lanes
+        // one reservation of each kind a block (the counters are two words that every block
+        // adds to)
         bool rest = valid && !sel;
         const unsigned sm = __ballot_sync(0xffffffffu, sel), rm = __ballot_sync(0xffffffffu, rest);
         const unsigned lt = (1u << lane) - 1u;
-        int got = 0;
-        if (lane < 2 && (lane ? rm : sm)) got = atomicAdd(lane ? &cnt->n_rest : &cnt->n_sel, __popc(lane ? rm : sm));
-        int slot = __shfl_sync(0xffffffffu, got, 0) + __popc(sm & lt);
-        int rslot = __shfl_sync(0xffffffffu, got, 1) + __popc(rm & lt);
+        if (lane == 0) { wcount[0][warp] = __popc(sm); wcount[1][warp] = __popc(rm); }
+        __syncthreads();
+        if (threadIdx.x < 64) {
+            const int kind = threadIdx.x / 32;          // warp 0: selected, warp 1: the rest
+            int c = lane < 8 ? wcount[kind][lane] : 0, incl = c;
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            int got = 0;
+            if (lane == 7 && incl) got = atomicAdd(kind ? &cnt->n_rest : &cnt->n_sel, incl);
+            got = __shfl_sync(0xffffffffu, got, 7);
+            if (lane < 8) wbase[kind][lane] = got + incl - c;
+        }
+        __syncthreads();
+        int slot = wbase[0][warp] + __popc(sm & lt);
+        int rslot = wbase[1][warp] + __popc(rm & lt);
         const bool over = sel && slot >= w.sel_cap;         // work list full: stays pending
         if (sel && !over) store_win(w.sel, slot, W);
         if (__any_sync(0xffffffffu, over)) {
@@ -636,7 +652,7 @@ constexpr float kLocalF = 0x1p-20f;
 // round (one a lane; a round reads its entries before it writes the next round's), and fan
 // candidates on their way to the request list, so that no round waits for the slot of one.
 constexpr int kFanBuf = 16;
-constexpr int kChildBuf = 8;
+constexpr int kChildBuf = 16;
 struct WarpMem {
     double d[32], A[32], px[32], py[32], ax[32];
     union {
@@ -653,7 +669,6 @@ struct WarpMem {
     FanReq fan[kFanBuf];
     int n_fan, pad[7];
 };
-static_assert(sizeof(WarpMem) == 72 * 32 + kFanBuf * sizeof(FanReq) + 32 && sizeof(WarpMem) % 16 == 0, "layout");
 constexpr int kPropSmemBytesPerThread = (int)sizeof(WarpMem) / 32;
 static_assert(sizeof(WarpMem) % 32 == 0, "bytes a thread");
 
@@ -950,6 +965,10 @@ __device__ __forceinline__ void propagate_pairs(const Work& w, Counters* cnt, Fa
     const unsigned before = ((1u << even) - 1u) & kPairLanes;
     int seen_child = *(volatile int*)&cnt->n_child;
     unsigned n_prop = 0, n_chain = 0, n_exam = 0, n_occ = 0, n_comp = 0, n_ray = 0;
+    // the first `quota` windows of a warp are its by position: no atomic, and as the quota is
+    // the list over the resident warps, usually the whole list
+    int first = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * quota;
+    const int handed = (int)((gridDim.x * blockDim.x) >> 5) * quota;
     bool dry = false;
     int nq = 0, nout = 0;                               // queued windows, children held back
     for (;;) {
@@ -961,10 +980,13 @@ __device__ __forceinline__ void propagate_pairs(const Work& w, Counters* cnt, Fa
         W.d = W.e = W.px = W.py = W.ex = 0.0;
         if (have) pair_get(m, lane, W);
         if (nq < quota && !dry) {
-            int base = 0;
-            if (lane == 0) base = atomicAdd(&cnt->work_next, quota - nq);
-            base = __shfl_sync(full, base, 0);
-            if (base + quota - nq >= n) dry = true;
+            int base = first;
+            if (first < 0) {
+                if (lane == 0) base = handed + atomicAdd(&cnt->work_next, quota - nq);
+                base = __shfl_sync(full, base, 0);
+            }
+            if (base + quota - nq >= n || (first >= 0 && handed >= n)) dry = true;
+            first = -1;
             const int idx = base + slot - nq;
             if (slot >= nq && slot < quota && idx < n) {
                 const int fi = w.sel.inst[idx];
@@ -1261,6 +1283,9 @@ __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int
     int seen_child = *(volatile int*)&cnt->n_child;
     // statistics, kept per warp and added to the counters once when the warp ends
     unsigned n_prop = 0, n_chain = 0, n_exam = 0, n_occ = 0, n_comp = 0, n_ray = 0;
+    // the first `quota` windows of a warp are its by position, the others handed out in order
+    int first = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * quota;
+    const int handed = nwarps * quota;
     bool dry = false;          // the selected list is exhausted
     int nq = 0;                // queue entries
     for (;;) {
@@ -1282,10 +1307,13 @@ __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int
         }
         const unsigned need = __ballot_sync(full, !have) & take_mask;   // lanes nq.. below the quota
         if (need && !dry) {
-            int base = 0;
-            if (lane == 0) base = atomicAdd(&cnt->work_next, __popc(need));
-            base = __shfl_sync(full, base, 0);
-            if (base + __popc(need) >= n) dry = true;
+            int base = first;
+            if (first < 0) {
+                if (lane == 0) base = handed + atomicAdd(&cnt->work_next, __popc(need));
+                base = __shfl_sync(full, base, 0);
+            }
+            if (base + __popc(need) >= n || (first >= 0 && handed >= n)) dry = true;
+            first = -1;
             if ((need >> lane) & 1u) {
                 const int idx = base + __popc(need & lt);
                 if (idx < n) {
