@@ -102,8 +102,9 @@ typedef struct {
     int32_t block;            /* threads per block of the propagation kernel, a multiple of 32
                                  in [32, 256] (0 = default 64) */
     int32_t flags;            /* PCH_FLAG_* */
-    int32_t hops;             /* windows one propagation lane may chain within an iteration's
-                                 band (1 = the paper's one hop per iteration; 0 = default 32) */
+    int32_t hops;             /* windows one propagation lane may chain within an iteration, up to
+                                 16 mean edge lengths past the selection's threshold (1 = the
+                                 paper's one hop per iteration; 0 = default 32) */
 } pch_options;
 
 enum {

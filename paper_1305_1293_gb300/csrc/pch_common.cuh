@@ -131,7 +131,7 @@ struct InstCtl {
     float last_ratio;           // children / selected of the previous iteration
     float ctl_out;              // last controller output
     int active;
-    float tauf;                 // tau as an FP32 image (scaled by the instance's power of two)
+    float tauf;                 // chaining limit (tau and kChainAhead edge lengths) as an FP32 image
 };
 
 // ---- global counters of one solve -------------------------------------------------
