@@ -40,13 +40,13 @@ __device__ __forceinline__ double ldg_dist(const unsigned long long* g, unsigned
 }
 
 // Crossing position on an edge of length L in units of 2^-44 of it (only the order of
-// positions on one edge matters, so 1 / L is the single-precision estimate, the same for
+// positions on one edge matters, so 1 / L is the hardware approximation, the same for
 // every window on it), clamped to [0, 2^44): an integer made from the product's bits, as
 // a conversion would run on the FP64 unit.
 constexpr int kPosBits = 44;
 constexpr long long kPosMax = (1ll << kPosBits) - 1;
 __device__ __forceinline__ long long edge_pos(double x, double L) {
-    const double r = nr_range(L) ? widen_normal(rcp_approx_f32(narrow_seed(L))) : 1.0 / L;
+    const double r = nr_range(L) ? rcp_approx(L) : 1.0 / L;
     const unsigned long long q = dbits(x * r);
     const int shift = 1023 + 52 - kPosBits - (int)(q >> 52);          // of the 53-bit mantissa, to the right
     if ((long long)q < 0 || shift > 52) return 0;                     // negative or below one unit
