@@ -103,8 +103,9 @@ typedef struct {
                                  in [32, 256] (0 = default 64) */
     int32_t flags;            /* PCH_FLAG_* */
     int32_t hops;             /* windows one propagation lane may chain within an iteration, up to
-                                 16 mean edge lengths past the selection's threshold (1 = the
-                                 paper's one hop per iteration; 0 = default 32) */
+                                 16 mean edge lengths past the selection's threshold; fewer
+                                 are chained while the front meets many pseudo-sources (1 =
+                                 the paper's one hop per iteration; 0 = default 32) */
 } pch_options;
 
 enum {

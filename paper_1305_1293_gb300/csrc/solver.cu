@@ -19,6 +19,7 @@
 // the first event of Algorithm 4's (key, value) order; angle_split is one packed 64-bit
 // word per half-edge (rounded-up distance | crossing position), also updated by atomicMin.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstddef>
 #include <cstring>
@@ -344,6 +345,20 @@ __global__ void k_init_sources(Work w, const SrcDev* __restrict__ srcs, int n_sr
 // hops) was no faster; 4 edge lengths took 22 ms.
 constexpr double kChainAhead = 16.0;
 
+// How many hops the next iteration's chains may take (at most the caller's), from the windows
+// the last one examined and the pseudo-source fans it made.  Fans are made between
+// iterations, so on a surface dense in saddles a long chain runs ahead of the shorter
+// distances that the fans behind it will bring, and most of its windows are useless: 24
+// uneven meshes (22 windows a fan) took 28.2 ms and 67M windows with 32 hops, 14.4 ms and 34M
+// with 6; 64 sources on a noisy sphere (17 a fan) 2.15 and 1.31 ms.  With few fans short
+// chains only add iterations: 512 x 512 terrain (370 a fan) 7.3 ms with 32 hops, 7.9 with
+// 8.  Lines at 32 and 100 windows a fan; 16 hops between them suit 5,120 faces (46 a fan:
+// 1.13 -> 0.80 ms).  Before the first windows: 8.
+__device__ __forceinline__ int hop_limit(float examined, float fans) {
+    if (examined < 64.f) return 8;
+    return examined < 32.f * fans ? 5 : (examined < 100.f * fans ? 16 : INT_MAX);
+}
+
 // Loop control, then per instance the selection threshold: the plain control selects the k
 // nearest windows (Section 4.2, Step 1) through the key histogram: tau = upper edge of the
 // first bin where the cumulative count reaches k.  Also rolls the histogram reference and
@@ -463,6 +478,9 @@ __global__ void __launch_bounds__(kBins) k_ctrl(Work w, int control, const float
                     cnt->peak_pending = (unsigned long long)(n_pool + n_new);
             }
             if (!halt) {
+                cnt->hops = hop_limit((float)(cnt->examined - cnt->examined0), (float)(cnt->fans - cnt->fans0));
+                cnt->examined0 = cnt->examined;
+                cnt->fans0 = cnt->fans;
                 cnt->n_pool = n_pool;
                 cnt->n_new = n_new;
                 cnt->n_req = n_req;
@@ -1269,6 +1287,7 @@ __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int
     const unsigned lt = (1u << lane) - 1u;
     const int it = cnt->iter;
     const int n = min(cnt->n_sel, w.sel_cap);
+    hops = min(hops, cnt->hops);
     FanReq* req = w.req[it & 1];
     // The arena cannot overflow: past `room` a warp stops chaining once it has seen the fill
     // (at its next write, of 32 children at most), and after that its 32 queued windows
