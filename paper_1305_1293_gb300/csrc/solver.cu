@@ -375,8 +375,8 @@ __global__ void __launch_bounds__(kBins) k_ctrl(Work w, int control, const float
     __shared__ unsigned prefix[kBins];
     __shared__ unsigned wsum[kBins / 32];
     __shared__ float feat[kFeatures];
-    __shared__ float hb0[kHidden], hb1[kHidden];
-    __shared__ float y;
+    __shared__ float hidden[kHidden];
+    static_assert(kBins == 4 * kHidden, "MlpRows");
     __shared__ long long s_k;
     Counters* cnt = w.cnt;
     const int t = threadIdx.x, lane = t & 31;
@@ -429,12 +429,14 @@ __global__ void __launch_bounds__(kBins) k_ctrl(Work w, int control, const float
             if (t == 0) c.last_ratio = n_sel > 0 ? (float)n_child / (float)n_sel : 0.f;
             const bool learned = control == PCH_CONTROL_LEARNED && mlp != nullptr && np > 0;
             if (learned || w.trace) {
+                MlpRows mlp_rows;
+                if (learned) mlp_rows.load(mlp);
                 prefix[t] = incl;
                 __syncthreads();
                 if (t < kFeatures) controller_features(c, w.inst[inst], prefix, np, it, feat);
                 __syncthreads();
                 if (learned) {
-                    mlp_forward_block(mlp, feat, hb0, hb1, &y);
+                    const float y = mlp_rows.forward(feat, hidden);
                     if (t == 0) {
                         c.ctl_out = y;
                         // y = log2(windows to select) / 24, clamped to the range of k the network
