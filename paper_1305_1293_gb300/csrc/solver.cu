@@ -567,7 +567,8 @@ __device__ __forceinline__ double window_key(const Win& W) {
 __device__ __forceinline__ bool created_useless(const Inst& I, const Win& W) {
     const HERec& R = I.rec[W.he];
     const double g0 = ldg_dist(I.g, R.v0 & ~kPseudoBit), g1 = ldg_dist(I.g, R.v1 & ~kPseudoBit);
-    return dominated(W.key, g0 + W.B) || dominated(W.key, g1 + (R.L - W.A)) || stale_source(I, W.src, W.d);
+    const bool stale = stale_source(I, W.src, W.d);
+    return dominated(W.key, g0 + W.B) || dominated(W.key, g1 + (R.L - W.A)) || stale;
 }
 
 // Compaction: selected windows to the work list, the rest to the next pool.  Reads the
@@ -576,31 +577,38 @@ __device__ __forceinline__ bool created_useless(const Inst& I, const Win& W) {
 __global__ void __launch_bounds__(256) k_compact(Work w) {
     __shared__ PoolStats ps;
     Counters* cnt = w.cnt;
-    if (cnt->halt) return;
     __shared__ int wcount[2][8], wbase[2][8];
-    const int it = cnt->iter, lane = threadIdx.x & 31, warp = threadIdx.x / 32;
+    // (loads that do not depend on one another are issued together here and below: on a
+    // short list the kernel's time is its chain of loads)
+    const int halt = cnt->halt, it = cnt->iter, n_pool = cnt->n_pool, n = n_pool + cnt->n_new;
+    if (halt || blockIdx.x * blockDim.x >= n) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x / 32;
     const WinSoA cur = w.pool[it & 1], nxt = w.pool[(it + 1) & 1];
-    const int n_pool = cnt->n_pool, n = n_pool + cnt->n_new;
     unsigned* g_hist = w.hist[(it + 1) & 1];
-    if (blockIdx.x * blockDim.x >= n) return;
     stats_begin(ps, w.n_inst);
     int created = 0;
     for (int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
         const int i = base + threadIdx.x;
         bool valid = i < n;
         Win W{0, 0, -1, 0u, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        double tau = -INFINITY;
         if (valid) {
             if (i < n_pool) {
                 W = load_win(cur, i);
                 W.key = cur.key[i];
+                tau = w.ctl[W.inst].tau;
                 if (stale_source(w.inst[W.inst], W.src, W.d)) valid = false;   // dropped from the pool
-            } else if (w.arena.he[i - n_pool] < 0) {
-                valid = false;                                                 // an empty slot
             } else {
                 W = load_win(w.arena, i - n_pool);
-                W.key = window_key(W);
-                valid = !created_useless(w.inst[W.inst], W);
-                created += valid ? 1 : 0;
+                if (W.he < 0) {                                                // an empty slot
+                    valid = false;
+                    W.inst = 0;
+                } else {
+                    tau = w.ctl[W.inst].tau;
+                    W.key = window_key(W);
+                    valid = !created_useless(w.inst[W.inst], W);
+                    created += valid ? 1 : 0;
+                }
             }
         }
         bool sel;
@@ -609,7 +617,7 @@ __global__ void __launch_bounds__(256) k_compact(Work w) {
             const unsigned long long kb = dbits(W.key), tk = w.sthr_key[t];
             sel = valid && (kb < tk || (kb == tk && i <= w.sthr_idx[t]));
         } else {
-            sel = valid && le_s(W.key, w.ctl[W.inst].tau);
+            sel = valid && le_s(W.key, tau);
         }
         // one reservation of each kind a block (the counters are two words that every block
         // adds to)
@@ -1302,13 +1310,12 @@ __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int
     extern __shared__ double prop_smem[];   // blockDim.x * kPropSmemBytesPerThread bytes
     WarpMem& m = reinterpret_cast<WarpMem*>(prop_smem)[threadIdx.x >> 5];
     Counters* cnt = w.cnt;
-    if (cnt->halt) return;
+    const int halt = cnt->halt, it = cnt->iter, n = min(cnt->n_sel, w.sel_cap);
+    hops = min(hops, cnt->hops);
+    if (halt) return;
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    const int it = cnt->iter;
-    const int n = min(cnt->n_sel, w.sel_cap);
-    hops = min(hops, cnt->hops);
     FanReq* req = w.req[it & 1];
     // The arena cannot overflow: past `room` a warp stops chaining once it has seen the fill
     // (at its next write, of 32 children at most), and after that its 32 queued windows
@@ -1517,8 +1524,9 @@ __device__ __forceinline__ double fan_hit(const HERec& Ro, double2 z) {
 template <bool PROV>
 __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
     Counters* cnt = w.cnt;
-    if (cnt->halt) return;
+    const int halt = cnt->halt, it = cnt->iter;
     const int nreq = min(cnt->n_req, w.req_cap), n_prop = min(cnt->n_child, w.arena_cap);
+    if (halt) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&cnt->fan_cand, (unsigned long long)nreq);
     // (the fans' candidates go to the last blocks, the statistics to the first, so that a
     // short list of each runs side by side)
@@ -1527,7 +1535,7 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
     // first the selection statistics of the windows that the propagation created (here, where
     // the GPU has little else to do: from inside the propagation kernel they cost 8% of it)
     __shared__ PoolStats ps;
-    unsigned* g_hist = w.hist[(cnt->iter + 1) & 1];
+    unsigned* g_hist = w.hist[(it + 1) & 1];
     if (!w.append) {
         stats_begin(ps, w.n_inst);
         for (int base = blockIdx.x * blockDim.x; base < n_prop; base += gridDim.x * blockDim.x) {
@@ -1541,7 +1549,6 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
     const int lead = lane & ~(kFanLanes - 1);
     const unsigned gmask = ((1u << kFanLanes) - 1u) << lead;
     const unsigned below = (1u << sl) - 1u;
-    const int it = cnt->iter;
     const FanReq* req = w.req[it & 1];
     FanReq* req_nx = w.req[(it + 1) & 1];
     const unsigned stamp_fan = (unsigned)it + 1u;
