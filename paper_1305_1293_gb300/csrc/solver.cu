@@ -1572,9 +1572,19 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
         // deferred now (a tie, or a candidate that did not make the fan but carries the
         // final distance within the margin)
         int kind = 0;
+        const unsigned long long gv = __ldcg(I.g + v), db = dbits(D);
+        unsigned old = stamp_fan;
+        if (sl == 0 && rq.tie == kReqLowered && db == gv) old = atomicExch(I.stamp + v, stamp_fan);
+        // (nor does each lane's first corner wait for it)
+        int hv_first = 0;
+        float c_first = 0.f, ang_first = 0.f;
+        if (s + sl < e) {
+            hv_first = I.vlist[s + sl];
+            c_first = I.vphi[hv_first];
+            ang_first = I.hang[hv_first];
+        }
         if (sl == 0) {
-            const unsigned long long gv = __ldcg(I.g + v), db = dbits(D);
-            if (rq.tie == kReqLowered && db == gv && atomicExch(I.stamp + v, stamp_fan) != stamp_fan) {
+            if (old != stamp_fan) {
                 kind = 1;
             } else if (db <= gv + kDomUlps) {
                 if (rq.tie == kReqDeferredTie) kind = 2;
@@ -1688,13 +1698,13 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
             double s0 = 0.0, s1 = 0.0;
             HERec Ro;
             if (j < e) {
-                const int hv = I.vlist[j];
+                const int hv = j0 == s ? hv_first : I.vlist[j];
                 bool ex0 = false, ex1 = false;
                 int shift = 0;
                 if (all) {
                     has = true;
                 } else {
-                    const float c0 = I.vphi[hv], c1 = c0 + I.hang[hv];
+                    const float c0 = j0 == s ? c_first : I.vphi[hv], c1 = c0 + (j0 == s ? ang_first : I.hang[hv]);
                     for (int k = 0; k < nw && !has; ++k)
                         for (int sh = boundary ? 0 : -2; sh <= (boundary ? 0 : 1) && !has; ++sh) {
                             const float lo = wlo[k] + (float)sh * T, hi = whi[k] + (float)sh * T;
