@@ -216,6 +216,7 @@ struct Work {
     InstCtl* ctl;
     int n_inst;
     int append;             // new windows reach the pool through k_append, not from the arena
+    int ahead;              // a child's record is prefetched while the child is computed
     Counters* cnt;
     float* trace;           // controller trace rows
     int trace_cap;
