@@ -710,18 +710,17 @@ constexpr float kLocalF = 0x1p-20f;
 constexpr int kFanBuf = 16;
 constexpr int kChildBuf = 16;
 struct WarpMem {
-    double d[32], A[32], px[32], py[32], ax[32];
+    int4 id[32];                            // half-edge, instance, source, hops and flags
+    double2 AB[32], I[32];                  // (A, B), (px, py)
     union {
-        struct {
-            double B[32], bx[32];
-        };
+        double2 ab[32];                     // (ax, bx)
         struct {                            // pairs of lanes (propagate_pairs) keep one end a lane:
             double d[kChildBuf], A[kChildBuf], B[kChildBuf], px[kChildBuf], py[kChildBuf];
             int he[kChildBuf], inst[kChildBuf], src[kChildBuf];
             float key[kChildBuf];
         } child;                            // here children on their way to the arena
     };
-    int he[32], inst[32], src[32], hop[32];
+    double d[32];
     FanReq fan[kFanBuf];
     int n_fan, pad[7];
 };
@@ -982,16 +981,20 @@ struct PairWin {
 __device__ __forceinline__ double shfl_other(double x) { return __shfl_xor_sync(0xffffffffu, x, 1); }
 
 __device__ __forceinline__ void pair_put(WarpMem& m, int at, const PairWin& W, int hop) {
-    m.he[at] = W.h; m.inst[at] = W.inst; m.src[at] = W.src; m.hop[at] = hop;
-    m.d[at] = W.d; m.A[at] = W.e; m.px[at] = W.px; m.py[at] = W.py; m.ax[at] = W.ex;
+    m.id[at] = make_int4(W.h, W.inst, W.src, hop);
+    m.AB[at] = make_double2(W.e, W.ex);
+    m.I[at] = make_double2(W.px, W.py);
+    m.d[at] = W.d;
 }
 __device__ __forceinline__ void pair_get(const WarpMem& m, int at, PairWin& W) {
-    const int hop = m.hop[at];
-    W.h = m.he[at]; W.inst = m.inst[at]; W.src = m.src[at];
+    const int4 id = m.id[at];
+    const double2 e = m.AB[at], I = m.I[at];
+    const int hop = id.w;
+    W.h = id.x; W.inst = id.y; W.src = id.z;
     W.task = (hop & kHopTask) != 0;
     W.pend = (hop >> kHopPend & 1) != 0;
     W.hop = hop & kHopMask;
-    W.d = m.d[at]; W.e = m.A[at]; W.px = m.px[at]; W.py = m.py[at]; W.ex = m.ax[at];
+    W.d = m.d[at]; W.e = e.x; W.px = I.x; W.py = I.y; W.ex = e.y;
 }
 
 // (whole warp) The buffered children to the arena; returns its fill after them.
@@ -1307,7 +1310,7 @@ __device__ __forceinline__ void propagate_pairs(const Work& w, Counters* cnt, Fa
 // PROV: also record the distance events (geodesic paths).
 template <bool PROV>
 __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int take_min) {
-    extern __shared__ double prop_smem[];   // blockDim.x * kPropSmemBytesPerThread bytes
+    extern __shared__ double2 prop_smem[];   // blockDim.x * kPropSmemBytesPerThread bytes
     WarpMem& m = reinterpret_cast<WarpMem*>(prop_smem)[threadIdx.x >> 5];
     Counters* cnt = w.cnt;
     const int halt = cnt->halt, it = cnt->iter, n = min(cnt->n_sel, w.sel_cap);
@@ -1353,13 +1356,14 @@ __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int
         W.pend = 0u;
         W.d = W.A = W.B = W.px = W.py = W.ax = W.bx = 0.0;
         if (have) {
-            const int q = lane;
-            W.h = m.he[q]; W.inst = m.inst[q]; W.src = m.src[q];
-            const int hop = m.hop[q];
+            const int4 id = m.id[lane];
+            const double2 AB = m.AB[lane], I = m.I[lane], ab = m.ab[lane];
+            const int hop = id.w;
+            W.h = id.x; W.inst = id.y; W.src = id.z;
             W.task = (hop & kHopTask) != 0;
             W.pend = (unsigned)hop << (30 - kHopPend) & (kPendA | kPendB);
             W.hop = hop & kHopMask;
-            W.d = m.d[q]; W.A = m.A[q]; W.B = m.B[q]; W.px = m.px[q]; W.py = m.py[q]; W.ax = m.ax[q]; W.bx = m.bx[q];
+            W.d = m.d[lane]; W.A = AB.x; W.B = AB.y; W.px = I.x; W.py = I.y; W.ax = ab.x; W.bx = ab.y;
         }
         const unsigned need = __ballot_sync(full, !have) & take_mask;   // lanes nq.. below the quota
         if (need && !dry) {
@@ -1407,16 +1411,21 @@ __global__ void __maxnreg__(128) k_propagate(Work w, int hops, int tail_cut, int
         const int ntask = __popc(tm);
         if (defer) {
             const int q = __popc(tm & lt);
-            m.he[q] = W.h; m.inst[q] = W.inst; m.src[q] = W.src; m.hop[q] = W.hop | kHopTask;
-            m.d[q] = W.d; m.A[q] = W.A; m.B[q] = W.B; m.px[q] = W.px; m.py[q] = W.py; m.ax[q] = W.ax; m.bx[q] = W.bx;
+            m.id[q] = make_int4(W.h, W.inst, W.src, W.hop | kHopTask);
+            m.d[q] = W.d;
+            m.AB[q] = make_double2(W.A, W.B);
+            m.I[q] = make_double2(W.px, W.py);
+            m.ab[q] = make_double2(W.ax, W.bx);
         }
         if (cont) {
             const int slot = ntask + __popc(cm & lt);
             if (slot < 32) {
                 const int q = slot;
-                m.he[q] = c.he; m.inst[q] = W.inst; m.src[q] = W.src;
-                m.hop[q] = (W.hop + 1) | (int)(c.pend >> (30 - kHopPend));
-                m.d[q] = W.d; m.A[q] = c.A; m.B[q] = c.B; m.px[q] = c.px; m.py[q] = c.py; m.ax[q] = c.ax; m.bx[q] = c.bx;
+                m.id[q] = make_int4(c.he, W.inst, W.src, (W.hop + 1) | (int)(c.pend >> (30 - kHopPend)));
+                m.d[q] = W.d;
+                m.AB[q] = make_double2(c.A, c.B);
+                m.I[q] = make_double2(c.px, c.py);
+                m.ab[q] = make_double2(c.ax, c.bx);
             } else {
                 cont = false;
             }
