@@ -769,7 +769,7 @@ __device__ __forceinline__ void flush_fans(const Work& w, Counters* cnt, FanReq*
 // |I A|, |I B| that the filters compare are two-float values made from the coordinates
 // when they are needed, so no rounding of theirs accumulates along a lineage.  With all of
 // it in FP64, 62 instructions a window, eight fields on the 327,680-face sphere took
-// 86.1 ms and take 39.2, the 1M-face torus 49.3 and 22.5.
+// 86.1 ms and the 1M-face torus 49.3; like this 39.2 and 22.5 (36.6 and 20.7 by now).
 template <bool PROV>
 __device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, FanReq* req, WarpMem& m, const LaneWin& W,
                                                  ChildOut& c, bool& has_child, bool& defer, bool& occ, bool& comp) {
@@ -966,8 +966,8 @@ __device__ __forceinline__ bool propagate_window(const Work& w, Counters* cnt, F
 // through shared memory).  Chosen when at most kPairQuota windows a resident warp are
 // selected, half a warp: lists of 16 a warp still run faster in pairs (terrain 512 x 512 7.89
 // -> 7.54 ms; with lines at 4 and 8 a warp 7.69 and 7.62), longer ones fill whole warps.
-// 187 x 331 grid 4.50 -> 3.77 ms, 64 sources on 100,820 faces 2.66 -> 2.31, Voronoi labels
-// on 327,680 faces 10.5 -> 9.1, 5,120 faces 1.31 -> 1.21.
+// When they came in: 187 x 331 grid 4.50 -> 3.77 ms, 64 sources on 100,820 faces 2.66 -> 2.31,
+// Voronoi labels on 327,680 faces 10.5 -> 9.1, 5,120 faces 1.31 -> 1.21.
 constexpr int kPairQuota = 16;
 constexpr unsigned kPairLanes = 0x55555555u;        // the even lane of every pair
 
@@ -1527,7 +1527,7 @@ __device__ __forceinline__ double fan_hit(const HERec& Ro, double2 z) {
 // instructions of 64 cycles): the new windows are filtered in FP32 before their slots are
 // reserved, directions keep their length, and the statistics are collected in shared memory
 // (per window, global atomics on an instance's few words took a third of the kernel). 24 uneven
-// meshes, 4.3M fan windows: 32.9 -> 29.9 ms a call.
+// meshes, 4.3M fan windows (1.8M since the hop limit): 32.9 -> 29.9 ms a call.
 // kFanLanes lanes per fan candidate; lane j of the group handles corners j, j + 8, ...
 // of the vertex's one-ring.  PROV: also record the distance events (geodesic paths).
 template <bool PROV>
@@ -2324,7 +2324,11 @@ static SolveCfg make_cfg(const pch_options* opt, int n_inst, long long total_key
     cfg.hops = std::min((opt && opt->hops > 0) ? opt->hops : default_hops(), kHopMask);
     cfg.tail_cut = default_tail_cut();
     cfg.take_min = default_take_min();
-    cfg.unroll = 2;
+    // Iterations a pass of the graph's loop: the loop's own evaluation costs about 2 us, an
+    // iteration after the last (its kernels return at once) 5.  With 1, 2, 4, 6: 5,120 faces 0.800,
+    // 0.775, 0.762, 0.767 ms; 64 sources 1.195, 1.155, 1.140, 1.145; 24 uneven meshes 13.50, 13.25,
+    // 13.15, 13.09.
+    cfg.unroll = 4;
     // Step 3 organises the new windows into a gap-free pool: the next iteration's compaction
     // reads them from the arena, or with PCH_FLAG_EDGE_SORT they are ordered by (instance,
     // half-edge) for the per-edge trimming and appended
