@@ -455,9 +455,9 @@ def run_gpu(args):
 # mid-solve launches of a smaller batched sphere of the same family (profiles/), valid
 # only for the kernel sources it was taken on (their hash); scaled to a launch of the
 # benchmark by its windows.  Any change of the sources reports null until it is taken again.
-PROP_TRAFFIC = {"sources_sha256_16": "0db47d1f64d77651", "bytes_per_window": 13.27}
+PROP_TRAFFIC = {"sources_sha256_16": "815a9b2e8a782919", "bytes_per_window": 21.98}
 PROP_SOURCES = ("paper_1305_1293_gb300/csrc/solver.cu", "paper_1305_1293_gb300/csrc/pch_common.cuh",
-                "paper_1305_1293_gb300/csrc/fastmath.cuh")
+                "paper_1305_1293_gb300/csrc/fastmath.cuh", "paper_1305_1293_gb300/csrc/twofloat.cuh")
 
 
 def prop_sources_hash():
@@ -480,9 +480,11 @@ def phase_rooflines(pst, passes, hbm):
     algorithmic work counted in one profiled solve (bytes per window as in the comments below)."""
     ph = pst["ms_phase"]
     out = {"propagate_fp64_tflops": pst["prop_fp64_ops"] / max(ph["propagate"], 1e-9) / 1e9}
-    sel_bytes = 160 * pst["windows_scanned"]                        # 76 B in + 76 B out + 8 B gather
-    sort_bytes = pst["windows_sorted"] * (8 + 20 * passes)          # pass 0 reads he/inst; 4+8+8 B a pass
-    app_bytes = 276 * pst["windows_sorted"]                         # key/index 8, window 76, record 96, g 16, out 76
+    # pool windows: 60 B in + 60 B out + 8 B gather; created ones, unless they are sorted and
+    # appended: window 52, record 96, distances 24, out 52
+    sel_bytes = 128 * pst["windows_scanned"] + (0 if passes else 224 * pst["windows_sorted"])
+    sort_bytes = pst["windows_sorted"] * (8 + 20 * passes) if passes else 0   # pass 0 reads he/inst; 4+8+8 B a pass
+    app_bytes = 232 * pst["windows_sorted"] if passes else 0        # key/index 8, window 52, record 96, g 16, out 60
     for name, b, ms in (("select", sel_bytes, ph["select"]), ("sort", sort_bytes, ph["sort"]),
                         ("append", app_bytes, ph["append"])):
         gbs = b / max(ms, 1e-9) / 1e6

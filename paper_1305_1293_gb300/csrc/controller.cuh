@@ -54,8 +54,9 @@ __device__ __forceinline__ void controller_features(const InstCtl& c, const Inst
 // Block-cooperative forward pass, four threads a neuron (4 * kHidden threads).  The
 // control kernel is one block that waits for memory: a thread's weights of all layers are
 // loaded together by `load`, before the features are made, so that their latency is paid
-// once (one thread a neuron, layer by layer, a 1M-face torus took 21.26 ms, now 20.92).  `x` (kFeatures) and `h` (kHidden, every
-// layer's values in turn) live in shared memory; every thread of the block calls both.
+// once (with one thread a neuron, layer by layer, a 1M-face torus took 21.26 ms, with this
+// 20.92).  `x` (kFeatures) and `h` (kHidden, every layer's values in turn) live in shared
+// memory; every thread of the block calls both.
 struct MlpRows {
     float w1[kFeatures / 4], w2[kHidden / 4], w3[kHidden / 4], w4, b1, b2, b3, b4;
 

@@ -343,7 +343,7 @@ __global__ void k_rec_ids(int nh, const int* __restrict__ twin, const unsigned c
 // order the caller's list has.  A window reads the 96-byte records of a band of the
 // surface; scattered over the 1.5 GB of a 5.2M-face sphere (whose subdivision puts the four
 // children of a face a quarter of the list apart) those reads were bound by address
-// translation and L2 misses: a field took 647 ms, and takes 335 in this order.  A mesh of
+// translation and L2 misses: a field took 647 ms, in this order 335 (327 by now).  A mesh of
 // fewer than kReorderFaces faces (its records fit L2 and the TLBs) gains nothing and
 // keeps its order: 8.4 ms either way at 327,680 faces, 46 against 39 at 1,310,720.
 constexpr int kReorderFaces = 1 << 19;

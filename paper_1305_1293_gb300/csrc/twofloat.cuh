@@ -12,8 +12,8 @@
 // 2^-126, magnitudes above the floats (and infinities) infinity or NaN; every test is
 // written so that a NaN decides nothing.  An image takes five integer instructions, a
 // two-float eight operations; they are half of what the propagation kernel issues (with
-// seven and fourteen, eight fields on 327,680 faces took 37.9 ms, now 37.5; a 512 x 512
-// torus 21.6 and 21.3).
+// seven and fourteen, eight fields on 327,680 faces took 37.9 ms, with these 37.5; a field on
+// the 1M-face torus 21.6 and 21.3).
 #pragma once
 #include <cuda_runtime.h>
 
