@@ -353,10 +353,13 @@ constexpr double kChainAhead = 16.0;
 // with 6; 64 sources on a noisy sphere (17 a fan) 2.15 and 1.31 ms.  With few fans short
 // chains only add iterations: 512 x 512 terrain (370 a fan) 7.3 ms with 32 hops, 7.9 with
 // 8.  Lines at 32 and 100 windows a fan; 16 hops between them suit 5,120 faces (46 a fan:
-// 1.13 -> 0.80 ms).  Before the first windows: 8.
+// 1.13 -> 0.80 ms).  Below 32 a fan, 4 hops rather than 5 where an iteration examines more than
+// 2^16 windows: then the useless windows cost time, in smaller iterations the additional
+// iterations do (24 uneven meshes 13.14 -> 12.52 ms; with 4 everywhere a noisy sphere of
+// 18,000 faces 1.51 -> 1.59, of 50,000 2.75 -> 2.86; 3 hops 12.8).  Before the first windows: 8.
 __device__ __forceinline__ int hop_limit(float examined, float fans) {
     if (examined < 64.f) return 8;
-    return examined < 32.f * fans ? 5 : (examined < 100.f * fans ? 16 : INT_MAX);
+    return examined < 32.f * fans ? (examined > 65536.f ? 4 : 5) : (examined < 100.f * fans ? 16 : INT_MAX);
 }
 
 // Loop control, then per instance the selection threshold: the plain control selects the k
