@@ -1025,7 +1025,10 @@ __device__ __forceinline__ void propagate_pairs(const Work& w, Counters* cnt, Fa
     const int lane = threadIdx.x & 31, slot = lane >> 1, even = lane & ~1;
     const bool end_b = (lane & 1) != 0;
     const unsigned before = ((1u << even) - 1u) & kPairLanes;
-    int seen_child = *(volatile int*)&cnt->n_child;
+    // The two lanes of a pair act as one, and all lanes on one arena fill: what other warps may
+    // change meanwhile and a branch depends on (the fill, the superseded source, the split word)
+    // is decided once for all of them, not by each lane's own load.
+    int seen_child = __shfl_sync(full, *(volatile int*)&cnt->n_child, 0);
     unsigned n_prop = 0, n_chain = 0, n_exam = 0, n_occ = 0, n_comp = 0, n_ray = 0;
     // the first `quota` windows of a warp are its by position: no atomic, and as the quota is
     // the list over the resident warps, usually the whole list
@@ -1082,7 +1085,7 @@ __device__ __forceinline__ void propagate_pairs(const Work& w, Counters* cnt, Fa
         double g0 = ldg_dist(Ip->g, R.v0 & ~kPseudoBit);
         double g1 = ldg_dist(Ip->g, R.v1 & ~kPseudoBit);
         double g2 = ldg_dist(Ip->g, R.v2 & ~kPseudoBit);
-        bool stale = mine && stale_source(*Ip, W.src, W.d);
+        bool stale = (__ballot_sync(full, mine && stale_source(*Ip, W.src, W.d)) >> even & 3u) != 0;
         unsigned long long aw = kEmptyAngle;
         if (mine) aw = __ldcg(Ip->ang + W.h);
         bool left = false, right = false, occ = false, prop = mine;
