@@ -120,7 +120,7 @@ struct Inst {
 
 struct InstCtl {
     double tau;                 // selection threshold of the current iteration
-    double ref;                 // histogram reference (a lower bound of every pending key)
+    double ref;                 // histogram reference (the smallest pending key up to its image's rounding)
     unsigned kminf;             // running min of the pending keys' FP32 images (bits; ~0: none)
     float reff;                 // ref as an FP32 image
     int n_pending;              // pending windows of this instance

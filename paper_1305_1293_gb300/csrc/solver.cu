@@ -362,6 +362,15 @@ __device__ __forceinline__ int hop_limit(float examined, float fans) {
     return examined < 32.f * fans ? (examined > 65536.f ? 4 : 5) : (examined < 100.f * fans ? 16 : INT_MAX);
 }
 
+// The selection threshold is never below the nearest pending window.  The histogram, its
+// reference and the running minimum are made of the keys' FP32 images, the compaction compares
+// the FP64 keys: from 2^17 mean edge lengths on one step of the images is wider than the
+// first bin, and a threshold at that bin's edge can lie below every key (no window would be
+// selected in this or any later iteration).  A pool window's key is below the step after its
+// image (images are truncated); a created window's image is rounded a few steps to either
+// side, but one that is not selected has an exact image in the next iteration.
+constexpr unsigned kImageSlack = 4;
+
 // Loop control, then per instance the selection threshold: the plain control selects the k
 // nearest windows (Section 4.2, Step 1) through the key histogram: tau = upper edge of the
 // first bin where the cumulative count reaches k.  Also rolls the histogram reference and
@@ -456,7 +465,10 @@ __global__ void __launch_bounds__(kBins) k_ctrl(Work w, int control, const float
             if ((t == kBins - 1 || (long long)incl >= k) && (t == 0 || (long long)(incl - in_bin) < k)) {
                 double tau = INFINITY;
                 if (np == 0) tau = -INFINITY;
-                else if ((long long)np > k && t < kBins - 1) tau = bin_upper(t, c_in.ref, lbar);
+                else if ((long long)np > k && t < kBins - 1) {
+                    tau = bin_upper(t, c_in.ref, lbar);
+                    tau = bitsd(max(dbits(tau), dbits(of_f_bits(c_in.kminf + kImageSlack, fbias))));
+                }
                 if (w.trace && np > 0) {
                     int row = atomicAdd(w.trace_rows, 1);
                     if (row < w.trace_cap) {
