@@ -104,13 +104,17 @@ __device__ __forceinline__ pch_contour_segment segment(const int* __restrict__ t
 // Writes the segments in face order.  A block adds up the counts of the blocks before it
 // and scans its own faces, so that no array of per-face offsets is written and scanned
 // between the two kernels.  The faces of a tile first list their (face, level) pairs in
-// shared memory; the divisions then run with every lane on a segment.
+// shared memory; the divisions then run with every lane on a segment.  Nothing is written
+// when all blocks together have more than 2^31 - 1 segments: the host refuses such a call,
+// and the 32-bit offsets within a tile hold no more.
 constexpr int kTileSegments = 2048;
 __global__ void __launch_bounds__(256) k_contour_write(const int* __restrict__ tri, int nf, const double* __restrict__ dist,
                                                        const double* __restrict__ levels,
                                                        const long long* __restrict__ image, int n_levels,
                                                        const unsigned long long* __restrict__ block_count,
+                                                       const unsigned long long* __restrict__ total,
                                                        long long capacity, pch_contour_segment* __restrict__ out) {
+    if (*total > (unsigned long long)INT_MAX) return;
     const long long C = ((long long)nf + gridDim.x - 1) / gridDim.x;
     const int f0 = (int)min((long long)nf, C * blockIdx.x), f1 = (int)min((long long)nf, C * (blockIdx.x + 1));
     const int lane = threadIdx.x & 31, warp = threadIdx.x / 32;
@@ -214,7 +218,8 @@ extern "C" pch_status pch_iso_contours(const pch_mesh* m, const double* dist, in
     }
     const double* dd = dist_on_device ? dist : t.dist;
     auto write = [&](long long room, pch_contour_segment* seg) {
-        k_contour_write<<<grid, 256, 0, s>>>(m->dm.tri, nf, dd, t.lev, t.image, n_levels, t.count, room, seg);
+        k_contour_write<<<grid, 256, 0, s>>>(m->dm.tri, nf, dd, t.lev, t.image, n_levels, t.count, t.total, room,
+                                               seg);
         return cudaGetLastError();
     };
     if (!e) {
