@@ -1527,6 +1527,16 @@ __device__ __forceinline__ double2 cmul_conj(double2 a, double2 b) {   // a * co
     return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.y, b.x, -a.x * b.y));
 }
 
+// The vector scaled by a power of two so that its longer component lies in [1, 2): exact (a
+// component 2^-1022 times shorter becomes 0).  Directions come with the lengths of the mesh,
+// which single precision and products of two of them may not hold.
+__device__ __forceinline__ double2 scaled_dir(double x, double y) {
+    const int hx = __double2hiint(x), hy = __double2hiint(y);
+    const int ex = hx & 0x7ff00000, ey = hy & 0x7ff00000, s = max(ex, ey) - 0x3ff00000;
+    return make_double2(ex > max(s, 0) ? __hiloint2double(hx - s, __double2loint(x)) : 0.0,
+                        ey > max(s, 0) ? __hiloint2double(hy - s, __double2loint(y)) : 0.0);
+}
+
 // x clamped to [0, L] on the integer images (a NaN: `nan`).
 __device__ __forceinline__ double clamp_s(double x, double L, double nan) {
     return sbits(x) < 0 ? 0.0 : (lt_s(L, x) ? (sbits(x) > 0x7ff0000000000000ll ? nan : L) : x);
@@ -1635,10 +1645,11 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
         float wlo[2] = {0.f, 0.f}, whi[2] = {0.f, 0.f};
         bool lo_open[2] = {false, false}, hi_open[2] = {false, false};
         if (!all) {
-            float phi = phi_ref + atan2f((float)rq.dy, (float)rq.dx);
+            const double2 in = scaled_dir(rq.dx, rq.dy);
+            float phi = phi_ref + atan2f(f_of(in.y, 896u << 20), f_of(in.x, 896u << 20));
             // the incoming ray in the vertex's angular frame, turned by pi: the direction of
             // phi + pi (and of phi - pi); zb is that of phi + T - pi
-            const double2 E = cmul(rot_ref, make_double2(rq.dx, rq.dy));
+            const double2 E = cmul(rot_ref, in);
             za = make_double2(-E.x, -E.y);
             tr = rot_v;
             zb = cmul(za, tr);
