@@ -286,6 +286,12 @@ __global__ void __launch_bounds__(256) k_reset(Work w, unsigned long long* g, lo
     if (t == 0 && w.trace_rows) *w.trace_rows = 0;
 }
 
+// A face-point source nearer to a corner than this, relative to the longer edge there, is
+// taken as the corner at the point's distance (too long by less than 2^-36 of that edge).  Up
+// to about 2^-38 its windows on the edges that meet there are edge-on within the tolerances:
+// their rays past the corner are lost, and they still win vertices from those that are not.
+constexpr double kCornerReach = 0x1p-37;
+
 // Algorithm 1, initialisation: geod_dist = 0 at the sources; a window on every edge
 // opposite a source (issued as the source's fan request); for a point inside a face,
 // one window on each edge of the face and the three corner distances.
@@ -303,19 +309,33 @@ __global__ void k_init_sources(Work w, const SrcDev* __restrict__ srcs, int n_sr
         // a point inside a face: corner distances and three windows, to the child arena of
         // iteration 0
         const int face = I.finv ? I.finv[s.face] : s.face;
+        bool at_corner = false;
+        double wx[3], wy[3];                                       // the point in the half-edges' frames
         for (int k = 0; k < 3; ++k) {
             int h = 3 * face + k;
             HERec R = I.rec[h];
             // barycentric weights of h's end vertex and apex (its start vertex sits at 0)
             double b1 = s.bary[(k + 1) % 3], b2 = s.bary[(k + 2) % 3];
-            double x = b1 * R.L + b2 * R.xc, y = b2 * R.yc;        // point in h's frame
+            double x = b1 * R.L + b2 * R.xc, y = b2 * R.yc;
+            wx[k] = x;
+            wy[k] = y;
             double dstart = sqrt(x * x + y * y);
             double gc = ldg_dist(I.g, R.v0 & ~kPseudoBit);
             const EvSrc es{s.inst, h, -1 - s.label, 2, x, y};
-            if (const int ev = w.plog ? vertex_event<true>(I, R.v0, dstart, gc, &w, &es) : vertex_event(I, R.v0, dstart, gc)) {
+            const int ev = w.plog ? vertex_event<true>(I, R.v0, dstart, gc, &w, &es) : vertex_event(I, R.v0, dstart, gc);
+            if (dstart <= kCornerReach * fmax(R.L, R.L2)) {
+                // at this corner: its fan covers every direction, as a vertex source's
+                at_corner = true;
+                push_fan(w.req[0], &cnt->n_req_next, w.req_cap, &cnt->error, s.inst, R.v0 & ~kPseudoBit, dstart, -1, 0.0, 0.0);
+            } else if (ev) {
                 // incoming direction: from the corner towards the point, inside face(h)
                 push_fan(w.req[0], &cnt->n_req_next, w.req_cap, &cnt->error, s.inst, R.v0 & ~kPseudoBit, dstart, h, x, y, ev);
             }
+        }
+        for (int k = 0; k < 3 && !at_corner; ++k) {
+            int h = 3 * face + k;
+            HERec R = I.rec[h];
+            const double x = wx[k], y = wy[k];
             if (R.twin < 0) continue;
             // window on twin(h) = (v1 -> v0): point at (L - x, -y), interval [0, L]
             double px = R.L - x, py = -y;
