@@ -482,7 +482,8 @@ def phase_rooflines(pst, passes, hbm):
     out = {"propagate_fp64_tflops": pst["prop_fp64_ops"] / max(ph["propagate"], 1e-9) / 1e9}
     # pool windows: 60 B in + 60 B out + 8 B gather; created ones, unless they are sorted and
     # appended: window 52, record 96, distances 24, out 52
-    sel_bytes = 128 * pst["windows_scanned"] + (0 if passes else 224 * pst["windows_sorted"])
+    created = 0 if passes else pst["windows_sorted"]
+    sel_bytes = 128 * (pst["windows_scanned"] - created) + 224 * created
     sort_bytes = pst["windows_sorted"] * (8 + 20 * passes) if passes else 0   # pass 0 reads he/inst; 4+8+8 B a pass
     app_bytes = 232 * pst["windows_sorted"] if passes else 0        # key/index 8, window 52, record 96, g 16, out 60
     for name, b, ms in (("select", sel_bytes, ph["select"]), ("sort", sort_bytes, ph["sort"]),

@@ -127,7 +127,7 @@ typedef struct {
     int64_t iterations;
     int64_t windows_created;      /* windows written to the pool (children + fans) */
     int64_t windows_propagated;   /* selected windows that passed the filter and were propagated */
-    int64_t peak_pending;         /* largest pending pool seen */
+    int64_t peak_pending;         /* most windows pending at once, after the filters */
     double ms_total;              /* device time of the solve loop (CUDA events) */
     double ms_setup;              /* device time of initialisation */
     int64_t bytes_workspace;      /* device bytes held by the solver workspace */
@@ -139,8 +139,11 @@ typedef struct {
     int64_t fan_candidates;       /* distance events at pseudo-source vertices examined */
     int64_t windows_chained;      /* children propagated in the same iteration (hops > 1) */
     int64_t prop_fp64_ops;        /* algorithmic FP64 operations of the propagation kernel */
-    int64_t windows_scanned;      /* pending windows read by the selection compaction */
-    int64_t windows_sorted;       /* new windows sorted by the organisation step */
+    int64_t windows_scanned;      /* windows read by the selection compaction: the pending pool
+                                     and, unless they were appended to it (PCH_FLAG_EDGE_SORT,
+                                     strided control), the new windows before their filters */
+    int64_t windows_sorted;       /* new windows organised (Step 3) before their filters; they are
+                                     sorted when sort_passes > 0 */
     int64_t sort_passes;          /* 8-bit radix passes per sort */
     int64_t windows_examined;     /* windows the propagation kernel tested (selected + chained) */
     int64_t windows_occupied;     /* of those, windows whose rays reach the opposite vertex */

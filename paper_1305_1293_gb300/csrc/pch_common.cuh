@@ -155,10 +155,10 @@ struct Counters {
     unsigned long long created, propagated, filtered, trimmed, peak_pending;
     unsigned long long fans, fan_windows, fan_cand, chained;
     unsigned long long examined, occupied, children, rays;   // propagation path counts (FP64 op tally)
-    unsigned long long scanned, sorted;               // windows read by compaction / sorted
+    unsigned long long scanned, sorted;               // windows read by compaction / organised
     unsigned long long fan_ties;                      // deferred ties fanned (a new direction)
     int hops;               // limit of this iteration's chains (hop_limit)
-    unsigned long long examined0, fans0;              // examined, fans up to the last iteration
+    unsigned long long examined0, fans0, created0;    // examined, fans, created up to the last iteration
     int work_next;          // next work-list index handed to a propagation lane
     int n_plog;             // unused (kept for the layout); see n_plog_shard
     int n_plog_shard[32];   // provenance records reserved per shard (geodesic paths)

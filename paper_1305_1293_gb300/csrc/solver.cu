@@ -528,12 +528,16 @@ __global__ void __launch_bounds__(kBins) k_ctrl(Work w, int control, const float
             cnt->n_pending = n_pool + n_new;
             if (!halt || done || error) {
                 cnt->iter = it;
-                cnt->scanned = C.scanned + (unsigned long long)n_pool;
+                cnt->scanned = C.scanned + (unsigned long long)(n_pool + n_new);
                 cnt->sorted = C.sorted + (unsigned long long)n_child;
-                if ((unsigned long long)(n_pool + n_new) > C.peak_pending)
-                    cnt->peak_pending = (unsigned long long)(n_pool + n_new);
+                // pending windows, the created ones after their filters: in the pool, or known
+                // now for the last iteration, whose compaction filtered them
+                const unsigned long long pending =
+                    w.append ? (unsigned long long)n_pool : (unsigned long long)C.n_pool + (C.created - C.created0);
+                if (pending > C.peak_pending) cnt->peak_pending = pending;
             }
             if (!halt) {
+                cnt->created0 = C.created;
                 cnt->hops = hop_limit((float)(C.examined - C.examined0), (float)(C.fans - C.fans0));
                 cnt->examined0 = C.examined;
                 cnt->fans0 = C.fans;
