@@ -242,6 +242,7 @@ extern "C" pch_status pch_iso_contours(const pch_mesh* m, const double* dist, in
             e = cudaMemcpyAsync(segments, t.seg, sizeof(pch_contour_segment) * (size_t)keep, cudaMemcpyDeviceToHost, s);
         if (!e) e = cudaStreamSynchronize(s);
     }
+    if (e) cudaStreamSynchronize(s);       // a call that fails leaves nothing in flight
     if (tmp) cudaFreeAsync(tmp, s);
     if (seg_tmp) cudaFreeAsync(seg_tmp, s);
     if (e) return set_error(e == cudaErrorMemoryAllocation ? PCH_ERR_OOM : PCH_ERR_CUDA, "iso-contours: %s",

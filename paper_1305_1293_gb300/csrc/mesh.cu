@@ -657,8 +657,7 @@ extern "C" void pch_destroy(pch_mesh* m) {
     int cur = 0;
     cudaGetDevice(&cur);
     cudaSetDevice(m->device);
-    cudaDeviceSynchronize();          // work of asynchronous calls may still use the memory
-    if (m->ws) destroy_workspace(m->ws);
+    if (m->ws) destroy_workspace(m->ws);   // (waits for the mesh's last call)
     dev_free(m->mem);
     cudaSetDevice(cur);
     delete m;

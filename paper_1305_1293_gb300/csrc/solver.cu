@@ -1967,6 +1967,7 @@ struct Workspace {
     double2* fandir_all = nullptr;
     Counters* cnt_host = nullptr;
     cudaEvent_t ev[2] = {nullptr, nullptr};
+    cudaEvent_t used = nullptr;       // recorded after what a call leaves in flight (device outputs)
     // graph cache: rebuilt when pointers or launch parameters change
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -1977,8 +1978,14 @@ struct Workspace {
     bool trace_on = false;
 };
 
+// Waits until no call's work uses the workspace any more.  Nothing here waits for the whole
+// device: that is not allowed while any thread captures a stream (as build_graph does), and
+// would end that thread's capture with an error.
+static cudaError_t wait_unused(const Workspace* ws) { return cudaEventSynchronize(ws->used); }
+
 void destroy_workspace(Workspace* ws) {
     if (!ws) return;
+    wait_unused(ws);
     if (ws->exec) cudaGraphExecDestroy(ws->exec);
     if (ws->graph) cudaGraphDestroy(ws->graph);
     dev_free(ws->pools);
@@ -1989,6 +1996,7 @@ void destroy_workspace(Workspace* ws) {
     if (ws->cnt_host) cudaFreeHost(ws->cnt_host);
     if (ws->setup_host) cudaFreeHost(ws->setup_host);
     for (auto& e : ws->ev) if (e) cudaEventDestroy(e);
+    if (ws->used) cudaEventDestroy(ws->used);
     delete ws;
 }
 
@@ -2079,7 +2087,7 @@ static pch_status ensure_pools(Workspace* ws, int sel_cap, int pool_cap, int req
         cudaMemcpy(nw.arena.B, w.arena.B, na * 8, cudaMemcpyDeviceToDevice);
         cudaMemcpy(nw.arena.px, w.arena.px, na * 8, cudaMemcpyDeviceToDevice);
         cudaMemcpy(nw.arena.py, w.arena.py, na * 8, cudaMemcpyDeviceToDevice);
-        e = cudaDeviceSynchronize();
+        e = cudaStreamSynchronize(cudaStreamLegacy);   // (the copies run on it)
         if (e) { dev_free(fresh); return set_error(PCH_ERR_CUDA, "pool growth copy: %s", cudaGetErrorString(e)); }
     }
     dev_free(ws->pools);
@@ -2109,6 +2117,11 @@ static pch_status ensure_workspace(pch_mesh* owner, Workspace** out) {
         }
         cudaEventCreate(&ws->ev[0]);
         cudaEventCreate(&ws->ev[1]);
+        if (cudaEventCreateWithFlags(&ws->used, cudaEventDisableTiming) != cudaSuccess) {
+            cudaFreeHost(ws->cnt_host);
+            delete ws;
+            return set_error(PCH_ERR_CUDA, "event creation failed");
+        }
         owner->ws = ws;
     }
     *out = owner->ws;
@@ -2124,7 +2137,7 @@ static size_t setup_bytes(int n_inst, int n_src) {
 static pch_status ensure_instances(Workspace* ws, int n_inst, long long g_total, long long a_total, int n_src) {
     if (n_inst > ws->inst_cap || n_src > ws->src_cap || g_total > ws->g_cap || a_total > ws->ang_cap) {
         drop_graph(ws);
-        PCH_CUDA(cudaDeviceSynchronize());
+        PCH_CUDA(wait_unused(ws));
         dev_free(ws->inst_mem);
         Work& w = ws->w;
         const int ic = std::max(n_inst, ws->inst_cap), sc = std::max(n_src, std::max(ws->src_cap, 64));
@@ -2419,7 +2432,7 @@ static pch_status ensure_plog(Workspace* ws, long long cap) {
     cap = std::min<long long>(cap, 1LL << 30);
     if (cap <= ws->plog_cap) return PCH_OK;
     drop_graph(ws);
-    PCH_CUDA(cudaDeviceSynchronize());
+    PCH_CUDA(wait_unused(ws));
     dev_free(ws->plog_mem);
     ws->plog_cap = 0;
     ws->plog = nullptr;
@@ -2461,6 +2474,12 @@ pch_status solve_instances(pch_mesh* const* meshes, int n_inst, const SrcDev* sr
     Workspace* ws;
     pch_status st = ensure_workspace(meshes[0], &ws);
     if (st != PCH_OK) return st;
+    // a call that fails leaves nothing in flight
+    struct Finish {
+        cudaStream_t s;
+        bool done = false;
+        ~Finish() { if (!done) cudaStreamSynchronize(s); }
+    } finish{s};
     // instance layout
     long long goff = 0, aoff = 0, kbase = 0;
     std::vector<long long> gofs(n_inst), aofs(n_inst);
@@ -2528,7 +2547,7 @@ pch_status solve_instances(pch_mesh* const* meshes, int n_inst, const SrcDev* sr
     w.ahead = rec_bytes < kAheadBytes;
     if (cfg.stride_T > ws->sthr_cap) {
         drop_graph(ws);
-        PCH_CUDA(cudaDeviceSynchronize());
+        PCH_CUDA(wait_unused(ws));
         dev_free(ws->sthr);
         ws->sthr_cap = 0;
         for (int pass = 0; pass < 2; ++pass) {
@@ -2569,7 +2588,8 @@ pch_status solve_instances(pch_mesh* const* meshes, int n_inst, const SrcDev* sr
     for (int attempt = 0;; ++attempt) {
         w.plog = prov ? ws->plog : nullptr;
         w.plog_cap = prov ? ws->plog_cap : 0;
-        // upload tables, clear state
+        // upload tables, clear state (the last call's output, on whatever stream, is read)
+        PCH_CUDA(cudaStreamWaitEvent(s, ws->used));
         PCH_CUDA(cudaMemcpyAsync(ws->setup, ws->setup_host, src_at + sizeof(SrcDev) * n_src, cudaMemcpyHostToDevice, s));
         if (stats) std::memset(stats, 0, sizeof(pch_stats));
         k_reset<<<grid_for(4), 256, 0, s>>>(w, ws->g_all, goff, ws->ang_all, aoff, ws->stamp_all, ws->fanphi_all);
@@ -2607,6 +2627,8 @@ pch_status solve_instances(pch_mesh* const* meshes, int n_inst, const SrcDev* sr
     }
     PCH_CUDA(cudaGetLastError());
     if (out_mode != kOutDevice) PCH_CUDA(cudaStreamSynchronize(s));
+    else PCH_CUDA(cudaEventRecord(ws->used, s));
+    finish.done = true;
     return PCH_OK;
 }
 
@@ -2816,7 +2838,8 @@ static pch_status trace_paths(pch_mesh* m, const SrcDev* sd, int n_src, const pc
     cudaFreeAsync(dtg, s);
     cudaFreeAsync(dn, s);
     cudaFreeAsync(dpts, s);
-    if (!e) e = cudaStreamSynchronize(s);
+    const cudaError_t es = cudaStreamSynchronize(s);
+    if (!e) e = es;
     if (e) return set_error(e == cudaErrorMemoryAllocation ? PCH_ERR_OOM : PCH_ERR_CUDA, "path trace: %s",
                             cudaGetErrorString(e));
     if (stats) stats->kernel_launches += n_targets > 0 ? 2 : 1;
@@ -2907,7 +2930,8 @@ static pch_status voronoi(pch_mesh* m, const SrcDev* sd, int n_src, const pch_op
     cudaFreeAsync(dvsrc, s);
     cudaFreeAsync(dlab, s);
     cudaFreeAsync(dsd, s);
-    if (!e) e = cudaStreamSynchronize(s);
+    const cudaError_t es = cudaStreamSynchronize(s);
+    if (!e) e = es;
     if (e) return set_error(e == cudaErrorMemoryAllocation ? PCH_ERR_OOM : PCH_ERR_CUDA, "voronoi: %s",
                             cudaGetErrorString(e));
     if (stats) stats->kernel_launches += 4;
