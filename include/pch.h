@@ -270,7 +270,9 @@ typedef struct {
 pch_status pch_iso_contours(const pch_mesh* m, const double* dist, int32_t dist_on_device, const double* levels,
                             int32_t n_levels, pch_contour_segment* segments, int64_t capacity, int64_t* n_segments);
 
-/* Release a mesh and its workspace (NULL is a no-op). */
+/* Release a mesh and its workspace (NULL is a no-op).  While other meshes are alive on the
+ * device, up to 512 MB of released memory stay with the library for the next mesh or
+ * temporary; releasing the last one gives all of it back. */
 void pch_destroy(pch_mesh* m);
 
 /* Message of the last error on the calling host thread ("" if none). */
@@ -290,7 +292,9 @@ pch_status pch_mlp_set_weights(const float* params, int32_t n_params);
 pch_status pch_mlp_forward(const float* params_dev, const float* x_dev, int32_t n, float* y_dev,
                            void* stream);
 /* Gradient of 0.5 * mean((y - target)^2) w.r.t. the parameters (device pointers);
- * grad_dev gets num_params floats, loss_dev one float.  Deterministic reduction. */
+ * grad_dev gets num_params floats, loss_dev one float.  Deterministic reduction.  Its
+ * scratch (40 KB an SM at most) is allocated and freed on the stream; the library keeps that
+ * memory for the next call until a mesh, if any, is the last one released. */
 pch_status pch_mlp_backward(const float* params_dev, const float* x_dev, const float* target_dev,
                             int32_t n, float* grad_dev, float* loss_dev, void* stream);
 /* Same result as pch_mlp_backward, without allocating: for callers that cannot call

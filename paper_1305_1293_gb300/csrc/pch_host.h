@@ -21,12 +21,13 @@ struct Workspace;   // solver.cu
 namespace pch {
 
 // ---- device memory -------------------------------------------------------------------
-// The library's own stream-ordered pool, one per device and context (safe for several
-// threads and streams, as the driver's pools are): up to kPoolKeep bytes of freed memory
-// stay with it for the next mesh, workspace or temporary, the rest goes back to the
-// driver at the next synchronisation.  (cudaMalloc / cudaFree of a mesh and its workspace
-// took 4 ms a mesh, and temporaries of the default pool, which keeps nothing, were mapped
-// anew after every synchronising call.)
+// The library's own stream-ordered pools, one per device and context (safe for several
+// threads and streams, as the driver's pools are): while a mesh is alive, up to kPoolKeep bytes
+// of freed memory stay for the next mesh, workspace or temporary and the rest goes back to the
+// driver at the next synchronisation; when the last mesh is destroyed, or an allocation
+// fails, all of it does.  (cudaMalloc / cudaFree of a mesh and its workspace took 4 ms a
+// mesh, and temporaries of the default pool, which keeps nothing, were mapped anew after
+// every synchronising call.)
 constexpr unsigned long long kPoolKeep = 512ull << 20;
 
 // A block of memory that any stream may use once dev_alloc returns.  Blocks above half of
@@ -34,6 +35,8 @@ constexpr unsigned long long kPoolKeep = 512ull << 20;
 struct DevMem {
     void* p = nullptr;
     size_t bytes = 0;
+    unsigned long long ctx = 0;       // context and device it was allocated in
+    int dev = 0;
     bool pooled = false;
 };
 cudaError_t dev_alloc(DevMem& m, size_t bytes);
