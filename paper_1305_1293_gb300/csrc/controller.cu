@@ -3,6 +3,7 @@
 // controller.cuh; none of this has a counterpart in the paper, which fixes k by hand
 // (Section 5.2).
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstddef>
 #include <cstdlib>
@@ -103,6 +104,10 @@ constexpr int kTile = 64;                // samples per tile
 constexpr int kTilePad = kTile + 4;      // row stride of activations [neuron][sample]
 constexpr int kMlpThreads = 256;         // 16 x 16 threads, 4 x 4 outputs each
 constexpr int kGrid = 16;
+// Tiles of n samples (n up to INT_MAX: the sum n + kTile - 1 would not hold).
+__host__ __device__ constexpr int mlp_tile_count(int n) { return n / kTile + (n % kTile ? 1 : 0); }
+static_assert(mlp_tile_count(1) == 1 && mlp_tile_count(kTile) == 1 && mlp_tile_count(kTile + 1) == 2, "tiles");
+static_assert(mlp_tile_count(INT_MAX) == 1 << 25, "no overflow at the largest n");
 static_assert(kHidden == 4 * kGrid && kTile == 4 * kGrid && kFeatures <= 2 * kGrid, "tile layout");
 
 struct MlpTile {
@@ -254,7 +259,7 @@ __global__ void __launch_bounds__(GROUPS * kMlpThreads)
     float g3[4][4] = {}, g2[4][4] = {}, g1[4][2] = {};
     float gv = 0.f, gb4 = 0.f;      // one of W4, b3, b2, b1 (by thread / 64); b4
     double loss = 0.0;
-    const int tiles = (n + kTile - 1) / kTile;
+    const int tiles = mlp_tile_count(n);
     MlpTile& T = group ? S.tile1 : S.tile0;
     auto sync = [&] {                // the group's barrier
         if (GROUPS == 1) __syncthreads();
@@ -392,7 +397,7 @@ __global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ pa
 }
 
 // Blocks of a training pass over n samples: one an SM at most.
-static int mlp_blocks(int n) { return std::max(1, std::min((n + kTile - 1) / kTile, sm_count())); }
+static int mlp_blocks(int n) { return std::min(mlp_tile_count(n), sm_count()); }
 
 // Launches the pass with `scratch` for mlp_blocks(n) partial results of kMlpParams floats, the
 // losses (doubles) first.
@@ -404,7 +409,7 @@ static cudaError_t launch_backward(const float* params, const float* x, const fl
     // Two tiles at once on an SM as soon as some SM has two: 31,722 samples 96.4 -> 86.2 us; with
     // one tile an SM at most the second group is only more threads to start (512 samples: 39.1
     // and 41.1 us).
-    const bool two = (n + kTile - 1) / kTile > blocks;
+    const bool two = mlp_tile_count(n) > blocks;
     const auto kernel = two ? k_mlp_tiles<true, 2> : k_mlp_tiles<true, 1>;
     const size_t smem = two ? sizeof(MlpShared) : offsetof(MlpShared, tile1);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -477,7 +482,7 @@ extern "C" pch_status pch_mlp_forward(const float* params_dev, const float* x_de
     if (!params_dev || !x_dev || !y_dev || n <= 0) return set_error(PCH_ERR_INVALID_ARG, "bad arguments");
     cudaStream_t s = (cudaStream_t)stream;
     PCH_CUDA(cudaFuncSetAttribute(k_mlp_tiles<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMlpForwardBytes));
-    const int blocks = std::min((n + kTile - 1) / kTile, 2 * sm_count());
+    const int blocks = std::min(mlp_tile_count(n), 2 * sm_count());
     k_mlp_tiles<false, 1><<<blocks, kMlpThreads, kMlpForwardBytes, s>>>(params_dev, x_dev, nullptr, n, y_dev, nullptr, nullptr);
     PCH_CUDA(cudaGetLastError());
     return PCH_OK;
@@ -538,7 +543,7 @@ extern "C" pch_status pch_measure_fp64_peak(double* tflops) {
 // until the process exits.
 namespace pch {
 constexpr int kNoAllocMaxSamples = 4096;
-constexpr size_t kNoAllocBlocks = (kNoAllocMaxSamples + kTile - 1) / kTile;
+constexpr size_t kNoAllocBlocks = mlp_tile_count(kNoAllocMaxSamples);
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBlocks * (sizeof(double) + sizeof(float) * kMlpParams)];
 // Host side: the array's device address, resolved once per device and context (a reset
 // device gets a new context, and the array a new address).  The symbol itself is only a
