@@ -1591,8 +1591,9 @@ __global__ void __launch_bounds__(256) k_fan(Work w, int full_fan) {
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&cnt->fan_cand, (unsigned long long)nreq);
     // (the fans' candidates go to the last blocks, the statistics to the first, so that a
     // short list of each runs side by side)
+    // (compared in candidates: nreq * kFanLanes may not fit 32 bits)
     const int fan_block = gridDim.x - 1 - blockIdx.x;
-    if (blockIdx.x * blockDim.x >= n_prop && fan_block * blockDim.x >= nreq * kFanLanes) return;
+    if (blockIdx.x * blockDim.x >= n_prop && fan_block * (blockDim.x / kFanLanes) >= nreq) return;
     // first the selection statistics of the windows that the propagation created (here, where
     // the GPU has little else to do: from inside the propagation kernel they cost 8% of it)
     __shared__ PoolStats ps;
