@@ -280,8 +280,9 @@ const char* pch_last_error(void);
 
 /* ---- learned selection controller (build-only; no counterpart in the paper) -----------
  * A 3 x 64 hidden-layer fp32 MLP maps per-iteration frontier statistics to the number of
- * windows the next selection takes (output log2(k) / 24, k in [2^8, 2^26]).  Weights are a flat fp32 array of pch_mlp_num_params() values
- * (layer by layer: W then b, W row-major [out][in]). */
+ * windows the next selection takes (output log2(k) / 24, clamped to k in [2^12, 2^24]).
+ * Weights are a flat fp32 array of pch_mlp_num_params() values (layer by layer: W then b, W
+ * row-major [out][in]). */
 int32_t pch_mlp_num_features(void);
 int32_t pch_mlp_num_params(void);
 /* Install weights used by PCH_CONTROL_LEARNED on the current device (host array, copied

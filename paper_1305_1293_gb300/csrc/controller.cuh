@@ -5,7 +5,8 @@
 // fixed k by a 3 x 64 hidden-layer fp32 MLP that maps the frontier statistics of one
 // instance to log2 of the number of windows to select, divided by 24.  Any window order
 // gives the same distances (Section 4.3, Remark 2), so the controller can change speed,
-// never results; a non-finite or out-of-range output falls back to the plain k.
+// never results; an output outside 2^12 to 2^24 windows is clamped, and only one that is not
+// finite falls back to the plain k.
 #pragma once
 #include "pch_common.cuh"
 
@@ -29,7 +30,7 @@ constexpr int kMlpParams = kMlpB4 + 1;
 //  f17     log2(faces) / 24
 //  f18     log2(mean edge length) / 8
 //  f19     log2(1 + iteration) / 16
-//  f20     children per selected window in the previous iteration / 4
+//  f20     windows created (before their filters) per selected one in the previous iteration / 4
 //  f21     log2(1 + front distance / mean edge length) / 16
 //  f22     log2(1 + pending / faces) / 8
 //  f23     1

@@ -123,20 +123,15 @@ struct InstCtl {
     double ref;                 // histogram reference (the smallest pending key up to its image's rounding)
     unsigned kminf;             // running min of the pending keys' FP32 images (bits; ~0: none)
     float reff;                 // ref as an FP32 image
-    int n_pending;              // pending windows of this instance
     int n_next;                 // windows pending for the next iteration: left in the pool, or created
-    int n_sel;                  // selected this iteration
-    int n_child;                // children written this iteration
     long long k_target;         // plain control: windows to select
     float last_ratio;           // children / selected of the previous iteration
     float ctl_out;              // last controller output
-    int active;
     float tauf;                 // chaining limit (tau and kChainAhead edge lengths) as an FP32 image
 };
 
 // ---- global counters of one solve -------------------------------------------------
 struct Counters {
-    int n_pending;          // pending windows: in the current pool and in the arena
     int n_pool;             // windows in the current pool
     int n_new;              // arena slots the last iteration's propagation and fans filled
     int n_rest;             // not-selected windows copied to the next pool
@@ -150,9 +145,8 @@ struct Counters {
     int ticket;             // blocks of k_ctrl that are done
     int error;              // bitmask of kErr*
     int done;
-    int sort_bits;          // bits of the sort key
     int halt;               // set by k_ctrl when the loop must stop; every kernel no-ops
-    unsigned long long created, propagated, filtered, trimmed, peak_pending;
+    unsigned long long created, propagated, trimmed, peak_pending;
     unsigned long long fans, fan_windows, fan_cand, chained;
     unsigned long long examined, occupied, children, rays;   // propagation path counts (FP64 op tally)
     unsigned long long scanned, sorted;               // windows read by compaction / organised
@@ -160,7 +154,6 @@ struct Counters {
     int hops;               // limit of this iteration's chains (hop_limit)
     unsigned long long examined0, fans0, created0;    // examined, fans, created up to the last iteration
     int work_next;          // next work-list index handed to a propagation lane
-    int n_plog;             // unused (kept for the layout); see n_plog_shard
     int n_plog_shard[32];   // provenance records reserved per shard (geodesic paths)
 };
 // Distance-event records are split into kPlogShards equal shards, one counter each, chosen

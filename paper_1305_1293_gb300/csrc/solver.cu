@@ -503,7 +503,6 @@ __global__ void __launch_bounds__(kBins) k_ctrl(Work w, int control, const float
                 if (control == PCH_CONTROL_STRIDED) tau = -INFINITY;
                 c.tau = tau;
                 c.tauf = f_of(tau + kChainAhead * lbar, fbias);
-                c.n_pending = np;
                 c.n_next = 0;
                 if (c_in.kminf != ~0u) {           // min key of the pending windows
                     c.ref = of_f_bits(c_in.kminf, fbias);
@@ -525,7 +524,6 @@ __global__ void __launch_bounds__(kBins) k_ctrl(Work w, int control, const float
         if (last) {
             cnt->error = error;
             cnt->done = done ? 1 : 0;
-            cnt->n_pending = n_pool + n_new;
             if (!halt || done || error) {
                 cnt->iter = it;
                 cnt->scanned = C.scanned + (unsigned long long)(n_pool + n_new);
@@ -2529,11 +2527,10 @@ pch_status solve_instances(pch_mesh* const* meshes, int n_inst, const SrcDev* sr
         c.kminf = ~0u;
         c.ref = 0.0;
         c.k_target = cfg.k;
-        c.active = 1;
     }
     // the work list never needs more than the pending windows, which rarely exceed the
     // half-edge count; a larger k only leaves the rest pending.  Under the learned control
-    // the network may pick up to 2^26 windows an iteration: the list is sized for that
+    // the network may pick up to 2^24 windows an iteration: the list is sized for that
     // (within the same caps), not for the plain k it falls back to
     const long long k_size = cfg.control == PCH_CONTROL_LEARNED ? std::max<long long>(cfg.k, 1LL << 22) : cfg.k;
     long long sel_want = std::max<long long>(65536, 4LL * k_size * std::min(n_inst, 64));
