@@ -175,6 +175,12 @@ void dev_free(DevMem& m) {
 }
 
 cudaError_t tmp_alloc(void** p, size_t bytes, cudaStream_t s) {
+    // a captured allocation belongs to the graph, and a pool cannot be made while a stream is
+    // captured (the legacy stream never is)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (s && s != cudaStreamLegacy && cudaStreamIsCapturing(s, &capture) == cudaSuccess &&
+        capture == cudaStreamCaptureStatusActive)
+        return cudaMallocAsync(p, bytes ? bytes : 1, s);
     std::lock_guard<std::mutex> lk(g_pool_mu);
     PoolSlot* ps = nullptr;
     cudaError_t e = current_pool(&ps);
