@@ -57,7 +57,9 @@ typedef enum {
 /* A source: a mesh vertex (kind 0), or a point inside face `face` with barycentric
  * weights `bary` over that face's three corners in their stored order (kind 1).
  * Algorithm 1 takes sources in V; the face point is the same initialisation applied
- * to the three edges of the face. */
+ * to the three edges of the face.  A point within 2^-37 of the longer edge at a corner is
+ * taken as that corner, at the point's distance from it (paths then end at the corner when
+ * the point lies on it exactly). */
 typedef struct {
     int32_t kind;
     int32_t vertex;
