@@ -74,8 +74,9 @@ struct PoolSlot {
     int blocks = 0;                   // dev_alloc blocks that live in it
 };
 constexpr int kMaxPoolDevices = 64;
-// the pools of each device, one a context (those of a destroyed context are gone with it)
-static std::vector<PoolSlot> g_pools[kMaxPoolDevices];
+// the pools of each device, one a context (those of a destroyed context are gone with it);
+// never destroyed, as a mesh may be released while the process exits
+static std::vector<PoolSlot>* const g_pools = new std::vector<PoolSlot>[kMaxPoolDevices];
 static std::mutex g_pool_mu;
 
 // The current device's pool in its current context.  Call with g_pool_mu held; the slot is
